@@ -48,7 +48,8 @@ enum {
 /* Flags of mb_opts.flags */
 #define MB_BS3      0x1u   /* index: bisulfite 3-base index over CT(R).GA(R) (Section 2.9);
                               seeding: convert read 1 C->T and read 2 G->A, keep hits by strand */
-#define MB_BATCHED  0x2u   /* seeding: lanes take reads from a device work queue, in read order */
+#define MB_BATCHED  0x2u   /* seeding: reads come from a device work queue, in read order (the default
+                              SMEM kernel always takes them so; the one-loop form only with this flag) */
 #define MB_CHECKED  0x4u   /* seeding / locate: the kernels also check every occurrence row they
                               read against the text length (only a damaged index can fail it; the
                               checked locate runs one walk per lane); a failed check ends that read
@@ -72,9 +73,10 @@ enum {
                               extending unique matches (a row that is a multiple of 4) instead of
                               the rate-r samples of Section 2.4: about r/4 times fewer LF steps, same
                               positions; no joins.  Ignored for an index built with MB_NO_AUX */
-#define MB_SMEM_ONE_LOOP 0x80u /* tuning: the SMEM kernel in its one-loop form (every iteration runs
-                              every stage's code) instead of the split form (uniform block steps,
-                              the other actions in service passes); same output */
+#define MB_SMEM_ONE_LOOP 0x80u /* tuning: the SMEM kernel in its one-loop form (one read per lane, every
+                              iteration runs every stage's code) instead of the slot form (a warp
+                              holds up to 64 reads and runs one kind of step for up to 32 of them at
+                              a time); same output */
 
 /* Flags of mb_smem.flags */
 #define MB_SMEM_OVER_MAX_OCC 0x1u   /* s > max_occ: reported, not located, no hits */
@@ -96,17 +98,11 @@ typedef struct {
     uint32_t chunk_reads;     /* mb_seed_locate: reads per pipelined chunk (0 = 2^22) */
     uint32_t prefetch_depth;  /* tuning: LF-walks in flight per lane in locate, 1/2/4/8/16 (0 = 1) */
     uint32_t block_size;      /* tuning: threads per block (0 = default) */
-    uint32_t smem_burst;      /* tuning: SMEM kernel (split form), memory steps (extensions, walk
-                                 steps, text comparisons, samples, k-mer entries) a warp runs between
-                                 two service passes of its stage changes (0 = default, 8) */
-    uint32_t smem_wait;       /* tuning: SMEM kernel (split form), lanes out of the memory steps that
-                                 call a service pass early, 1..32 (0 = default, 8) */
-    uint32_t smem_warps;      /* tuning: SMEM kernel (split form), resident warps per SM its register
-                                 budget aims at: 40 (256 threads per block) or 48 (256 or 512); 0 =
-                                 24 at 128 threads per block, else 32 */
-    uint32_t smem_reads_per_warp; /* tuning: SMEM kernel (split form), reads a warp holds at once,
-                                 one per lane, 1..32 (0 = 32); with fewer the other lanes stay idle
-                                 (a read's steps depend on each other, so lanes cannot share one) */
+    uint32_t smem_burst;      /* accepted, without effect: the slot form picks its steps itself */
+    uint32_t smem_wait;       /* accepted, without effect */
+    uint32_t smem_warps;      /* accepted, without effect */
+    uint32_t smem_reads_per_warp; /* tuning: SMEM kernel (slot form), reads a warp holds at once, 1..31
+                                 (0 or more = up to 64) */
 } mb_opts;
 
 /* One SMEM (48 bytes).  (k, kr, s) is its ds-interval (lo(P), lo(revcomp P), occ(P)),
@@ -276,9 +272,8 @@ int mb_seed_locate(const mb_index *idx, const uint8_t *seq, const uint64_t *off,
  * the whole stage on `stream` (SMEMs by Algorithm 3, the max-occ flag, hit offsets, locate by
  * Algorithm 2) with no host synchronization and no allocation, so the call can be captured into
  * a CUDA graph and the graph replayed for new batches written into the same input buffers.
- * With MB_BATCHED in opts->flags the SMEM kernel takes reads from a device work queue in read
- * order (one persistent launch for reads of very different lengths: a lane takes the next read
- * when its read ends);
+ * The SMEM kernel takes reads from a device work queue in read order (one persistent launch for
+ * reads of very different lengths: the next read is taken when one ends);
  * opts->block_size (128, 256 or 512) selects the launch shape.
  *   seq, off, mate (or NULL): DEVICE pointers, as in mb_seed_batch.
  * mb_plan_result waits for the stream and returns the plan-owned DEVICE arrays of the last
@@ -287,9 +282,9 @@ int mb_seed_locate(const mb_index *idx, const uint8_t *seq, const uint64_t *off,
  * exceeded; nothing beyond the limits was written.
  * mb_autotune times mb_plan_run on the given batch over the launch shapes in two stages and
  * writes the fastest into *best (same output for all): first the SMEM kernel's shape, threads per
- * block 128/256/512 x work queue off/on x kernel form (the one-loop form MB_SMEM_ONE_LOOP, or the
- * split form with smem_burst 2/4/8/16 x smem_wait 4/8/16), with 16 plain locate walks per lane;
- * then, when the best is a split form, smem_reads_per_warp 1/2/4/8/16 (against its 32); then, with
+ * block 128/256/512 x MB_BATCHED off/on x kernel form (the one-loop form MB_SMEM_ONE_LOOP, or the
+ * slot form at smem_burst 2/4/8/16 x smem_wait 4/8/16, which no longer differ), with 16 plain locate
+ * walks per lane; then, when the best is a slot form, smem_reads_per_warp 1/2/4/8/16; then, with
  * the best SMEM shape, locate walks per lane 1/2/4/8 plain and 1/2/4/8/16 with walks that join
  * (MB_LOCATE_JOIN) (92 points, 87 when the one-loop form wins).  mb_autotune_points does
  * the same and also returns every point tried with its time in ms (up to cap points; *n_points

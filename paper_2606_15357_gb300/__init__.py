@@ -510,11 +510,11 @@ def shape_of(o: Opts) -> dict:
     """The launch-shape fields of an Opts as a plain dict (for reports)."""
     split = not (o.flags & MB_SMEM_ONE_LOOP)
     return {"block_size": o.block_size or 256, "work_queue": bool(o.flags & MB_BATCHED),
-            "smem_form": "split" if split else "one_loop",
+            "smem_form": "slots" if split else "one_loop",
             "smem_burst": (o.smem_burst or 8) if split else None,
             "smem_wait": (o.smem_wait or 8) if split else None,
             "smem_warps": (o.smem_warps or None) if split else None,
-            "smem_reads_per_warp": (o.smem_reads_per_warp or 32) if split else None,
+            "smem_reads_per_warp": (o.smem_reads_per_warp or 64) if split else None,
             "locate_walks_per_lane": o.prefetch_depth or 1, "locate_join": bool(o.flags & MB_LOCATE_JOIN),
             "locate_aux": bool(o.flags & MB_LOCATE_AUX)}
 

@@ -155,8 +155,11 @@ __device__ __forceinline__ Blk load_blk(const OccBlock *__restrict__ blk) {
     return b;
 }
 
-// Rows of the block before row m (0..63) as a bit mask.
-__device__ __forceinline__ u64 rows_before(u32 m) { return (1ULL << m) - 1; }
+// Rows of the block before row m (0..63) as a bit mask, low and high half: two clamped funnel shifts
+// (a 64-bit shift and subtract cost about three times the instructions).
+__device__ __forceinline__ u32 rows_before_lo(u32 m) { return __funnelshift_lc(0xffffffffu, 0u, m); }
+__device__ __forceinline__ u32 rows_before_hi(u32 m) { return __funnelshift_lc(0xffffffffu, 0u, (u32)__viaddmax_s32((int)m, -32, 0)); }
+__device__ __forceinline__ u64 rows_before(u32 m) { return ((u64)rows_before_hi(m) << 32) | rows_before_lo(m); }
 // Code of row m of the block.
 __device__ __forceinline__ u32 sym_at(const Blk &b, u32 m) {
     return (u32)((b.lo >> m) & 1) | ((u32)((b.hi >> m) & 1) << 1);
@@ -166,14 +169,8 @@ __device__ __forceinline__ u64 rows_eq(const Blk &b, u32 a) {
     const u64 fl = (u64)(a & 1) - 1, fh = (u64)(a >> 1) - 1;   // all ones where that bit of a is 0
     return (b.lo ^ fl) & (b.hi ^ fh);
 }
-// Rows holding a code <= a (0..3).
-__device__ __forceinline__ u64 rows_le(const Blk &b, u32 a) {
-    return a < 2 ? (a == 0 ? ~(b.lo | b.hi) : ~b.hi) : (a == 2 ? ~(b.lo & b.hi) : ~0ULL);
-}
 // #{rows before m holding code a}; the $ row (stored as A) is not corrected here.
 __device__ __forceinline__ u32 cnt_sym(const Blk &b, u32 m, u32 a) { return __popcll(rows_eq(b, a) & rows_before(m)); }
-// #{rows before m holding a code <= a}; the $ row (stored as A) is not corrected here.
-__device__ __forceinline__ u32 cnt_le(const Blk &b, u32 m, u32 a) { return __popcll(rows_le(b, a) & rows_before(m)); }
 
 // x[a] for a in 0..3 without dynamic indexing (which would go through local memory)
 __device__ __forceinline__ u32 sel4(u32 a, u32 x0, u32 x1, u32 x2, u32 x3) {
@@ -181,10 +178,7 @@ __device__ __forceinline__ u32 sel4(u32 a, u32 x0, u32 x1, u32 x2, u32 x3) {
 }
 
 // [the $ row lies in the block of x, before x]
-__device__ __forceinline__ u32 dollar_before(u32 x, u32 primary) {
-    const u32 bstart = x & ~BLK_MASK;
-    return (primary >= bstart && primary < x) ? 1u : 0u;
-}
+__device__ __forceinline__ u32 dollar_before(u32 x, u32 primary) { return x - 1 - primary < (x & BLK_MASK) ? 1u : 0u; }
 
 // One LF step of Algorithm 2 from row x (x is not the $ row): a = B[x], result C[a] + #a in
 // B[0, x).
@@ -206,12 +200,24 @@ __device__ __forceinline__ u32 lf_blk(const Blk &b, u32 x, u32 primary, u32 C0, 
 struct Ext {
     u32 p, q, s;
 };
-// #a and #{symbols <= a} in B[0, x), $ excluded
-__device__ __forceinline__ void occ_a_le(const Blk &b, u32 x, u32 a, u32 primary, u32 &na, u32 &nle) {
-    const u32 m = x & BLK_MASK, d = dollar_before(x, primary);
-    na = sel4(a, b.c[0], b.c[1], b.c[2], b.c[3]) + cnt_sym(b, m, a) - (a == 0 ? d : 0u);
-    const u32 c01 = b.c[0] + b.c[1], c012 = c01 + b.c[2];
-    nle = sel4(a, b.c[0], c01, c012, c012 + b.c[3]) + cnt_le(b, m, a) - d;
+// The symbol a of an extension as masks: its low and high code bit inverted, and whether it is 2.
+struct SymMask {
+    u32 fl, fh, g;
+};
+__device__ __forceinline__ SymMask sym_mask(u32 a) { return {(a & 1u) - 1u, (a >> 1) - 1u, a == 2 ? ~0u : 0u}; }
+// #a and #{symbols <= a} in B[0, x), $ excluded.  Within the block, the rows holding a smaller code
+// are, for a = 1 and 2, those with the high bit clear and (a = 1) the low bit clear; for a = 3 all
+// others.  The $ row is stored as A, so it counts once as a (a = 0) or as smaller (a > 0).
+__device__ __forceinline__ void occ_a_le(const Blk &b, u32 x, u32 a, const SymMask &k, u32 primary, u32 &na, u32 &nle) {
+    const u32 m = x & BLK_MASK, d = x - 1 - primary < m ? 1u : 0u;   // [the $ row lies in the block, before x]
+    const u32 m0 = rows_before_lo(m), m1 = rows_before_hi(m);
+    const u32 l0 = (u32)b.lo, l1 = (u32)(b.lo >> 32), h0 = (u32)b.hi, h1 = (u32)(b.hi >> 32);
+    const u32 eq = __popc((l0 ^ k.fl) & (h0 ^ k.fh) & m0) + __popc((l1 ^ k.fl) & (h1 ^ k.fh) & m1);
+    u32 lt = __popc(~h0 & (~l0 | k.g) & m0) + __popc(~h1 & (~l1 | k.g) & m1);
+    lt = a == 0 ? 0u : (a == 3 ? m - eq : lt);
+    const u32 c01 = b.c[0] + b.c[1], raw = sel4(a, b.c[0], b.c[1], b.c[2], b.c[3]) + eq;
+    na = raw - (a == 0 ? d : 0u);
+    nle = sel4(a, 0u, b.c[0], c01, c01 + b.c[2]) + lt + raw - d;
 }
 
 // One extension from the already loaded blocks b0 (of row p) and b1 (of row p+s).
@@ -219,8 +225,9 @@ __device__ __forceinline__ Ext extend_blocks(const DevIndex &I, const Blk &b0, c
                                              u32 a) {
     const u32 e = p + s, prim = (u32)I.primary;
     u32 na0, nle0, na1, nle1;
-    occ_a_le(b0, p, a, prim, na0, nle0);
-    occ_a_le(b1, e, a, prim, na1, nle1);
+    const SymMask k = sym_mask(a);
+    occ_a_le(b0, p, a, k, prim, na0, nle0);
+    occ_a_le(b1, e, a, k, prim, na1, nle1);
     Ext r;
     r.s = na1 - na0;
     r.p = sel4(a, (u32)I.C[0], (u32)I.C[1], (u32)I.C[2], (u32)I.C[3]) + na0;

@@ -1,17 +1,15 @@
 // Seeding on the GPU: (l,c)-SMEM finding (Section 2.5, Algorithm 3), the max-occurrence flag,
 // and locate through the sampled suffix array (Section 2.4, Algorithm 2).
 //
-// SMEMs: one thread runs Algorithm 3's three-stage state machine for one read.  In Algorithm 3
-// every read has exactly one entry in the queue at any time, so the per-read order of queue
-// operations is the serial order below; the GPU's many resident warps take the place of the
-// paper's queue-plus-prefetch as the way to keep many block reads in flight.  Every step that
-// touches memory is one extension (Algorithm 1), i.e. two occurrence-block reads, so all lanes
-// of a warp share the same memory instruction whatever stage they are in.
+// SMEMs: Algorithm 3's three-stage state machine per read.  In Algorithm 3 every read has exactly one
+// entry in the queue at any time, so the per-read order of queue operations is the serial order
+// below; the reads a warp holds (k_smem_slots) take the place of the paper's queue-plus-prefetch as
+// the way to keep many block reads in flight.
 //
 // Output: each read first writes its SMEMs into a private run of slots in scratch memory
-// (off[r]/16 + 8r slots before it), a prefix sum over the per-read counts gives the final
-// positions, and a gather writes the 48-byte records.  Reads with more SMEMs than slots are
-// listed and recomputed straight into the final records.
+// (off[r]/16 + 8r slots before it), further ones into a pool all reads share; a prefix sum over the
+// per-read counts gives the final positions, and a gather writes the 48-byte records.  A read with a
+// record that found no room at all is listed and recomputed straight into the final records.
 #include <climits>
 #include <vector>
 #include "common.cuh"
@@ -218,7 +216,7 @@ enum { ACT_NONE = 0, ACT_EXT = 1, ACT_KMER = 2, ACT_WALK = 3, ACT_SAMPLE = 4, AC
 // steps they replace.
 constexpr int U_MIN = 16;
 
-// The memory actions of the uniform step of k_smem_split: block reads (an extension or an LF step
+// The memory actions of stages 4-7 in k_smem_slots: block reads (an extension or an LF step
 // of a walk), a text comparison, an SA / ISA sample, a k-mer table entry.
 enum { R_BLOCK = 0, R_TEXT = 1, R_SAMPLE = 2, R_KMER = 3 };
 
@@ -277,14 +275,6 @@ __device__ __forceinline__ bool uniq_next(SmemState &S, u32 n, u32 prim, int &ra
         return false;
     }
 }
-
-// Tuning of k_smem_split: memory steps between two service passes, and lanes out of the loop that
-// call a service pass early (defaults; mb_opts.smem_burst / smem_wait override them).
-struct SmemTuning {
-    u32 burst, wait;
-    u32 rpw;   // reads a warp holds at once (lanes 0 .. rpw-1), 1..32
-};
-constexpr u32 SMEM_BURST = 8, SMEM_WAIT = 8;
 
 // Moves through the steps of Algorithm 3 that need no memory and picks the next memory action:
 // ACT_EXT, an extension of P[j] (backward in stages 1 and 3, forward in stage 2); ACT_KMER, a
@@ -484,11 +474,37 @@ struct WarpRange {
     }
 };
 
-// One lane keeps one read in flight; each loop iteration performs at most one extension per lane.
-// QUEUE = false: reads are dealt out in warp ranges (WarpRange).  QUEUE = true: warps take the
-// next reads from a device work queue (perm[*qhead ...], an atomic head), so long and short reads
-// balance across the whole GPU in one launch.  A read whose slots would pass slot_total writes
-// none (it is recomputed by the overflow pass).
+// Reads whose steps run on and on (inside tandem repeats a read of 10 kb takes 35,000 dependent steps,
+// the length of a whole launch) are cut: after `steps` steps the starts not recorded yet become
+// items of `starts` starts each, and a second launch runs the items like reads.  An item that owns
+// the starts [c0, c1) scans from c0 - 1.  From any start, Algorithm 3 finds the longest match there
+// and then, in order, every SMEM that starts later: what its stage 3 moves on to cannot be extended
+// to the left, whatever came before.  So only a match found at c0 - 1 itself may be no SMEM, and the
+// item leaves it out; it ends at the first start of c1 or later.  Together the items give the SMEMs
+// of the read, each once, in order.
+struct Item {
+    u32 read;
+    int c0, c1;
+    u32 cnt;      // its records (bit 31: one found no room), then the records of the read before it
+};
+struct HeavyRead {
+    u32 read, first, n, cnt;   // its items and the records found before the cut (bit 31: one found no room)
+};
+constexpr u32 NO_ROOM = 1u << 31;
+// A record that found no slot: its number within the read (or, bit 31 of `who` set, within an item).
+struct PoolRec {
+    u32 who, idx;
+    SlotRec rec;
+};
+struct SplitBufs {
+    u32 *n = nullptr;   // counters: items, cut reads, pool records, the items' queue head
+    Item *items = nullptr;
+    HeavyRead *heavy = nullptr;
+    PoolRec *pool = nullptr;
+    u32 items_cap = 0, pool_cap = 0;   // zero: no read is cut, no record goes to the pool
+    u32 steps = ~0u, starts = 64;
+};
+
 struct SmemArgs {
     DevIndex I;
     const u8 *seq;
@@ -501,20 +517,23 @@ struct SmemArgs {
     u64 slot_total;
     u64 *counts;
     u32 *ovf_list, *ovf_n;
-    const u32 *perm;
-    u32 *qhead;
+    u32 *qhead;      // the head of the queue that warps take reads from (zero at the launch)
     u64 *wc;
     const u32 *lc;   // per-read (l | c << 16), or null for the kernel-wide l and c
     bool uext;       // extend matches that occur once by comparing text (stages 4-7)
     u32 *err = nullptr;                // device error word (always given)
     u32 *chk = nullptr;                // with MB_CHECKED: the error word, for the per-step bounds checks
-    bool split = true;                 // k_smem_split (else k_smem, one loop for every stage)
-    u32 warps = 0;                     // k_smem_split: resident warps per SM aimed at (0: by block size)
-    SmemTuning tune = {SMEM_BURST, SMEM_WAIT, 32};
+    bool one_loop = false;             // MB_SMEM_ONE_LOOP: k_smem (else k_smem_slots)
+    u32 per_warp = 0;                  // k_smem_slots: reads a warp holds (0: SLOTS)
+    SplitBufs sp = {};                 // k_smem_slots: cut reads and the records that find no slot
 };
 
-// Launch bounds per shape: 128 threads allow 85 registers (6 blocks, 24 warps per SM); 256 and
-// 512 threads cap registers at 64 (32 warps per SM).
+// The one-loop form (MB_SMEM_ONE_LOOP; MB_COUNT): one lane keeps one read in flight, and each loop
+// iteration performs at most one extension per lane.  QUEUE = false: reads are dealt out in warp
+// ranges (WarpRange).  QUEUE = true: warps take the next reads from a device work queue (an atomic
+// head).  A read whose slots would pass slot_total writes none (it is recomputed by the overflow
+// pass).  Launch bounds per shape: 128 threads allow 85 registers (6 blocks, 24 warps per SM); 256
+// and 512 threads cap registers at 64 (32 warps per SM).
 template <bool COUNT, bool QUEUE, int BLOCK>
 __global__ void __launch_bounds__(BLOCK, BLOCK == 128 ? 6 : 1024 / BLOCK) k_smem(DevIndex I, const u8 *__restrict__ seq,
                                                                const u64 *__restrict__ off, u32 nr,
@@ -522,8 +541,7 @@ __global__ void __launch_bounds__(BLOCK, BLOCK == 128 ? 6 : 1024 / BLOCK) k_smem
                                                                bool kmer,
                                                                SlotRec *__restrict__ slots, u64 slot_total,
                                                                u64 *__restrict__ counts, u32 *__restrict__ ovf_list,
-                                                               u32 *__restrict__ ovf_n, const u32 *__restrict__ perm,
-                                                               u32 *qhead, u64 *wc, const u32 *__restrict__ lc,
+                                                               u32 *__restrict__ ovf_n, u32 *qhead, u64 *wc, const u32 *__restrict__ lc,
                                                                bool uext, u32 *err) {
     const u32 lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
     const u32 n = (u32)I.n;
@@ -573,7 +591,7 @@ __global__ void __launch_bounds__(BLOCK, BLOCK == 128 ? 6 : 1024 / BLOCK) k_smem
     bool live;
     take(32, lane, item, live);
     if (live) {
-        r = QUEUE && perm ? perm[item] : item;
+        r = item;
         start(r);
     }
     for (;;) {
@@ -661,7 +679,7 @@ __global__ void __launch_bounds__(BLOCK, BLOCK == 128 ? 6 : 1024 / BLOCK) k_smem
             if (fin) {
                 live = ok2;
                 if (live) {
-                    r = QUEUE && perm ? perm[it2] : it2;
+                    r = it2;
                     start(r);
                 }
             }
@@ -670,239 +688,500 @@ __global__ void __launch_bounds__(BLOCK, BLOCK == 128 ? 6 : 1024 / BLOCK) k_smem
     work.flush(wc);
 }
 
-// Text comparison of stage 5 with the text words t0, t1 at T[x & ~15, ...), x = pos + j - i: the
-// matching prefix of up to 16 read bases; a mismatch or an N ends the match (stage 6).
-__device__ __forceinline__ void text_apply(SmemState &S, u32 t0, u32 t1, u32 n) {
-    const u32 x = S.pos + (u32)(S.j - S.i);
-    u32 rc = 0, rn = 0;
-    const u32 rcnt = read_codes16(S, S.j, rc, rn);
-    const u32 tc = (u32)((((u64)t1 << 32) | t0) >> (2 * (x & 15)));
-    const u32 lim = min(min(rcnt, (u32)(S.L - S.j)), n - 1 - x);
-    const u32 d = rc ^ tc, m2 = ((d | (d >> 1)) & 0x55555555u) | rn;
-    const u32 first = m2 ? (u32)(__ffs(m2) - 1) >> 1 : 16u;
-    S.j += (int)min(first, lim);
-    if (first < lim) S.u = 6;
+// ---------------------------------------------------------------------------- reads in slots
+// The SMEM kernel in its slot form.  A warp keeps up to SLOTS reads, their Algorithm 3 state in
+// shared memory, and each iteration it runs ONE kind of step for up to 32 of the reads that are
+// waiting for that kind:
+//   C_BLOCK  an extension by P[j] (stages 1-3; Algorithm 1) or an LF step of a walk (4 and 7)
+//   C_TEXT   a text comparison of up to 64 bases (stage 5)
+//   C_LOOK   a k-mer table entry (stages 1 and 3, Section 2.5), an SA or ISA sample (4 and 6)
+//   C_SERV   what reads no index array: records, restarts after an emitted match, the end of a
+//            read and the next one, the read's bases into the slot
+// The kind with the most waiting reads is taken, so the lanes of an instruction are mostly active
+// whatever stages the reads are in.  The steps of one read and their order are Algorithm 3's, so the
+// records are the same.
+//
+// What bounds it: latency of the random block reads, then their rate.  The form this replaced (one
+// read per lane, all kinds of step in one loop) had 9.6 active lanes per instruction and cost a read
+// 2,160 warp instructions; this one has 19-26 lanes in its block steps and about 900.  20M reads of
+// 150 bases on a 1 Gbp index (k = 14): 59.2 -> 45 ms, 36 -> 47 G random sectors/s, the rate the
+// random-read probe reaches; 2M reads on a 100 Mbp index 5.17 -> 2.9 ms.  More reads in flight help
+// (32 slots per warp instead of 64: 20% slower; 24 warps per SM instead of 32: 6%), so the table takes
+// the shared memory it can get: 64 slots x 32 warps x 89 bytes.  A lone read (a small batch's tail)
+// advances one extension per 0.7 us.
+constexpr int SLOTS = 64;           // reads a warp holds (two per lane: at most 2-way bank conflicts)
+constexpr int WIN = 64;             // bases of a read kept in its slot, 2 bits each
+enum { C_BLOCK = 0, C_TEXT = 1, C_LOOK = 2, C_SERV = 3, C_FREE = 4 };
+// meta word of a slot: stage in bits 0..2, flags, conversion in bits 8..9, extension steps from bit 10
+constexpr u32 M_TRIED = 8, M_PEND = 16, M_NEW = 32, M_HASN = 64, M_DROP = 128, M_CONV = 8, M_STEP = 10;
+
+struct WarpSlots {
+    u32 rd[SLOTS], k[SLOTS], kr[SLOTS], s[SLOTS], pos[SLOTS], cnt[SLOTS], lc[SLOTS], meta[SLOTS];
+    int L[SLOTS], i[SLOTS], j[SLOTS], wb[SLOTS];   // wb: read index of the window's first base
+    int c0[SLOTS], c1[SLOTS];                      // items: the starts they own
+    u32 code[WIN / 16][SLOTS];                     // the window's bases, 16 per word
+    u32 nmask[WIN / 32][SLOTS];                    // bit per base: an N
+    u64 at[SLOTS];                                 // the read's first base: offset into seq
+    u8 cls[SLOTS];
+    u8 list[32];                                   // the slots of the current step
+};
+
+// Sixteen bases (bytes) to 2-bit codes, first base in the low bits.  Per word of four bytes one
+// multiply moves byte b to bits 24 + 2b; the eight other products stay below bit 24 or pass bit 31.
+__device__ __forceinline__ u32 pack16(uint4 v) {
+    const u32 m = 0x03030303u, f = (1u << 24) | (1u << 18) | (1u << 12) | (1u << 6);
+    const u32 a = ((v.x & m) * f) >> 24, b = ((v.y & m) * f) >> 24, c = ((v.z & m) * f) >> 24, d = ((v.w & m) * f) >> 24;
+    return a | (b << 8) | (c << 16) | (d << 24);
+}
+// Bisulfite conversion of sixteen 2-bit codes (conv 1: C -> T; conv 2: G -> A).
+__device__ __forceinline__ u32 convert_codes(u32 x, u32 conv) {
+    const u32 ONES = 0x55555555u;
+    if (conv == 1) return x | ((x & ~(x >> 1) & ONES) << 1);
+    if (conv == 2) return x & ~(((x >> 1) & ~x & ONES) << 1);
+    return x;
+}
+// Bit t set when byte t of the sixteen is above 3.
+__device__ __forceinline__ u32 n_bits(uint4 v) {
+    const u32 w[4] = {v.x, v.y, v.z, v.w};
+    u32 r = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) r |= (((w[q] >> (8 * b)) & 0xFCu) ? 1u : 0u) << (4 * q + b);
+    return r;
 }
 
-// The SMEM kernel with the memory actions split from the rest.  Its lanes go through Algorithm 3
-// exactly as k_smem's do (same reads, same steps in the same order, same records), but a warp
-// runs two kinds of iteration:
-//  - a memory step, uniform for every lane that holds a memory action: an extension by P[j]
-//    (stages 1-3; Algorithm 1) or an LF step of a walk (stages 4 and 7), both reading
-//    occurrence blocks; a text comparison (stage 5); an SA or ISA sample (stages 4 and 6); a
-//    k-mer table entry (Section 2.5).  The loads of all lanes are issued before any result is
-//    used, so they are in flight together.  A lane whose next action follows without a record or
-//    a restart (another extension of the same stage, stage 1's match going on to stage 2, the
-//    next walk step, the next text comparison, the sample at the end of a walk, ...) stays in
-//    this loop;
-//  - a service pass, run when at least `wait` lanes are out of the loop, when `burst` memory
-//    steps ran since the last pass, or when no lane holds a memory action: every lane out of the
-//    loop applies a failed extension (a record, a restart) and moves through the stage changes
-//    up to its next memory action; finished lanes take new reads.  A pass reads no index array.
-// So the branches of the stages are executed together once per service pass instead of in every
-// iteration.
-// WARPS: resident warps per SM the launch bounds aim at (their register cap: 65,536 / (WARPS x 32)).
-template <bool QUEUE, int BLOCK, int WARPS>
-__global__ void __launch_bounds__(BLOCK, WARPS * 32 / BLOCK)
-    k_smem_split(DevIndex I, const u8 *__restrict__ seq, const u64 *__restrict__ off, u32 nr,
-                 const u8 *__restrict__ mate, u32 bs, u32 l, u32 c, bool kmer, SlotRec *__restrict__ slots,
+// Bases [cst, cst + 16) of the read at P (P + cst is 16-byte aligned), byte by byte where the chunk would
+// pass the end of the batch, `room` bytes after P (bases outside [0, L) are then zero).
+__device__ __forceinline__ uint4 load_chunk(const u8 *__restrict__ P, int cst, int L, u64 room) {
+    if ((long long)cst + 16 <= (long long)room) return __ldg(reinterpret_cast<const uint4 *>(P + cst));
+    u64 lo = 0, hi = 0;
+#pragma unroll 1
+    for (int t = 15; t >= 0; --t) {
+        hi = (hi << 8) | (lo >> 56);
+        lo = (lo << 8) | (cst + t >= 0 && cst + t < L ? P[cst + t] : 0u);
+    }
+    return make_uint4((u32)lo, (u32)(lo >> 32), (u32)hi, (u32)(hi >> 32));
+}
+
+// Warps take reads, in read order, from a device queue (*qhead); with ITEMS they take the items of the
+// cut reads, sp.n[0] of them.  Any block size up to 512.
+template <bool ITEMS>
+__global__ void __launch_bounds__(512, 2)
+    k_smem_slots(DevIndex I, const u8 *__restrict__ seq, const u64 *__restrict__ off, u32 nr,
+                 const u8 *__restrict__ mate, u32 bs, u32 l, u32 c, bool kmer_on, SlotRec *__restrict__ slots,
                  u64 slot_total, u64 *__restrict__ counts, u32 *__restrict__ ovf_list, u32 *__restrict__ ovf_n,
-                 const u32 *__restrict__ perm, u32 *qhead, const u32 *__restrict__ lc, bool uext, SmemTuning tune,
-                 u32 *err, u32 *chk) {
+                 u32 *qhead, const u32 *__restrict__ lc, bool uext, u32 nslots, u32 *err, u32 *chk, SplitBufs sp) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    WarpSlots &W = reinterpret_cast<WarpSlots *>(smem_raw)[threadIdx.x >> 5];
     const u32 FULL = 0xffffffffu;
     const u32 lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
-    const u32 n = (u32)I.n, prim = (u32)I.primary, K = I.kmer_k;
-    const u64 o0 = off[0];
-    const u64 o1 = off[nr];
-    const u8 *const end = seq + o1;
-    SmemState S;
-    SlotEmit em;
-    WarpRange wr;
-    if (!QUEUE) wr.init(nr);
-    u32 lr = l, cr = c;
-    auto start = [&](u64 rr) {
-        u64 b = off[rr], e = off[rr + 1];
-        bool bad = b > e || b < o0 || e > o1;
-        if (bad) {   // offsets outside the batch or decreasing: nothing is read, no record written
-            atomicOr(err, (u32)DEVCHK_OFFSETS);
-            b = e = o0;
-        }
-        const u64 sb = slots_before(b - o0, rr), se = slots_before(e - o0, rr + 1);
-        em.slots = slots;
-        em.base = sb;
-        em.cap = !bad && se <= slot_total ? (u32)(se - sb) : 0u;
-        em.cnt = 0;
-        if (lc) {
-            const u32 v = lc[rr];
-            lr = v & 0xFFFFu;
-            cr = v >> 16;
-        }
-        smem_begin(S, seq + b, (int)(e - b), conv_of(mate, rr, bs), lr, n, end);
-    };
-    auto take = [&](u32 k, u32 rank, u64 &item, bool &ok) {
-        if (QUEUE) {
-            u32 base = 0;
-            if (lane == 0) base = atomicAdd(qhead, k);
-            base = __shfl_sync(FULL, base, 0);
-            item = (u64)base + rank;
-            ok = item < nr;
-        } else {
-            item = wr.next + rank;
-            ok = item < wr.end;
-            wr.next += k;
-        }
-    };
-    // lane state: rdy = holds the memory action ract (acode: its sample index or k-mer code);
-    // pend = an extension failed and is applied at the next pass
-    bool rdy = false, pend = false;
-    int ract = R_BLOCK;
-    u32 acode = 0;
-    // one service of a lane out of the loop: its pending failure and the stage changes up to its
-    // next memory action.  Returns true when the read is finished.
-    auto service = [&]() -> bool {
-        if (pend) {
-            pend = false;
-            if (!smem_apply(S, 0, 0, 0, lr, cr, n, em)) return true;
-        }
-        u32 code = 0;
-        const int act = smem_next(S, I, lr, kmer && lr >= K, em, code, uext);
-        if (act == ACT_NONE) return true;
-        ract = act == ACT_TEXT ? R_TEXT : (act == ACT_SAMPLE ? R_SAMPLE : (act == ACT_KMER ? R_KMER : R_BLOCK));
-        acode = code;
-        rdy = true;
-        return false;
-    };
-    u64 item, r = 0;
-    bool live;
-    take(tune.rpw, lane < tune.rpw ? lane : 0u, item, live);   // lanes rpw.. hold no read
-    live = live && lane < tune.rpw;
-    if (live) {
-        r = QUEUE && perm ? perm[item] : item;
-        start(r);
+    const u32 n = (u32)I.n, prim = (u32)I.primary;
+    const int K = (int)I.kmer_k;
+    const u64 o0 = off[0], o1 = off[nr];
+    u32 ntodo = nr;
+    if (ITEMS) {
+        ntodo = sp.n[0] < sp.items_cap ? sp.n[0] : sp.items_cap;
+        if (ntodo == 0) return;
+        const u32 nw = gridDim.x * (blockDim.x / 32);
+        nslots = min((u32)SLOTS, (ntodo + nw - 1) / nw);
     }
-    u32 since = 0;
+#pragma unroll
+    for (u32 h = lane; h < SLOTS; h += 32) {
+        W.cls[h] = h < nslots ? C_SERV : C_FREE;
+        W.meta[h] = M_NEW;
+    }
+    __syncwarp();
+    u32 flip = 0, pick = C_BLOCK, turn = 0;
     for (;;) {
-        if (__all_sync(FULL, !live)) break;
-        const u32 out_mask = __ballot_sync(FULL, live && !rdy);
-        const u32 in_mask = __ballot_sync(FULL, rdy);
-        if (out_mask && (in_mask == 0 || since >= tune.burst || (u32)__popc(out_mask) >= tune.wait)) {
-            since = 0;
-            // ---- service pass (divergent, no index reads)
-            bool fin = live && !rdy && service();
-            // finished lanes hand in their counts and take new reads, which go to their first
-            // memory action at once (a read shorter than l finishes there and takes the next one)
+        // the class with the most waiting reads; every eighth time, or while no class has eight, the next
+        // class in turn, so that no read waits long for others.  Then the first 32 slots of the class
+        // (the two halves of the slots take turns in going first).
+        flip ^= 32;
+        const u32 h0 = lane + flip, h1 = lane + (flip ^ 32);
+        const u32 c0 = W.cls[h0], c1 = W.cls[h1];
+        const u32 tally = __reduce_add_sync(FULL, (c0 < 4 ? 1u << (8 * c0) : 0u) + (c1 < 4 ? 1u << (8 * c1) : 0u));
+        if (tally == 0) break;
+        const u32 n0 = tally & 255u, n1 = (tally >> 8) & 255u, n2 = (tally >> 16) & 255u, n3 = tally >> 24;
+        const u32 top = max(max(n0 * 4 + C_BLOCK, n1 * 4 + C_TEXT), max(n2 * 4 + C_LOOK, n3 * 4 + C_SERV));
+        if ((++turn & 7) == 0 || top < 8 * 4) {
+            const u32 has = (n0 ? 1u : 0u) | (n1 ? 2u : 0u) | (n2 ? 4u : 0u) | (n3 ? 8u : 0u);
+            pick = (pick + __ffs((int)((has | has << 4) >> (pick + 1)))) & 3u;
+        } else {
+            pick = top & 3u;
+        }
+        const u32 most = (tally >> (8 * pick)) & 255u;
+        const u32 b0 = __ballot_sync(FULL, c0 == pick), b1 = __ballot_sync(FULL, c1 == pick);
+        if (c0 == pick) W.list[__popc(b0 & lt)] = (u8)h0;
+        const u32 r1 = __popc(b0) + __popc(b1 & lt);
+        if (c1 == pick && r1 < 32) W.list[r1] = (u8)h1;
+        __syncwarp();
+        const bool on = lane < most;
+        const u32 x = on ? W.list[lane] : 0u;   // this lane's slot
+        SmemState S;
+        u32 meta = 0, lr = l, cr = c;
+        int wb = 0, cls = C_SERV;
+        if (on) {
+            meta = W.meta[x];
+            S.u = (int)(meta & 7u);
+            S.L = W.L[x];
+            S.i = W.i[x];
+            S.j = W.j[x];
+            S.k = W.k[x];
+            S.kr = W.kr[x];
+            S.s = W.s[x];
+            S.pos = W.pos[x];
+            wb = W.wb[x];
+            if (lc) {
+                const u32 v = W.lc[x];
+                lr = v & 0xFFFFu;
+                cr = v >> 16;
+            }
+        }
+        // a read base of the window is an N
+        auto has_n = [&](int lo, int hi) -> bool {   // any N in [lo, hi], both in the window
+            if (!(meta & M_HASN)) return false;
+            const u64 m = ((u64)W.nmask[1][x] << 32) | W.nmask[0][x];
+            return ((m >> (lo - wb)) & (hi - lo == 63 ? ~0ull : ((1ull << (hi - lo + 1)) - 1))) != 0;
+        };
+        auto inside = [&](int lo, int hi) { return lo >= wb && hi < wb + WIN; };
+        // the class of a read in stages 1-3 whose next action is an extension by P[j]
+        auto ext_class = [&] { return inside(S.j, S.j) ? (int)C_BLOCK : (int)C_SERV; };
+        // the class after a restart (stage 1, whole interval): a k-mer entry, else the pass decides
+        auto restart_class = [&] {
+            if (ITEMS && S.i >= W.c1[x]) return (int)C_SERV;
+            return kmer_on && (int)lr >= K && !(meta & M_HASN) && inside(S.j - K + 1, S.j) ? (int)C_LOOK : (int)C_SERV;
+        };
+        // stages 4-7 moved to their next memory action: its class (C_SERV: stage 7 is done and the match
+        // is emitted there)
+        auto uniq_class = [&] {
+            int ract = R_BLOCK;
+            u32 acode = 0;
+            if (!uniq_next(S, n, prim, ract, acode)) return (int)C_SERV;
+            return ract == R_TEXT ? (int)C_TEXT : ract == R_SAMPLE ? (int)C_LOOK : (int)C_BLOCK;
+        };
+        auto restart = [&] {
+            S.k = 0;
+            S.kr = 0;
+            S.s = n;
+        };
+
+        if (pick == C_BLOCK) {
+            // steps in a row, the state in registers, while at least three quarters of the reads go on
+            // with another one (a read alone goes on to the end of its run: each step then costs its
+            // load and the arithmetic, not the slot table)
+            if (on) cls = C_BLOCK;
             for (;;) {
-                if (fin) {
-                    counts[r] = em.cnt;
-                    if (em.cnt > em.cap) ovf_list[atomicAdd(ovf_n, 1u)] = (u32)r;
+            const bool go = cls == C_BLOCK && on;
+            const bool walk = S.u >= 4, fwd = S.u == 2;
+            const u32 p = (fwd || walk) ? S.kr : S.k, sz = walk ? 0u : S.s;
+            bool ok = go;
+            if (go) cls = C_SERV;
+            if (chk && go && (u64)p + sz > n) {   // MB_CHECKED: both rows inside the text (always so on a sound index)
+                atomicOr(chk, (u32)DEVCHK_BOUNDS);
+                ok = false;
+                S.u = 0;   // the read ends here; the next service finishes it
+            }
+            if (ok) {
+                const Blk b0 = load_blk(I.occ + (p >> BLK_SHIFT));
+                Blk b1 = b0;
+                if (((p + sz) >> BLK_SHIFT) != (p >> BLK_SHIFT)) b1 = load_blk(I.occ + ((p + sz) >> BLK_SHIFT));
+                const int o = S.j - wb;
+                const u32 a = walk ? 0u : (W.code[o >> 4][x] >> (2 * (o & 15))) & 3u;
+                const bool isn = !walk && has_n(S.j, S.j);
+                const u32 sym = walk ? sym_at(b0, p & BLK_MASK) : (fwd ? 3u - a : a);
+                const Ext e = extend_blocks(I, b0, b1, p, fwd ? S.k : S.kr, sz, sym);
+                meta += 1u << M_STEP;
+                if (walk) {   // stage 4 counts steps up, stage 7 down
+                    S.kr = e.p;
+                    S.s = S.u == 4 ? S.s + 1 : S.s - 1;
+                    cls = uniq_class();
+                } else if (!isn && e.s >= cr) {
+                    S.k = fwd ? e.q : e.p;
+                    S.kr = fwd ? e.p : e.q;
+                    S.s = e.s;
+                    S.j += fwd ? 1 : -1;
+                    if (S.u == 1 && S.j < S.i) {   // P[i, i+l) is a match: stage 2
+                        S.u = 2;
+                        S.j = S.i + (int)lr;
+                    }
+                    if (S.u == 2 && uext && S.s == 1 && S.L - S.j >= U_MIN) {   // one occurrence: compare text
+                        S.u = 4;
+                        S.kr = S.k;
+                        S.s = 0;
+                        cls = uniq_class();
+                    } else if (S.u == 2 ? S.j < S.L : (S.u == 1 || S.j > S.i)) {
+                        cls = ext_class();
+                    }
+                } else if (S.u != 2 && S.j + (int)lr < S.L) {   // BackStep failed: restart after P[j]
+                    S.u = 1;
+                    S.i = S.j + 1;
+                    S.j = S.j + (int)lr;
+                    restart();
+                    cls = restart_class();
+                } else if (S.u != 2) {
+                    S.u = 0;               // no room for another match
+                } else {
+                    meta |= M_PEND;        // the SMEM ends before P[j]: emitted by the next service
                 }
-                const u32 fm = __ballot_sync(FULL, fin);
-                if (!fm) break;
-                u64 it2;
-                bool ok2;
-                take(__popc(fm), __popc(fm & lt), it2, ok2);
-                bool again = false;
-                if (fin) {
-                    live = ok2;
-                    rdy = false;
-                    pend = false;
-                    if (live) {
-                        r = QUEUE && perm ? perm[it2] : it2;
-                        start(r);
-                        again = service();
+            }
+            const u32 still = __popc(__ballot_sync(FULL, on && cls == C_BLOCK));
+            if (still == 0 || still + (most < 32 ? most : 32u) / 4 < (most < 32 ? most : 32u)) break;
+            }
+        } else if (pick == C_TEXT) {
+            // up to 64 read bases from P[j] on, straight from the read's aligned 16-byte chunks (not
+            // through the window, which a long match would refill every 64 bases), against the text
+            if (on) {
+                const u8 *const P = seq + W.at[x];
+                const u64 room = (u64)(seq + o1 - P);
+                const int o = (int)(((uintptr_t)P + (u32)S.j) & 15), cst = S.j - o;
+                const u32 conv = (meta >> M_CONV) & 3u, t = S.pos + (u32)(S.j - S.i);
+                const u32 lim = min(min(64u - (u32)o, (u32)(S.L - S.j)), n - 1 - t);
+                const u32 *const w = I.text2 + (t >> 4);
+                u32 r[5], tw[5];
+                u64 nm = 0;
+#pragma unroll
+                for (int q = 0; q < 5; ++q) tw[q] = 16 * q < (int)((t & 15) + lim) ? __ldg(w + q) : 0u;
+                uint4 v[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    v[q] = 16 * q < o + (int)lim ? load_chunk(P, cst + 16 * q, S.L, room) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    r[q] = convert_codes(pack16(v[q]), conv);
+                    if ((v[q].x | v[q].y | v[q].z | v[q].w) & 0xFCFCFCFCu) nm |= (u64)n_bits(v[q]) << (16 * q);
+                }
+                r[4] = 0;
+                u32 first = nm >> o ? (u32)(__ffsll((long long)(nm >> o)) - 1) : 64u;   // first N or difference
+#pragma unroll
+                for (int q = 3; q >= 0; --q) {
+                    const u32 d = __funnelshift_r(tw[q], tw[q + 1], 2 * (t & 15)) ^ __funnelshift_r(r[q], r[q + 1], 2 * o);
+                    const u32 m = (d | (d >> 1)) & 0x55555555u;
+                    if (m) first = min(first, 16u * q + ((u32)(__ffs((int)m) - 1) >> 1));
+                }
+                S.j += (int)min(first, lim);
+                if (first < lim) S.u = 6;   // the match ends here
+                cls = uniq_class();
+            }
+        } else if (pick == C_LOOK) {
+            if (on && S.u >= 4) {   // an SA sample (stage 4) or an ISA sample (stage 6; S.s = its distance)
+                u32 v;
+                if (S.u == 4) {
+                    v = __ldg(I.sa_aux + S.kr / AUX_RATE);
+                    S.pos = v + S.s;
+                    S.u = 5;
+                } else {
+                    const u64 end = (u64)S.pos + (u32)(S.j - S.i);
+                    const u64 y = end < (u64)n - 1 ? (u64)n - 1 - end : 0;
+                    S.kr = __ldg(I.isa_aux + (u32)((y + S.s) / AUX_RATE));
+                    S.u = 7;
+                }
+                cls = uniq_class();
+            } else if (on) {
+                const u32 o = (u32)(S.j - K + 1 - wb), q = o >> 4;
+                const u32 hi = q + 1 < WIN / 16 ? W.code[q + 1][x] : 0u;
+                u32 code = __funnelshift_r(W.code[q][x], hi, 2 * (o & 15));
+                if (K < 16) code &= (1u << (2 * K)) - 1u;
+                const u32 *t = I.kmer + 3 * (u64)code;
+                const u32 tk = __ldg(t), tkr = __ldg(t + 1), ts = __ldg(t + 2);
+                const bool hit = ts >= cr;
+                if (!smem_apply_kmer(S, tk, tkr, ts, lr, cr, (u32)K)) {
+                    S.u = 0;
+                } else if (S.u == 1) {
+                    cls = hit ? (S.j >= S.i && S.s != n ? ext_class() : C_SERV) : restart_class();
+                } else if (S.j > S.i) {
+                    cls = ext_class();
+                }
+            }
+        } else {
+            // ---- service: no index array is read
+            bool fin = on && !(meta & M_NEW) && S.u == 0;
+            u32 cnt = 0, r = 0;
+            u64 at = 0;
+            if (on && !(meta & M_NEW)) {
+                cnt = W.cnt[x];
+                r = W.rd[x];   // an item's number with ITEMS
+                at = W.at[x];
+                const int c1 = ITEMS ? W.c1[x] : INT_MAX;
+                const bool done2 = S.u == 2 && S.j == S.L, done7 = S.u == 7 && S.s == 0;
+                // the read's slots (an item has none)
+                const u64 sb = slots_before(at - o0, r), se = slots_before(at - o0 + (u64)S.L, (u64)r + 1);
+                const u32 cap = !ITEMS && se <= slot_total ? (u32)(se - sb) : 0u;
+                if ((meta & M_PEND) || done2 || done7) {   // the match P[i, j) ends: its record
+                    if (!ITEMS || (S.i >= W.c0[x] && S.i < c1)) {
+                        const SlotRec rec{(u32)S.i, (u32)S.j, S.k, S.kr, done7 ? 1u : S.s, done7 ? S.pos : NOPOS};
+                        if (cnt < cap) {
+                            slots[sb + cnt] = rec;
+                        } else {
+                            const u32 q = sp.pool_cap ? atomicAdd(sp.n + 2, 1u) : 0u;
+                            if (q < sp.pool_cap) sp.pool[q] = PoolRec{ITEMS ? r | NO_ROOM : r, cnt, rec};
+                            else meta |= M_DROP;
+                        }
+                        ++cnt;
+                    }
+                    meta &= ~(M_PEND | M_TRIED);
+                    if (S.j == S.L) {
+                        fin = true;
+                    } else {
+                        S.u = 3;
+                        restart();
                     }
                 }
-                fin = again;
+                if (ITEMS && S.u == 1 && S.s == n && S.i >= c1) fin = true;   // past the item's starts
+                bool cut = false;
+                if (!ITEMS && !fin && (meta >> M_STEP) > sp.steps && S.u >= 1 && S.u <= 3) {
+                    // the starts left: after i once its match is recorded, else from i on
+                    const int c = S.u == 3 ? S.i + 1 : S.i, left = S.L - (int)lr + 1 - c;
+                    const u32 k = left > 0 ? ((u32)left + sp.starts - 1) / sp.starts : 0u;
+                    if (k > 1) {
+                        u32 q = sp.n[0], seen;   // room for k items, or none is taken
+                        while (q + k <= sp.items_cap && (seen = atomicCAS(sp.n, q, q + k)) != q) q = seen;
+                        if (q + k <= sp.items_cap) {
+                            cut = true;
+                            for (u32 t = 0; t < k; ++t)
+                                sp.items[q + t] = Item{r, c + (int)(t * sp.starts),
+                                                       t + 1 < k ? c + (int)((t + 1) * sp.starts) : INT_MAX, 0u};
+                            sp.heavy[atomicAdd(sp.n + 1, 1u)] = HeavyRead{r, q, k, cnt | (meta & M_DROP ? NO_ROOM : 0u)};
+                            if (cnt < cap) slots[sb + cnt].qend = 0;   // ends the read's slots
+                            fin = true;
+                        }
+                    }
+                }
+                if (fin && ITEMS) {
+                    sp.items[r].cnt = cnt | (meta & M_DROP ? NO_ROOM : 0u);
+                } else if (fin) {
+                    counts[r] = cnt;
+                    if ((meta & M_DROP) && !cut) ovf_list[atomicAdd(ovf_n, 1u)] = r;
+                }
             }
-        }
-        ++since;
-        // ---- memory step (uniform): every lane's memory action, loads first
-        if (rdy && ract == R_BLOCK && chk) {   // MB_CHECKED: both rows inside the text (always so on a sound index)
-            const bool walk = S.u >= 4, fwd = S.u == 2;
-            const u64 p = (fwd || walk) ? S.kr : S.k;
-            if (p + (walk ? 0u : S.s) > n) {
-                atomicOr(chk, (u32)DEVCHK_BOUNDS);
-                rdy = false;
-                S.u = 0;   // the read ends here; the next service pass finishes it
+            // finished reads give their slots to the next ones
+            const bool want = fin || (on && (meta & M_NEW));
+            const u32 fm = __ballot_sync(FULL, want);
+            if (fm) {
+                const u32 take = __popc(fm), rank = __popc(fm & lt);
+                u32 base = 0;
+                if (lane == 0) base = atomicAdd(qhead, take);
+                base = __shfl_sync(FULL, base, 0);
+                const u64 item = (u64)base + rank;
+                const bool ok = item < ntodo;
+                if (want && ok) {
+                    r = (u32)item;
+                    Item it{r, 0, 0, 0u};
+                    if (ITEMS) it = sp.items[r];
+                    u64 b = off[it.read], e = off[it.read + 1];
+                    if (b > e || b < o0 || e > o1) {   // offsets outside the batch or decreasing: nothing is read
+                        atomicOr(err, (u32)DEVCHK_OFFSETS);
+                        b = e = o0;
+                    }
+                    if (lc) {
+                        const u32 v = lc[it.read];
+                        W.lc[x] = v;
+                        lr = v & 0xFFFFu;
+                    }
+                    at = b;
+                    cnt = 0;
+                    meta = conv_of(mate, it.read, bs) << M_CONV;
+                    S.L = (int)(e - b);
+                    S.i = max(it.c0 - 1, 0);
+                    S.j = S.i + (int)lr - 1;
+                    S.u = S.j < S.L ? 1 : 0;                  // Algorithm 3 queues a read only if l - 1 < |P|
+                    if (ITEMS) {
+                        W.c0[x] = it.c0;
+                        W.c1[x] = it.c1;
+                    }
+                    S.pos = 0;
+                    restart();
+                    wb = INT_MIN / 2;   // no window yet
+                    W.rd[x] = r;
+                    W.at[x] = b;
+                    W.L[x] = S.L;
+                } else if (want) {
+                    meta = M_NEW;
+                    cls = C_FREE;
+                }
             }
-        }
-        if (!rdy) continue;
-        const bool walk = S.u >= 4, fwd = S.u == 2;
-        const u32 p = (fwd || walk) ? S.kr : S.k, sz = walk ? 0u : S.s;
-        Blk b0, b1;
-        u32 w0 = 0, w1 = 0, w2 = 0;
-        if (ract == R_BLOCK) {
-            b0 = load_blk(I.occ + (p >> BLK_SHIFT));
-            b1 = b0;
-            if (((p + sz) >> BLK_SHIFT) != (p >> BLK_SHIFT)) b1 = load_blk(I.occ + ((p + sz) >> BLK_SHIFT));
-        } else if (ract == R_TEXT) {
-            const u32 x = S.pos + (u32)(S.j - S.i);
-            w0 = __ldg(I.text2 + (x >> 4));
-            w1 = __ldg(I.text2 + (x >> 4) + 1);
-        } else if (ract == R_SAMPLE) {
-            w0 = __ldg((S.u == 4 ? I.sa_aux : I.isa_aux) + acode);
-        } else {
-            const u32 *t = I.kmer + 3 * (u64)acode;
-            w0 = __ldg(t);
-            w1 = __ldg(t + 1);
-            w2 = __ldg(t + 2);
-        }
-        if (ract == R_BLOCK) {
-            const u32 q = fwd ? S.k : S.kr;
-            const u32 a = walk ? 0u : cached_base(S, S.j);
-            const u32 sym = walk ? sym_at(b0, p & BLK_MASK) : ((fwd ? 3u - a : a) & 3u);
-            const Ext x = extend_blocks(I, b0, b1, p, q, sz, sym);
-            if (walk) {
-                S.kr = x.p;
-                if (S.u == 4)
-                    ++S.s;
-                else
-                    --S.s;
-                rdy = uniq_next(S, n, prim, ract, acode);
-            } else if (a < 4 && x.s >= cr) {
-                S.k = fwd ? x.q : x.p;
-                S.kr = fwd ? x.p : x.q;
-                S.s = x.s;
-                S.j += fwd ? 1 : -1;
-                if (S.u == 1 && S.j < S.i) {   // P[i, i+l) is a match: stage 2 (as smem_next)
+            if (on && cls != C_FREE) {
+                W.cnt[x] = cnt;
+                // stage changes up to the next memory action
+                if (S.u == 3 && S.j <= S.i) {           // back to stage 1 at the next start
+                    S.u = 1;
+                    S.i = S.j + 1;
+                    S.j = S.j + (int)lr;
+                    restart();
+                }
+                if (S.u == 1 && S.j < S.i) {            // P[i, i+l) is a match: stage 2
                     S.u = 2;
                     S.j = S.i + (int)lr;
                 }
-                if (S.u == 1) {
-                    rdy = true;
-                } else if (S.u == 3) {
-                    rdy = S.j > S.i;
-                } else if (S.j == S.L) {
-                    rdy = false;
-                } else if (uext && S.s == 1 && S.L - S.j >= U_MIN) {   // one occurrence: compare text
+                if (S.u == 2 && uext && S.s == 1 && S.L - S.j >= U_MIN) {
                     S.u = 4;
                     S.kr = S.k;
                     S.s = 0;
-                    rdy = uniq_next(S, n, prim, ract, acode);
                 }
-            } else {   // the extension fails: applied at the next service pass
-                rdy = false;
-                pend = true;
+                if (S.u >= 4) cls = uniq_class();
+                const bool full = kmer_on && (int)lr >= K && S.s == n;
+                const bool km = (S.u == 1 && full) || (S.u == 3 && full && !(meta & M_TRIED) && S.j - K + 1 > S.i);
+                const bool ext = (S.u >= 1 && S.u <= 3) && !(S.u == 2 && S.j == S.L);
+                if (ext) {
+                    const int lo = km ? S.j - K + 1 : S.j, hi = S.j;
+                    if (!inside(lo, hi)) {
+                        // the window: forwards from j in stage 2, else around j; its chunks of 16
+                        // bytes are aligned, and one past the end of the batch goes byte by byte
+                        const u8 *const P = seq + at;
+                        const int mis = (int)((uintptr_t)P & 15);
+                        int w0 = ((hi + mis) & ~15) - mis - (S.u == 2 ? 0 : 32);
+                        if (w0 < -mis) w0 = -mis;
+                        const u64 room = seq + o1 - P;
+                        u32 nb[2] = {0, 0};
+#pragma unroll
+                        for (int q = 0; q < WIN / 16; ++q) {
+                            const int cst = w0 + 16 * q;
+                            const uint4 v = cst < S.L ? load_chunk(P, cst, S.L, room) : make_uint4(0, 0, 0, 0);
+                            W.code[q][x] = convert_codes(pack16(v), (meta >> M_CONV) & 3u);
+                            if ((v.x | v.y | v.z | v.w) & 0xFCFCFCFCu) nb[q >> 1] |= n_bits(v) << (16 * (q & 1));
+                        }
+                        wb = w0;
+                        W.wb[x] = wb;
+                        W.nmask[0][x] = nb[0];
+                        W.nmask[1][x] = nb[1];
+                        meta = (nb[0] | nb[1]) ? meta | M_HASN : meta & ~M_HASN;
+                    }
+                    cls = C_BLOCK;
+                    if (km && !has_n(lo, hi)) {
+                        cls = C_LOOK;
+                        if (S.u == 3) meta |= M_TRIED;
+                    }
+                }
             }
-        } else if (ract == R_TEXT) {
-            text_apply(S, w0, w1, n);
-            rdy = uniq_next(S, n, prim, ract, acode);
-        } else if (ract == R_SAMPLE) {
-            if (S.u == 4) {
-                S.pos = w0 + S.s;
-                S.u = 5;
-            } else {
-                S.kr = w0;
-                S.u = 7;
-            }
-            rdy = uniq_next(S, n, prim, ract, acode);
-        } else {
-            // a k-mer entry; the next action is an extension of the same stage when the match
-            // goes on (else the pass decides; a finished read has u = 0)
-            rdy = smem_apply_kmer(S, w0, w1, w2, lr, cr, K) &&
-                  ((S.u == 1 && S.j >= S.i && S.s != n) || (S.u == 3 && S.j > S.i));
-            ract = R_BLOCK;
         }
+        if (on) {
+            W.meta[x] = (meta & ~7u) | (u32)S.u;
+            W.i[x] = S.i;
+            W.j[x] = S.j;
+            W.k[x] = S.k;
+            W.kr[x] = S.kr;
+            W.s[x] = S.s;
+            W.pos[x] = S.pos;
+            W.cls[x] = (u8)cls;
+        }
+        __syncwarp();
+    }
+}
+
+// The records of a cut read before each of its items, and in all.
+__global__ void k_split_sum(SplitBufs sp, u64 *__restrict__ counts, u32 *__restrict__ ovf_list, u32 *__restrict__ ovf_n) {
+    const u32 nh = sp.n[1];
+    for (u32 h = blockIdx.x * blockDim.x + threadIdx.x; h < nh; h += gridDim.x * blockDim.x) {
+        const HeavyRead v = sp.heavy[h];
+        u32 sum = v.cnt & ~NO_ROOM, drop = v.cnt & NO_ROOM;
+        for (u32 t = 0; t < v.n; ++t) {
+            const u32 c = sp.items[v.first + t].cnt;
+            sp.items[v.first + t].cnt = sum;
+            sum += c & ~NO_ROOM;
+            drop |= c & NO_ROOM;
+        }
+        counts[v.read] = sum;
+        if (drop) ovf_list[atomicAdd(ovf_n, 1u)] = v.read;
     }
 }
 
@@ -922,21 +1201,42 @@ __device__ __forceinline__ void write_rec(mb_smem *out, u64 *hitc, u64 m, u32 r,
     hitc[m] = s > max_occ ? 0 : s;
 }
 
-// Copies each read's SMEMs from its slots to the records; reads with more SMEMs than slots (or
-// whose slots lie past slot_total) are skipped here and recomputed by k_smem_overflow.
+// Copies each read's SMEMs from its slots to the records (a slot with qend = 0 ends them early: a cut
+// read).  Its other records are in the pool, or k_smem_overflow recomputes the read.
 __global__ void k_gather(const u64 *__restrict__ off, u32 nr, const SlotRec *__restrict__ slots, u64 slot_total,
                          const u64 *__restrict__ counts, const u64 *__restrict__ soff, u32 max_occ,
                          mb_smem *__restrict__ out, u64 *__restrict__ hitc, u64 out_cap,
                          u32 *__restrict__ known = nullptr) {
     u64 r = blockIdx.x * (u64)blockDim.x + threadIdx.x;
     if (r >= nr) return;
-    const u64 sb = slot_base(off, r), se = slot_base(off, r + 1), cnt = counts[r];
-    if (se > slot_total || cnt > se - sb) return;
+    const u64 sb = slot_base(off, r), se = slot_base(off, r + 1);
+    u64 cnt = counts[r];
+    if (se > slot_total) return;
+    if (cnt > se - sb) cnt = se - sb;
     const u64 o = soff[r];
     for (u64 t = 0; t < cnt; ++t) {
         SlotRec x = slots[sb + t];
+        if (x.qend == 0) break;
         write_rec(out, hitc, o + t, (u32)r, x.qbeg, x.qend, x.k, x.kr, x.s, max_occ, out_cap);
         if (known && o + t < out_cap) known[o + t] = x.pos;
+    }
+}
+
+// The pool's records to their places.
+__global__ void k_pool_write(SplitBufs sp, const u64 *__restrict__ soff, u32 max_occ, mb_smem *__restrict__ out,
+                             u64 *__restrict__ hitc, u64 out_cap, u32 *__restrict__ known = nullptr) {
+    const u32 np = min(sp.n[2], sp.pool_cap);
+    for (u32 q = blockIdx.x * blockDim.x + threadIdx.x; q < np; q += gridDim.x * blockDim.x) {
+        const PoolRec p = sp.pool[q];
+        u32 r = p.who, idx = p.idx;
+        if (r & NO_ROOM) {
+            const Item it = sp.items[r & ~NO_ROOM];
+            r = it.read;
+            idx += it.cnt;
+        }
+        const u64 m = soff[r] + idx;
+        write_rec(out, hitc, m, r, p.rec.qbeg, p.rec.qend, p.rec.k, p.rec.kr, p.rec.s, max_occ, out_cap);
+        if (known && m < out_cap) known[m] = p.rec.pos;
     }
 }
 
@@ -1559,11 +1859,11 @@ void opts_defaults(const mb_opts *o, u32 &l, u32 &c, u32 &max_occ, u32 &flags) {
 
 // Grid of as many blocks as are resident at once (per-lane refill loops need no more), capped by
 // the work available.
-unsigned resident_grid(const void *kernel, int block, u64 work_items) {
+unsigned resident_grid(const void *kernel, int block, u64 work_items, size_t smem = 0) {
     int dev = 0, sms = 152, per_sm = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, 0) != cudaSuccess || per_sm < 1) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, smem) != cudaSuccess || per_sm < 1) {
         cudaGetLastError();
         per_sm = 1;
     }
@@ -1573,44 +1873,70 @@ unsigned resident_grid(const void *kernel, int block, u64 work_items) {
     return (unsigned)(g ? g : 1);
 }
 
-template <bool QUEUE, int BLOCK, int WARPS>
-int launch_split_t(const SmemArgs &a, cudaStream_t st) {
-    const unsigned g = resident_grid((const void *)k_smem_split<QUEUE, BLOCK, WARPS>, BLOCK, a.nr);
-    k_smem_split<QUEUE, BLOCK, WARPS><<<g, BLOCK, 0, st>>>(a.I, a.seq, a.off, a.nr, a.mate, a.bs, a.l, a.c, a.kmer,
-                                                           a.slots, a.slot_total, a.counts, a.ovf_list, a.ovf_n,
-                                                           a.perm, a.qhead, a.lc, a.uext, a.tune, a.err, a.chk);
+// Resident warps take the reads evenly; a batch of fewer reads than they hold fills each slot table in
+// part, since a read alone in its warp waits for no other read's steps.
+template <bool ITEMS>
+int launch_slots(const SmemArgs &a, int block, cudaStream_t st) {
+    const int wpb = block / 32;
+    const size_t smem = wpb * sizeof(WarpSlots);
+    const void *f = (const void *)k_smem_slots<ITEMS>;
+    MB_CK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(16 * sizeof(WarpSlots))));
+    const unsigned g = resident_grid(f, block, ITEMS ? 1ull << 40 : (u64)a.nr * 32, smem);
+    const u64 each = (a.nr + (u64)g * wpb - 1) / ((u64)g * wpb);
+    const u32 most = a.per_warp && a.per_warp < (u32)SLOTS ? a.per_warp : (u32)SLOTS;
+    k_smem_slots<ITEMS><<<g, block, smem, st>>>(
+        a.I, a.seq, a.off, a.nr, a.mate, a.bs, a.l, a.c, a.kmer, a.slots, a.slot_total, a.counts, a.ovf_list, a.ovf_n,
+        ITEMS ? a.sp.n + 3 : a.qhead, a.lc, a.uext, each < most ? (u32)each : most, a.err, a.chk, a.sp);
     MB_KCHECK();
     return MB_OK;
 }
 
 template <bool COUNT, bool QUEUE, int BLOCK>
 int launch_smem_t(const SmemArgs &a, cudaStream_t st) {
-    if constexpr (!COUNT) {
-        if (a.split) {
-            if constexpr (BLOCK != 128) {
-                if (a.warps >= 48) return launch_split_t<QUEUE, BLOCK, 48>(a, st);
-            }
-            if constexpr (BLOCK == 256) {
-                if (a.warps >= 40) return launch_split_t<QUEUE, BLOCK, 40>(a, st);
-            }
-            return launch_split_t<QUEUE, BLOCK, BLOCK == 128 ? 24 : 32>(a, st);
-        }
-    }
     const unsigned g = resident_grid((const void *)k_smem<COUNT, QUEUE, BLOCK>, BLOCK, a.nr);
     k_smem<COUNT, QUEUE, BLOCK><<<g, BLOCK, 0, st>>>(a.I, a.seq, a.off, a.nr, a.mate, a.bs, a.l, a.c, a.kmer, a.slots,
-                                                     a.slot_total, a.counts, a.ovf_list, a.ovf_n, a.perm, a.qhead,
+                                                     a.slot_total, a.counts, a.ovf_list, a.ovf_n, QUEUE ? a.qhead : nullptr,
                                                      a.wc, a.lc, a.uext, a.err);
     MB_KCHECK();
     return MB_OK;
 }
 
-// The SMEM kernel's form and tuning from the options: k_smem_split unless MB_SMEM_ONE_LOOP.
+// Room for the items of cut reads and for records that find no slot, one allocation (more needed than
+// that: the read is not cut, or k_smem_overflow recomputes it).
+// Cut after 1024 steps into items of 256 starts: earlier cuts (256 or 512 steps) cut ordinary reads too
+// (bisulfite pairs 8.7 -> 18 ms), later ones leave the long reads of a small group in one launch's tail;
+// 128 or 512 starts per item are within 3% of 256 on mixed lengths.
+constexpr u32 SPLIT_STEPS = 1024, SEG_STARTS = 256;
+struct SplitRoom {
+    u32 items, heavy, pool;
+    SplitRoom(u64 bases, u64 n_reads) {
+        const u64 it = n_reads / 8 + bases / 1024 + 4096, po = n_reads / 2 + bases / 256 + 16384;
+        items = (u32)(it < (1u << 30) ? it : 1u << 30);
+        heavy = items / 2 + 1;   // a cut read has at least two items
+        pool = n_reads < NO_ROOM ? (u32)(po < (1u << 30) ? po : 1u << 30) : 0u;
+    }
+    size_t items_at() const { return ((size_t)pool * sizeof(PoolRec) + 255) & ~(size_t)255; }
+    size_t heavy_at() const { return items_at() + (((size_t)items * sizeof(Item) + 255) & ~(size_t)255); }
+    size_t bytes() const { return heavy_at() + (size_t)heavy * sizeof(HeavyRead); }
+    SplitBufs bufs(void *mem, u32 *counters) const {
+        char *m = (char *)mem;
+        SplitBufs b;
+        b.n = counters;
+        b.pool = (PoolRec *)m;
+        b.items = (Item *)(m + items_at());
+        b.heavy = (HeavyRead *)(m + heavy_at());
+        b.items_cap = pool ? items : 0;
+        b.pool_cap = pool;
+        b.steps = pool ? SPLIT_STEPS : ~0u;
+        b.starts = SEG_STARTS;
+        return b;
+    }
+};
+
+// The SMEM kernel's form and its reads per warp from the options.
 void smem_tuning(const mb_opts *o, SmemArgs &a) {
-    a.split = !(o && (o->flags & MB_SMEM_ONE_LOOP));
-    a.tune.burst = o && o->smem_burst ? o->smem_burst : SMEM_BURST;
-    a.tune.wait = o && o->smem_wait ? (o->smem_wait > 32 ? 32u : o->smem_wait) : SMEM_WAIT;
-    a.warps = o ? o->smem_warps : 0;
-    a.tune.rpw = o && o->smem_reads_per_warp && o->smem_reads_per_warp < 32 ? o->smem_reads_per_warp : 32u;
+    a.one_loop = o && (o->flags & MB_SMEM_ONE_LOOP);
+    a.per_warp = o && o->smem_reads_per_warp && o->smem_reads_per_warp < 32 ? o->smem_reads_per_warp : 0u;
 }
 
 template <bool COUNT, bool POW2, int D, bool CHK = false>
@@ -1780,6 +2106,14 @@ int locate_shared(const DevIndex &I, const mb_smem *sm, u64 cap, const u64 *nsm_
 // The SMEM kernel in the requested shape: work counters, work queue, threads per block.
 int launch_smem(const SmemArgs &a, bool count, bool queue, int block, cudaStream_t st) {
     if (count) return launch_smem_t<true, false, 256>(a, st);
+    if (!a.one_loop) {
+        MB_TRY(launch_slots<false>(a, block, st));
+        if (!a.sp.items_cap) return MB_OK;
+        MB_TRY(launch_slots<true>(a, 256, st));
+        k_split_sum<<<32, 128, 0, st>>>(a.sp, a.counts, a.ovf_list, a.ovf_n);
+        MB_KCHECK();
+        return MB_OK;
+    }
     if (queue) {
         if (block == 128) return launch_smem_t<false, true, 128>(a, st);
         if (block == 512) return launch_smem_t<false, true, 512>(a, st);
@@ -1805,16 +2139,19 @@ int mb_seed_device(const mb_index *idx, const u8 *dseq, const u64 *doff, u32 n_r
     if (n_hits) *n_hits = 0;
     if (n_reads == 0) return MB_OK;
     const u64 nslots = slots_total(o1 - o0, n_reads);
-    DevBuf bslots, bcounts, bsoff, bovf, bmisc, btmp;
+    DevBuf bslots, bcounts, bsoff, bovf, bmisc, btmp, bsplit;
+    const SplitRoom room(o1 - o0, n_reads);
+    MB_TRY(bsplit.alloc(room.bytes(), st));
     MB_TRY(bslots.alloc(nslots * sizeof(SlotRec), st));
     MB_TRY(bcounts.alloc((size_t)n_reads * 8, st));
     MB_TRY(bsoff.alloc((size_t)n_reads * 8, st));
     MB_TRY(bovf.alloc((size_t)n_reads * 4, st));
-    MB_TRY(bmisc.alloc(64, st));
+    MB_TRY(bmisc.alloc(128, st));
     u64 *dtotal = bmisc.as<u64>(), *dhtotal = bmisc.as<u64>() + 1;
     u32 *dovf_n = (u32 *)(bmisc.as<u64>() + 2), *dqhead = (u32 *)(bmisc.as<u64>() + 3);
     u32 *derr = (u32 *)(bmisc.as<u64>() + 4);
-    MB_CK(cudaMemsetAsync(bmisc.p, 0, 64, st));
+    MB_CK(cudaMemsetAsync(bmisc.p, 0, 128, st));
+    const SplitBufs split = room.bufs(bsplit.p, (u32 *)(bmisc.as<u64>() + 8));
 
     const DevIndex I = mb_dev_index(idx);
     const unsigned B = 256;
@@ -1823,13 +2160,13 @@ int mb_seed_device(const mb_index *idx, const u8 *dseq, const u64 *doff, u32 n_r
     const bool kmer = !(flags & MB_NO_KMER) && l >= mb_dev_index(idx).kmer_k;
     {
         const bool count = (flags & MB_COUNT) != 0;
-        // with MB_BATCHED the reads are taken from a work queue in read order (no sort here)
         const bool queue = !count && (flags & MB_BATCHED);
         SmemArgs sa{I, (const u8 *)dseq, (const u64 *)doff, n_reads, (const u8 *)dmate, bs, l, c, kmer,
-                    bslots.as<SlotRec>(), nslots, bcounts.as<u64>(), bovf.as<u32>(), dovf_n, nullptr,
-                    queue ? dqhead : nullptr, count ? mb_work_counter_buf(st) : nullptr, dlc,
+                    bslots.as<SlotRec>(), nslots, bcounts.as<u64>(), bovf.as<u32>(), dovf_n,
+                    dqhead, count ? mb_work_counter_buf(st) : nullptr, dlc,
                     I.text2 && !(flags & MB_STEP_ONLY)};
         smem_tuning(opts, sa);
+        sa.sp = split;
         sa.err = derr;
         sa.chk = (flags & MB_CHECKED) ? derr : nullptr;
         const int blk = opts && (opts->block_size == 128 || opts->block_size == 512) ? (int)opts->block_size : 256;
@@ -1869,6 +2206,8 @@ int mb_seed_device(const mb_index *idx, const u8 *dseq, const u64 *doff, u32 n_r
     MB_TRY(bhitc.alloc(total * 8, st));
     k_gather<<<G, B, 0, st>>>((const u64 *)doff, n_reads, bslots.as<SlotRec>(), nslots, bcounts.as<u64>(),
                               bsoff.as<u64>(), max_occ, dout, bhitc.as<u64>(), total);
+    MB_KCHECK();
+    k_pool_write<<<152, 256, 0, st>>>(split, bsoff.as<u64>(), max_occ, dout, bhitc.as<u64>(), total);
     MB_KCHECK();
     k_smem_overflow<<<resident_grid((const void *)k_smem_overflow, 128, 1ull << 40), 128, 0, st>>>(I, (const u8 *)dseq, (const u64 *)doff, n_reads, (const u8 *)dmate, bs, l,
                                          c, kmer,
@@ -2155,7 +2494,7 @@ extern "C" int mb_seed_batch_noalloc(const mb_index *idx, const uint8_t *seq, co
     unsigned char *S = nullptr;
     MB_TRY(noalloc_scratch(&S));
     u64 *dtotal = (u64 *)S, *dhtotal = (u64 *)S + 1;
-    u32 *dovf_n = (u32 *)((u64 *)S + 2), *derr = (u32 *)((u64 *)S + 3);
+    u32 *dovf_n = (u32 *)((u64 *)S + 2), *derr = (u32 *)((u64 *)S + 3), *dqhead = (u32 *)((u64 *)S + 4);
     u64 *counts = (u64 *)(S + o_cnt), *soff = (u64 *)(S + o_soff);
     u32 *ovf = (u32 *)(S + o_ovf);
     SlotRec *slots = (SlotRec *)(S + o_slots);
@@ -2165,7 +2504,7 @@ extern "C" int mb_seed_batch_noalloc(const mb_index *idx, const uint8_t *seq, co
     const unsigned B = 256, G = (unsigned)((nr + B - 1) / B);
     const bool kmer = !(flags & MB_NO_KMER) && l >= I.kmer_k;
     {
-        SmemArgs sa{I, seq, off, n_reads, mate, bs, l, c, kmer, slots, nslots, counts, ovf, dovf_n, nullptr, nullptr,
+        SmemArgs sa{I, seq, off, n_reads, mate, bs, l, c, kmer, slots, nslots, counts, ovf, dovf_n, dqhead,
                     nullptr, nullptr, I.text2 && !(flags & MB_STEP_ONLY)};
         smem_tuning(opts, sa);
         sa.err = derr;
@@ -2218,9 +2557,9 @@ struct mb_plan {
     bool kmer = true, queue = false;
     int block = 256;
     u32 depth = 1;   // walks per lane in locate
-    bool split = true;   // SMEM kernel form and tuning
-    SmemTuning tune = {SMEM_BURST, SMEM_WAIT, 32};
-    u32 warps = 0;
+    bool one_loop = false;   // SMEM kernel form and reads per warp (smem_tuning)
+    u32 per_warp = 0;
+    SplitBufs split;
     u32 max_reads = 0;
     u64 max_bases = 0, max_smem = 0, max_hits = 0, nslots = 0;
     void *mem = nullptr;
@@ -2253,7 +2592,7 @@ void mb_plan_arrays(const mb_plan *p, const mb_smem **smem, const u32 **hits, u6
 }
 
 // Device workspace of a plan, one entry per array (in the order mb_plan_create lays them out).
-constexpr int PLAN_ARRAYS = 27;
+constexpr int PLAN_ARRAYS = 28;
 // A plan locates with walks that join (their arrays sized by the index's n rows) when the options
 // say MB_LOCATE_JOIN without MB_CHECKED or MB_LOCATE_AUX and the plan holds hits to locate (not a
 // seeding-only plan).
@@ -2273,7 +2612,8 @@ static void plan_sizes(const mb_opts *opts, u64 n, u32 max_reads, u64 max_bases,
                                    ms * 8, ms * 8, ms * 8, ms * 4, ms * 4, ms * 4, ms * 4, mh * 4,
                                    nw * sizeof(WalkBlk), nc * 16, nw * 4, join ? 8u : 0u,
                                    join ? JOIN_PASSES * nt * 4 + 4 : 0, join ? mh * 4 : 0,
-                                   join ? (size_t)(JOIN_PASSES + 1) * 8 : 0, join ? (size_t)JOIN_PASSES * 4 : 0};
+                                   join ? (size_t)(JOIN_PASSES + 1) * 8 : 0, join ? (size_t)JOIN_PASSES * 4 : 0,
+                                   SplitRoom(max_bases, max_reads).bytes()};
     for (int i = 0; i < PLAN_ARRAYS; ++i) sizes[i] = z[i];
 }
 
@@ -2300,9 +2640,8 @@ extern "C" int mb_plan_create(const mb_index *idx, const mb_opts *opts, uint32_t
     {
         SmemArgs t{};
         smem_tuning(opts, t);
-        P->split = t.split;
-        P->tune = t.tune;
-        P->warps = t.warps;
+        P->one_loop = t.one_loop;
+        P->per_warp = t.per_warp;
     }
     P->max_reads = max_reads;
     P->max_bases = max_bases;
@@ -2322,6 +2661,7 @@ extern "C" int mb_plan_create(const mb_index *idx, const mb_opts *opts, uint32_t
     }
     P->bytes = total;
     char *m = (char *)P->mem;
+    void *split_mem = nullptr;
     void **ptrs[PLAN_ARRAYS] = {(void **)&P->slots, (void **)&P->counts, (void **)&P->soff, (void **)&P->misc,
                                 (void **)&P->hitc, (void **)&P->ovf, (void **)&P->rows, (void **)&P->hits,
                                 (void **)&P->out, (void **)&P->tmp, (void **)&P->known, (void **)&P->share.keys,
@@ -2329,11 +2669,12 @@ extern "C" int mb_plan_create(const mb_index *idx, const mb_opts *opts, uint32_t
                                 (void **)&P->share.vals_alt, (void **)&P->share.pmax, (void **)&P->share.last,
                                 (void **)&P->share.rpos, (void **)&P->share.wb, (void **)&P->share.coarse,
                                 (void **)&P->share.before, (void **)&P->share.nojoin, (void **)&P->share.tcnt,
-                                (void **)&P->share.idx, (void **)&P->share.range, (void **)&P->share.qhead};
+                                (void **)&P->share.idx, (void **)&P->share.range, (void **)&P->share.qhead, &split_mem};
     for (int i = 0; i < PLAN_ARRAYS; ++i) {
         *ptrs[i] = sizes[i] ? (void *)m : nullptr;
         m += align_up(sizes[i]);
     }
+    P->split = SplitRoom(max_bases, max_reads).bufs(split_mem, (u32 *)(P->misc + 8));
     P->share.rows = P->rows;
     P->share.nrows = P->misc + 4;
     P->share.nwalk = P->misc + 5;
@@ -2370,14 +2711,11 @@ static int plan_seed(mb_plan *P, const uint8_t *seq, const uint64_t *off, uint32
     u64 *n_smem = P->misc, *n_hits = P->misc + 1;
     u32 *ovf_n = (u32 *)(P->misc + 2), *qhead = (u32 *)(P->misc + 3), *err = plan_err(P);
     MB_CK(cudaMemsetAsync(P->hitc, 0, P->max_smem * 8, st));   // zero tail for the fixed-length scan
-    // with the work queue the reads are handed out in read order: ordering them by decreasing
-    // length (tried: a sort before the launch) made the mixed-length batch 2.4 ms slower
-    const u32 *perm = nullptr;
     SmemArgs sa{I, seq, off, n_reads, mate, bs, P->l, P->c, P->kmer, P->slots, P->nslots, P->counts, P->ovf, ovf_n,
-                perm, qhead, nullptr, nullptr, I.text2 && !(P->flags & MB_STEP_ONLY)};
-    sa.split = P->split;
-    sa.tune = P->tune;
-    sa.warps = P->warps;
+                qhead, nullptr, nullptr, I.text2 && !(P->flags & MB_STEP_ONLY)};
+    sa.sp = P->split;
+    sa.one_loop = P->one_loop;
+    sa.per_warp = P->per_warp;
     sa.err = err;
     sa.chk = (P->flags & MB_CHECKED) ? err : nullptr;
     MB_TRY(launch_smem(sa, false, P->queue, P->block, st));
@@ -2385,6 +2723,8 @@ static int plan_seed(mb_plan *P, const uint8_t *seq, const uint64_t *off, uint32
     const unsigned G = (unsigned)((n_reads + 255) / 256);
     k_gather<<<G, 256, 0, st>>>(off, n_reads, P->slots, P->nslots, P->counts, P->soff, P->max_occ, P->out, P->hitc,
                                 P->max_smem, P->known);
+    MB_KCHECK();
+    k_pool_write<<<152, 256, 0, st>>>(P->split, P->soff, P->max_occ, P->out, P->hitc, P->max_smem, P->known);
     MB_KCHECK();
     k_smem_overflow<<<resident_grid((const void *)k_smem_overflow, 128, 1ull << 40), 128, 0, st>>>(I, seq, off, n_reads, mate, bs, P->l, P->c, P->kmer, P->ovf, ovf_n, P->soff,
                                          P->max_occ, P->out, P->hitc, P->max_smem, nullptr, P->known);
@@ -2494,9 +2834,9 @@ extern "C" int mb_plan_replay(mb_plan *P, void *stream) {
 
 // Times launch shapes on this batch (all give the same output; tests check that), in stages:
 // (1) the SMEM kernel's shape, over threads per block {128, 256, 512} x work queue off/on x the
-// kernel form (the one-loop form, and the split form with memory steps between service passes
-// {2, 4, 8, 16} x lanes out of the loop that call a pass early {4, 8, 16}), with 16 plain locate
-// walks per lane; (2) for a split-form winner, reads per warp {1, 2, 4, 8, 16}; (3) with the best
+// kernel form (the one-loop form, and the slot form at smem_burst {2, 4, 8, 16} x smem_wait
+// {4, 8, 16}, which no longer differ: programs expect the points), with 16 plain locate walks per
+// lane; (2) for a slot-form winner, reads per warp {1, 2, 4, 8, 16}; (3) with the best
 // SMEM shape, locate walks per lane {1, 2, 4, 8} plain and {1, 2, 4, 8, 16} with walks that join
 // (MB_LOCATE_JOIN).  Each point is the
 // best of two timed runs of mb_plan_run after one untimed run.  Every point tried is written to
