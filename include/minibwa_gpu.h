@@ -63,16 +63,17 @@ enum {
                               by comparing text */
 #define MB_STEP_ONLY 0x40u /* seeding: extend every match step by step (Algorithm 1), even where
                               the auxiliary arrays allow comparing text */
-#define MB_LOCATE_JOIN 0x100u /* locate: the walked rows go in 8 passes (by a hash of the row); a walk
-                              stops where it meets a walked row of an earlier pass and takes that
-                              row's position plus its distance (same positions, fewer LF steps; 36
-                              bytes per 64 index rows plus 4 bytes per walked row of device
-                              workspace).  Off under MB_CHECKED.  By default every LF-walk runs to
-                              its sampled row */
+#define MB_LOCATE_JOIN 0x100u /* locate, on an index built with MB_NO_AUX (or with MB_COUNT): the walked
+                              rows go in 8 passes (by a hash of the row); a walk stops where it meets
+                              a walked row of an earlier pass and takes that row's position plus its
+                              distance (same positions, fewer LF steps; 36 bytes per 64 index rows
+                              plus 4 bytes per walked row of device workspace).  Off under
+                              MB_CHECKED.  Other indexes locate faster without it (mb_locate) */
 #define MB_LOCATE_AUX 0x200u /* locate: walks stop at the rate-4 SA samples the index keeps for
                               extending unique matches (a row that is a multiple of 4) instead of
                               the rate-r samples of Section 2.4: about r/4 times fewer LF steps, same
-                              positions; no joins.  Ignored for an index built with MB_NO_AUX */
+                              positions; no joins.  The default but under MB_COUNT and MB_CHECKED.
+                              Ignored for an index built with MB_NO_AUX */
 #define MB_SMEM_ONE_LOOP 0x80u /* tuning: the SMEM kernel in its one-loop form (one read per lane, every
                               iteration runs every stage's code) instead of the slot form (a warp
                               holds up to 64 reads and runs one kind of step for up to 32 of them at
@@ -159,7 +160,8 @@ int mb_index_export_aux(const mb_index *idx, uint32_t *text2, uint32_t *sa_aux, 
  * ds-interval of the k-mer.  Reads n x 12 bytes of the table instead of copying all of it (51.5 GB
  * at k = 16).  MB_ERR_ARG for a null pointer or a code of 4^k or more (nothing written). */
 int mb_index_kmer_get(const mb_index *idx, const uint64_t *codes, uint64_t n, uint32_t *out);
-/* Free the full suffix array kept after the build (it is only needed for mb_index_export). */
+/* Free the full suffix array kept after the build (for mb_index_export; while it is there, locate reads
+ * each hit's position from it).  Waits for the device's work; plans and captured graphs stay valid. */
 int mb_index_drop_sa(mb_index *idx);
 
 /* ---------------------------------------------------------------------------------------
@@ -223,15 +225,18 @@ int mb_seed_batch_noalloc(const mb_index *idx, const uint8_t *seq, const uint64_
 /* ---------------------------------------------------------------------------------------
  * mb_locate — text positions of every row of every SMEM without MB_SMEM_OVER_MAX_OCC
  * (Section 2.4, Algorithm 2): row x is LF-walked to a sampled row; its position is
- * (steps + S(sampled row)) mod n.
+ * (steps + S(sampled row)) mod n.  Every row is a sample while the index keeps its full suffix array
+ * (until mb_index_drop_sa); else every fourth, or every r-th on an index built with MB_NO_AUX.
  *   smem     host or device, n_smem records from mb_seed_batch (hit_off must be as written).
  *   hits     host or device, room for `cap` u32 positions; hit t of record m is written at
  *            hits[m.hit_off + t], rows k..k+s-1 in order.
  *   n_hits   receives the total.  If it exceeds cap: MB_ERR_CAPACITY, nothing written.
  * With MB_BS3 in opts, hits are still all written; mb_bs_filter applies the strand rule.
- * A row that several records share (the same or nested intervals) is walked once and its
+ * Without the full array, and for more than 2^25 hits, an index built with MB_NO_AUX, MB_COUNT or
+ * MB_CHECKED, a row that several records share (the same or nested intervals) is walked once and its
  * position copied to each of their hits; with MB_COUNT the work counters count those walks.
- * Device workspace: about 40 bytes per record and 8 per hit, allocated per call.
+ * Device workspace, allocated per call: 8 bytes per 256 to 8,192 hits; with shared walks about 40
+ * bytes per record and 8 per hit.
  */
 int mb_locate(const mb_index *idx, const mb_smem *smem, uint64_t n_smem, const mb_opts *opts,
               void *stream, uint32_t *hits, uint64_t cap, uint64_t *n_hits);

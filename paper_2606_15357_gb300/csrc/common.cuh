@@ -133,6 +133,8 @@ struct DevIndex {
     const u32 *text2;   // T[0, n-1), 16 bases per word (null without the auxiliary arrays)
     const u32 *sa_aux;  // S(x * AUX_RATE)
     const u32 *isa_aux; // row of the suffix at text position p * AUX_RATE
+    const u32 *const *sa_ref;   // device word: the full suffix array, or null once it was dropped
+    bool has_sa;        // the array is there now (it may be dropped later: kernels go by sa_ref)
 };
 // Sample rate of the auxiliary SA / ISA samples used to extend unique matches by comparison.
 constexpr u32 AUX_RATE = 4;
@@ -277,7 +279,7 @@ int radix_sort_pairs(u64 *keys, u32 *vals, u64 *keys_alt, u32 *vals_alt, size_t 
 // the third), and its device result arrays
 size_t mb_plan_bytes(const mb_plan *p);
 // device bytes mb_plan_create would allocate for these limits (no allocation)
-size_t mb_plan_workspace_bytes(const mb_opts *opts, u64 n, u32 max_reads, u64 max_bases, u64 max_smem,
+size_t mb_plan_workspace_bytes(const mb_index *idx, const mb_opts *opts, u32 max_reads, u64 max_bases, u64 max_smem,
                                u64 max_hits);
 int mb_plan_counts_async(mb_plan *p, u64 *host_counts, cudaStream_t st);
 void mb_plan_arrays(const mb_plan *p, const mb_smem **smem, const u32 **hits, u64 *max_smem, u64 *max_hits);
@@ -294,10 +296,10 @@ const u32 *mb_plan_known(const mb_plan *p);
 int mb_seed_device(const mb_index *idx, const u8 *dseq, const u64 *doff, u32 n_reads, const u8 *dmate,
                    const u32 *dlc, u64 o0, u64 o1, const mb_opts *opts, cudaStream_t st, mb_smem *out, u64 cap,
                    u64 *n_out, u64 *n_hits);
-// Locate of device records (their hits at their hit offsets), D walks per lane, walks that join
-// when `join`, walks to the rate-4 samples when `aux`; workspace allocated in stream order.
+// Locate of device records (their hits at their hit offsets) with the walk form of the options
+// (null: the defaults); workspace allocated in stream order.
 int mb_locate_records(const mb_index *idx, const mb_smem *sm, u64 n_smem, const u32 *known, u32 *hits, u64 n_hits,
-                      u32 depth, bool join, bool aux, cudaStream_t st);
+                      const mb_opts *opts, cudaStream_t st);
 // build flags of an index (MB_BS3 for the 3-base bisulfite index)
 u32 mb_index_flags(const mb_index *x);
 // drops the host-buffer pipelines kept for an index (called when the index is freed)

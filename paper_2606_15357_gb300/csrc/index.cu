@@ -30,6 +30,8 @@ struct mb_index {
     u32 *text2 = nullptr;         // T[0, n-1) at 2 bits per base, 16 per word, first in the low bits
     u32 *sa_aux = nullptr;        // S(x * AUX_RATE)
     u32 *isa_aux = nullptr;       // row of the suffix at text position p * AUX_RATE
+    const u32 **sa_ref = nullptr; // device word holding sa, null once it is dropped: kernels (also those
+                                  // of graphs captured before) read it at every launch
     int device = 0;
 };
 
@@ -50,6 +52,8 @@ DevIndex mb_dev_index(const mb_index *x) {
     I.text2 = x->text2;
     I.sa_aux = x->sa_aux;
     I.isa_aux = x->isa_aux;
+    I.sa_ref = x->sa_ref;
+    I.has_sa = x->sa != nullptr;
     return I;
 }
 int mb_index_device(const mb_index *x) { return x->device; }
@@ -453,7 +457,14 @@ static void free_index(mb_index *x) {
     if (x->text2) cudaFree(x->text2);
     if (x->sa_aux) cudaFree(x->sa_aux);
     if (x->isa_aux) cudaFree(x->isa_aux);
+    if (x->sa_ref) cudaFree(x->sa_ref);
     delete x;
+}
+
+// The device word of an index that names its full suffix array.
+static int make_sa_ref(mb_index *x) {
+    if (cudaMalloc(&x->sa_ref, sizeof(u32 *)) != cudaSuccess) return MB_ERR_NOMEM;
+    return cudaMemcpy(x->sa_ref, &x->sa, sizeof(u32 *), cudaMemcpyHostToDevice) == cudaSuccess ? MB_OK : MB_ERR_CUDA;
 }
 
 // Suffix array of T (device, n symbols) by prefix doubling.  SA (device, n) receives it.
@@ -625,6 +636,7 @@ extern "C" int mb_index_build(const uint8_t *ref, uint64_t len, const mb_opts *o
             if (cudaGetLastError() != cudaSuccess) { rc = MB_ERR_CUDA; break; }
         }
         if (cudaStreamSynchronize(st) != cudaSuccess) { rc = MB_ERR_CUDA; break; }
+        if ((rc = make_sa_ref(X)) != MB_OK) break;
     } while (0);
     {
         // give the build's temporaries (tens of GB at 1 Gbp) back to the device
@@ -659,7 +671,12 @@ extern "C" int mb_index_info(const mb_index *idx, uint64_t *n, uint64_t *primary
 
 extern "C" int mb_index_drop_sa(mb_index *idx) {
     if (!idx) return MB_ERR_ARG;
-    if (idx->sa) cudaFree(idx->sa);
+    if (!idx->sa) return MB_OK;
+    // later launches find no suffix array; those under way finish before it is freed
+    const u32 *none = nullptr;
+    MB_CK(cudaMemcpy(idx->sa_ref, &none, sizeof none, cudaMemcpyHostToDevice));
+    MB_CK(cudaDeviceSynchronize());
+    cudaFree(idx->sa);
     idx->sa = nullptr;
     return MB_OK;
 }
@@ -885,6 +902,11 @@ extern "C" int mb_index_load(const char *path, void *stream, mb_index **out) {
         free_index(X);
         mb_set_error("mb_index_load: copy to device failed");
         return MB_ERR_CUDA;
+    }
+    if (make_sa_ref(X) != MB_OK) {
+        free_index(X);
+        mb_set_error("mb_index_load: device allocation failed");
+        return MB_ERR_NOMEM;
     }
     *out = X;
     return MB_OK;

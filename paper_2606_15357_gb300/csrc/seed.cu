@@ -872,61 +872,61 @@ __global__ void __launch_bounds__(512, 2)
             // load and the arithmetic, not the slot table)
             if (on) cls = C_BLOCK;
             for (;;) {
-            const bool go = cls == C_BLOCK && on;
-            const bool walk = S.u >= 4, fwd = S.u == 2;
-            const u32 p = (fwd || walk) ? S.kr : S.k, sz = walk ? 0u : S.s;
-            bool ok = go;
-            if (go) cls = C_SERV;
-            if (chk && go && (u64)p + sz > n) {   // MB_CHECKED: both rows inside the text (always so on a sound index)
-                atomicOr(chk, (u32)DEVCHK_BOUNDS);
-                ok = false;
-                S.u = 0;   // the read ends here; the next service finishes it
-            }
-            if (ok) {
-                const Blk b0 = load_blk(I.occ + (p >> BLK_SHIFT));
-                Blk b1 = b0;
-                if (((p + sz) >> BLK_SHIFT) != (p >> BLK_SHIFT)) b1 = load_blk(I.occ + ((p + sz) >> BLK_SHIFT));
-                const int o = S.j - wb;
-                const u32 a = walk ? 0u : (W.code[o >> 4][x] >> (2 * (o & 15))) & 3u;
-                const bool isn = !walk && has_n(S.j, S.j);
-                const u32 sym = walk ? sym_at(b0, p & BLK_MASK) : (fwd ? 3u - a : a);
-                const Ext e = extend_blocks(I, b0, b1, p, fwd ? S.k : S.kr, sz, sym);
-                meta += 1u << M_STEP;
-                if (walk) {   // stage 4 counts steps up, stage 7 down
-                    S.kr = e.p;
-                    S.s = S.u == 4 ? S.s + 1 : S.s - 1;
-                    cls = uniq_class();
-                } else if (!isn && e.s >= cr) {
-                    S.k = fwd ? e.q : e.p;
-                    S.kr = fwd ? e.p : e.q;
-                    S.s = e.s;
-                    S.j += fwd ? 1 : -1;
-                    if (S.u == 1 && S.j < S.i) {   // P[i, i+l) is a match: stage 2
-                        S.u = 2;
-                        S.j = S.i + (int)lr;
-                    }
-                    if (S.u == 2 && uext && S.s == 1 && S.L - S.j >= U_MIN) {   // one occurrence: compare text
-                        S.u = 4;
-                        S.kr = S.k;
-                        S.s = 0;
-                        cls = uniq_class();
-                    } else if (S.u == 2 ? S.j < S.L : (S.u == 1 || S.j > S.i)) {
-                        cls = ext_class();
-                    }
-                } else if (S.u != 2 && S.j + (int)lr < S.L) {   // BackStep failed: restart after P[j]
-                    S.u = 1;
-                    S.i = S.j + 1;
-                    S.j = S.j + (int)lr;
-                    restart();
-                    cls = restart_class();
-                } else if (S.u != 2) {
-                    S.u = 0;               // no room for another match
-                } else {
-                    meta |= M_PEND;        // the SMEM ends before P[j]: emitted by the next service
+                const bool go = cls == C_BLOCK && on;
+                const bool walk = S.u >= 4, fwd = S.u == 2;
+                const u32 p = (fwd || walk) ? S.kr : S.k, sz = walk ? 0u : S.s;
+                bool ok = go;
+                if (go) cls = C_SERV;
+                if (chk && go && (u64)p + sz > n) {   // MB_CHECKED: both rows inside the text (always so on a sound index)
+                    atomicOr(chk, (u32)DEVCHK_BOUNDS);
+                    ok = false;
+                    S.u = 0;   // the read ends here; the next service finishes it
                 }
-            }
-            const u32 still = __popc(__ballot_sync(FULL, on && cls == C_BLOCK));
-            if (still == 0 || still + (most < 32 ? most : 32u) / 4 < (most < 32 ? most : 32u)) break;
+                if (ok) {
+                    const Blk b0 = load_blk(I.occ + (p >> BLK_SHIFT));
+                    Blk b1 = b0;
+                    if (((p + sz) >> BLK_SHIFT) != (p >> BLK_SHIFT)) b1 = load_blk(I.occ + ((p + sz) >> BLK_SHIFT));
+                    const int o = S.j - wb;
+                    const u32 a = walk ? 0u : (W.code[o >> 4][x] >> (2 * (o & 15))) & 3u;
+                    const bool isn = !walk && has_n(S.j, S.j);
+                    const u32 sym = walk ? sym_at(b0, p & BLK_MASK) : (fwd ? 3u - a : a);
+                    const Ext e = extend_blocks(I, b0, b1, p, fwd ? S.k : S.kr, sz, sym);
+                    meta += 1u << M_STEP;
+                    if (walk) {   // stage 4 counts steps up, stage 7 down
+                        S.kr = e.p;
+                        S.s = S.u == 4 ? S.s + 1 : S.s - 1;
+                        cls = uniq_class();
+                    } else if (!isn && e.s >= cr) {
+                        S.k = fwd ? e.q : e.p;
+                        S.kr = fwd ? e.p : e.q;
+                        S.s = e.s;
+                        S.j += fwd ? 1 : -1;
+                        if (S.u == 1 && S.j < S.i) {   // P[i, i+l) is a match: stage 2
+                            S.u = 2;
+                            S.j = S.i + (int)lr;
+                        }
+                        if (S.u == 2 && uext && S.s == 1 && S.L - S.j >= U_MIN) {   // one occurrence: compare text
+                            S.u = 4;
+                            S.kr = S.k;
+                            S.s = 0;
+                            cls = uniq_class();
+                        } else if (S.u == 2 ? S.j < S.L : (S.u == 1 || S.j > S.i)) {
+                            cls = ext_class();
+                        }
+                    } else if (S.u != 2 && S.j + (int)lr < S.L) {   // BackStep failed: restart after P[j]
+                        S.u = 1;
+                        S.i = S.j + 1;
+                        S.j = S.j + (int)lr;
+                        restart();
+                        cls = restart_class();
+                    } else if (S.u != 2) {
+                        S.u = 0;               // no room for another match
+                    } else {
+                        meta |= M_PEND;        // the SMEM ends before P[j]: emitted by the next service
+                    }
+                }
+                const u32 still = __popc(__ballot_sync(FULL, on && cls == C_BLOCK));
+                if (still == 0 || still + (most < 32 ? most : 32u) / 4 < (most < 32 ? most : 32u)) break;
             }
         } else if (pick == C_TEXT) {
             // up to 64 read bases from P[j] on, straight from the read's aligned 16-byte chunks (not
@@ -1010,7 +1010,7 @@ __global__ void __launch_bounds__(512, 2)
                 if ((meta & M_PEND) || done2 || done7) {   // the match P[i, j) ends: its record
                     if (!ITEMS || (S.i >= W.c0[x] && S.i < c1)) {
                         const SlotRec rec{(u32)S.i, (u32)S.j, S.k, S.kr, done7 ? 1u : S.s, done7 ? S.pos : NOPOS};
-                        if (cnt < cap) {
+                        if (!ITEMS && cnt < cap) {
                             slots[sb + cnt] = rec;
                         } else {
                             const u32 q = sp.pool_cap ? atomicAdd(sp.n + 2, 1u) : 0u;
@@ -1042,7 +1042,7 @@ __global__ void __launch_bounds__(512, 2)
                                 sp.items[q + t] = Item{r, c + (int)(t * sp.starts),
                                                        t + 1 < k ? c + (int)((t + 1) * sp.starts) : INT_MAX, 0u};
                             sp.heavy[atomicAdd(sp.n + 1, 1u)] = HeavyRead{r, q, k, cnt | (meta & M_DROP ? NO_ROOM : 0u)};
-                            if (cnt < cap) slots[sb + cnt].qend = 0;   // ends the read's slots
+                            if (!ITEMS && cnt < cap) slots[sb + cnt].qend = 0;   // ends the read's slots
                             fin = true;
                         }
                     }
@@ -1836,6 +1836,166 @@ __global__ void __launch_bounds__(256, D <= 2 ? 4 : (D <= 4 ? 3 : (D <= 8 ? 2 : 
     work.flush(wc);
 }
 
+// ---------------------------------------------------------------------------- locate, every hit on its own
+// Where the samples lie dense (an index's rate-4 samples, or the full suffix array while it is kept) a
+// hit costs 1 to about 7 reads, less than the bookkeeping that lets records share their walks: no
+// sort, no scans, no row list.  A warp takes 32 records (their hits lie one after the other), and its
+// lanes take the hits in order: SA[row] where the full array is there, else an LF-walk to a row that
+// is a multiple of r (Algorithm 2), the lane going on to the next hit when its walk ends.  Lanes hold
+// neighbouring rows, whose blocks and samples mostly share sectors.  A group's hits after the first
+// `chunk` are left to a second launch, in pieces of `chunk`, so that records with many hits spread
+// over the whole chip.
+//
+// Bound: with the full array, the copy of each interval (2M reads on 100 Mbp, 13.6M hits: 0.15 ms for
+// the kernel, where walking each distinct row to the rate-32 samples and its bookkeeping took 2.2 ms
+// in about 45 launches); without it, the random reads of the walks (the same hits: 1.1 ms).
+struct DirectBufs {
+    u64 *list = nullptr;   // pieces left over: group << 32 | number of the piece (from 1), or DIRECT_NONE
+    u32 *n = nullptr;      // their count
+    u32 chunk = 0, cap = 0;
+};
+constexpr u64 DIRECT_NONE = ~0ull;
+// hits per piece: about one piece per resident warp of a small batch, at most 8192
+inline u32 direct_chunk(u64 hits) {
+    u64 c = 256;
+    while (c < 8192 && c * 4864 < hits) c *= 2;
+    return (u32)c;
+}
+inline u64 direct_list(u64 hits) { return hits / direct_chunk(hits) + 1; }
+inline DirectBufs direct_bufs(u64 *list, u32 *n, u64 hits) {
+    const u32 c = direct_chunk(hits);
+    return DirectBufs{list, n, c, hits > c ? (u32)direct_list(hits) : 0u};
+}
+
+struct DirectGroup {   // one piece: the records' hits as ranges of the piece
+    u32 end[32];       // hits of the piece before the end of record q
+    u32 row[32];       // row of record q's hits, less their number in the piece
+    u64 dst[32];       // their places in the output, less the same
+};
+
+template <bool REST>
+__global__ void __launch_bounds__(256)
+    k_locate_direct(DevIndex I, const mb_smem *__restrict__ sm, u64 cap, const u64 *__restrict__ nsm_dev,
+                    const u32 *__restrict__ known, u32 *__restrict__ hits, u64 hits_cap, DirectBufs D, u32 *err) {
+    __shared__ DirectGroup sg[8];
+    DirectGroup &G = sg[threadIdx.x >> 5];
+    const u32 FULL = 0xffffffffu, lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
+    const u64 nsm = count_of(cap, nsm_dev);
+    const u64 items = REST ? (u64)min(*D.n, D.cap) : (nsm + 31) / 32;
+    const u64 nwarps = ((u64)gridDim.x * blockDim.x) >> 5;
+    const u32 *const sa = *I.sa_ref;
+    const u32 prim = (u32)I.primary, n = (u32)I.n, rmask = I.r - 1, rshift = __ffs((int)I.r) - 1;
+    const u32 C0 = (u32)I.C[0], C1 = (u32)I.C[1], C2 = (u32)I.C[2], C3 = (u32)I.C[3];
+    for (u64 it = (blockIdx.x * (u64)blockDim.x + threadIdx.x) >> 5; it < items; it += nwarps) {
+        const u64 piece = REST ? D.list[it] : 0;
+        if (REST && piece == DIRECT_NONE) continue;
+        const u64 g = REST ? piece >> 32 : it, m = g * 32 + lane;
+        u64 base = REST ? (piece & 0xFFFFFFFFull) * D.chunk : 0;   // the piece's first hit
+        u64 cnt = 0, ho = 0;
+        u32 k = 0;
+        if (m < nsm) {
+            const u64 *p = reinterpret_cast<const u64 *>(sm + m);   // read, qbeg | qend, flags | k | kr | s | hit_off
+            const u64 k64 = __ldg(p + 2);
+            cnt = (__ldg(p + 1) >> 32) & MB_SMEM_OVER_MAX_OCC ? 0 : __ldg(p + 4);
+            ho = __ldg(p + 5);
+            k = (u32)k64;
+            if (cnt && (k64 >= I.n || cnt > I.n - k64)) {   // rows outside the text: left out
+                atomicOr(err, (u32)DEVCHK_RECORD);
+                cnt = 0;
+            } else if (cnt == 1 && known && known[m] != NOPOS) {   // found while seeding
+                if (!REST && ho < hits_cap) hits[ho] = known[m];
+                cnt = 0;
+            } else if (cnt) {
+                cnt = ho < hits_cap ? (cnt < hits_cap - ho ? cnt : hits_cap - ho) : 0;
+            }
+        }
+        u64 incl = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const u64 v = __shfl_up_sync(FULL, incl, o);
+            if (lane >= (u32)o) incl += v;
+        }
+        const u64 total = __shfl_sync(FULL, incl, 31);
+        u64 upto = total < base + D.chunk ? total : base + D.chunk;   // the hits this warp locates now
+        if (!REST && total > D.chunk) {
+            const u64 more = (total - 1) / D.chunk;
+            u32 at = D.cap;
+            if (more <= D.cap && __shfl_sync(FULL, *(volatile u32 *)D.n, 0) < D.cap) {   // (the count may pass cap, never wrap)
+                if (lane == 0) at = atomicAdd(D.n, (u32)more);
+                at = __shfl_sync(FULL, at, 0);
+            }
+            const bool room = at < D.cap && more <= D.cap - at;
+            for (u64 q = lane; q < more && at + q < D.cap; q += 32) D.list[at + q] = room ? (g << 32) | (q + 1) : DIRECT_NONE;
+            if (!room) upto = total;   // records that share places (only a caller's) can hold more hits than the output
+        }
+        for (; base < upto; base += D.chunk) {
+            const u32 len = (u32)(total - base < D.chunk ? total - base : D.chunk);
+            __syncwarp();   // the last piece's ranges were read
+            G.end[lane] = incl > base ? (u32)(incl - base < len ? incl - base : len) : 0u;
+            G.row[lane] = k - (u32)(incl - cnt - base);
+            G.dst[lane] = ho - (incl - cnt - base);
+            __syncwarp();
+            // the record of hit t of the piece: the first whose hits end after it
+            auto record = [&](u32 t) {
+                u32 q = 0;
+    #pragma unroll
+                for (u32 b = 16; b; b >>= 1)
+                    if (G.end[q + b - 1] <= t) q += b;
+                return q;
+            };
+            if (sa) {
+                for (u32 t0 = 0; t0 < len; t0 += 128) {   // four hits in flight per lane
+                    u32 v[4];
+                    u64 to[4];
+    #pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const u32 t = t0 + 32 * u + lane;
+                        if (t < len) {
+                            const u32 q = record(t);
+                            v[u] = __ldg(sa + (G.row[q] + t));
+                            to[u] = G.dst[q] + t;
+                        }
+                    }
+    #pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (t0 + 32 * u + lane < len) hits[to[u]] = v[u];
+                }
+                continue;   // the next piece
+            }
+            u32 next = 32, steps = 0, row = 0;
+            u64 to = 0;
+            bool live = lane < len;
+            if (live) {
+                const u32 q = record(lane);
+                row = G.row[q] + lane;
+                to = G.dst[q] + lane;
+            }
+            while (__any_sync(FULL, live)) {
+                const bool stop = live && ((row & rmask) == 0 || row == prim || steps > n);
+                if (stop) {   // steps > n: only on a damaged index
+                    const u32 s = (row & rmask) == 0 ? __ldg(I.ssa + (row >> rshift)) : 0u;
+                    hits[to] = steps > n ? 0xFFFFFFFFu : s + steps;
+                } else if (live) {
+                    row = lf_blk(load_blk(I.occ + (row >> BLK_SHIFT)), row, prim, C0, C1, C2, C3);
+                    ++steps;
+                }
+                const u32 done = __ballot_sync(FULL, stop);
+                if (stop) {
+                    const u32 t = next + __popc(done & lt);
+                    live = t < len;
+                    steps = 0;
+                    if (live) {
+                        const u32 q = record(t);
+                        row = G.row[q] + t;
+                        to = G.dst[q] + t;
+                    }
+                }
+                next += __popc(done);
+            }
+        }
+    }
+}
+
 __global__ void k_bs_filter(const mb_smem *__restrict__ sm, u64 nsm, const u8 *__restrict__ mate,
                             const u32 *__restrict__ hits, u64 nhits, u64 M, u8 *__restrict__ keep) {
     for (u64 h = blockIdx.x * (u64)blockDim.x + threadIdx.x; h < nhits; h += (u64)gridDim.x * blockDim.x) {
@@ -2089,10 +2249,11 @@ int locate_shared(const DevIndex &I, const mb_smem *sm, u64 cap, const u64 *nsm_
         for (u32 p = 0; p < (u32)JOIN_PASSES; ++p) MB_TRY(launch_join(I, b.rows, hits_cap, p, b.rpos, b, wc, count, depth, st));
         if (kt) kt->stop();
     } else {
-        DevIndex L = I;   // with MB_LOCATE_AUX the walks stop at the rate-4 samples
-        if (aux) {
+        DevIndex L = I;
+        if (aux) {   // short walks to the rate-4 samples: four per lane at least (2: 20% slower)
             L.ssa = I.sa_aux;
             L.r = AUX_RATE;
+            if (depth < 4) depth = 4;
         }
         if (kt) kt->start();
         MB_TRY(launch_locate(L, b.rows, hits_cap, b.nrows, b.rpos, b.lq, wc, count, depth, chk, st));
@@ -2101,6 +2262,47 @@ int locate_shared(const DevIndex &I, const mb_smem *sm, u64 cap, const u64 *nsm_
     k_share_copy<<<G, 256, 0, st>>>(b.keys, ss, sho, b.last, b.roff, cap, b.nwalk, b.rpos, hits_cap, hits, hits_cap);
     MB_KCHECK();
     return MB_OK;
+}
+
+// The hits of records sm[0, min(cap, *nsm_dev)) by k_locate_direct.
+int locate_direct(const DevIndex &I, const mb_smem *sm, u64 cap, const u64 *nsm_dev, const u32 *known, u32 *hits,
+                  u64 hits_cap, const DirectBufs &D, u32 *err, cudaStream_t st) {
+    if (cap == 0) return MB_OK;
+    DevIndex L = I;
+    if (I.sa_aux && I.r > AUX_RATE) {   // the denser samples
+        L.ssa = I.sa_aux;
+        L.r = AUX_RATE;
+    }
+    MB_CK(cudaMemsetAsync(D.n, 0, 4, st));
+    const unsigned g = resident_grid((const void *)k_locate_direct<false>, 256, cap);
+    k_locate_direct<false><<<g, 256, 0, st>>>(L, sm, cap, nsm_dev, known, hits, hits_cap, D, err);
+    MB_KCHECK();
+    if (D.cap == 0) return MB_OK;
+    const unsigned r = resident_grid((const void *)k_locate_direct<true>, 256, (u64)D.cap * 32);
+    k_locate_direct<true><<<r, 256, 0, st>>>(L, sm, cap, nsm_dev, known, hits, hits_cap, D, err);
+    MB_KCHECK();
+    return MB_OK;
+}
+
+// Whether locate gives every hit its own walk (k_locate_direct): the index has its full suffix array, or
+// samples every AUX_RATE rows and a batch of at most DIRECT_WALKS hits.  More hits repeat more rows, and
+// then sharing the walks pays for its sort: 13M / 27M / 82M hits on a 100 Mbp index without its full
+// array took 1.1 / 1.7-1.9 / 3.4 ms hit by hit and 1.3 / 1.2-2.3 / 2.3 ms shared (8% and 45% repeats),
+// 121M and 605M hits on 1 Gbp 4.8 / 19.9 ms and 3.0 / about 11 ms.  The work counters (MB_COUNT) and
+// MB_CHECKED belong to the shared walks.
+constexpr u64 DIRECT_WALKS = 32ull << 20;
+bool locate_is_direct(const DevIndex &I, u32 flags, u64 hits) {
+    return !(flags & (MB_COUNT | MB_CHECKED)) && (I.sa_aux || I.r == 1 || I.r == 2 || I.r == AUX_RATE) &&
+           (I.has_sa || hits <= DIRECT_WALKS);
+}
+// Shared walks stop at the rate-4 samples where the index has them (about an eighth of the LF steps of
+// rate 32, and fewer than walks that join take), except under MB_COUNT and MB_CHECKED, which keep the
+// walks their flags name.
+bool locate_aux(const DevIndex &I, u32 flags) {
+    return I.sa_aux && ((flags & MB_LOCATE_AUX) || !(flags & (MB_COUNT | MB_CHECKED)));
+}
+bool locate_joins(const DevIndex &I, u32 flags) {
+    return (flags & MB_LOCATE_JOIN) && !(flags & (MB_CHECKED | MB_LOCATE_AUX)) && !locate_aux(I, flags);
 }
 
 // The SMEM kernel in the requested shape: work counters, work queue, threads per block.
@@ -2304,14 +2506,23 @@ static int share_alloc(DevBuf &bw, u64 n_smem, u64 total, u64 n, bool join, cuda
 }
 
 int mb_locate_records(const mb_index *idx, const mb_smem *sm, u64 n_smem, const u32 *known, u32 *hits, u64 n_hits,
-                      u32 depth, bool join, bool aux, cudaStream_t st) {
+                      const mb_opts *opts, cudaStream_t st) {
     if (n_smem == 0 || n_hits == 0) return MB_OK;
     DevBuf bw;
-    ShareBufs b;
     const DevIndex I = mb_dev_index(idx);
-    MB_TRY(share_alloc(bw, n_smem, n_hits, I.n, join && !aux && n_hits > 1, st, b));
-    b.aux = aux;
-    return locate_shared(I, sm, n_smem, nullptr, known, hits, n_hits, b, nullptr, false, depth, nullptr, st);
+    const u32 flags = opts ? opts->flags & ~(u32)MB_COUNT : 0u;
+    if (locate_is_direct(I, flags & ~(u32)MB_CHECKED, n_hits)) {
+        MB_TRY(bw.alloc(64 + direct_list(n_hits) * 8, st));
+        u32 *w = bw.as<u32>();
+        MB_CK(cudaMemsetAsync(w, 0, 64, st));
+        return locate_direct(I, sm, n_smem, nullptr, known, hits, n_hits,
+                             direct_bufs(bw.as<u64>() + 8, w, n_hits), w + 1, st);
+    }
+    ShareBufs b;
+    MB_TRY(share_alloc(bw, n_smem, n_hits, I.n, locate_joins(I, flags) && n_hits > 1, st, b));
+    b.aux = locate_aux(I, flags);
+    return locate_shared(I, sm, n_smem, nullptr, known, hits, n_hits, b, nullptr, false,
+                         opts ? opts->prefetch_depth : 0, nullptr, st);
 }
 
 extern "C" int mb_locate(const mb_index *idx, const mb_smem *smem, uint64_t n_smem, const mb_opts *opts,
@@ -2346,15 +2557,24 @@ extern "C" int mb_locate(const mb_index *idx, const mb_smem *smem, uint64_t n_sm
     const bool count = opts && (opts->flags & MB_COUNT);
     DevBuf bw;
     ShareBufs b;
-    MB_TRY(share_alloc(bw, n_smem, total, I.n,
-                       opts && (opts->flags & MB_LOCATE_JOIN) && !(opts->flags & (MB_CHECKED | MB_LOCATE_AUX)), st,
-                       b));
-    b.aux = opts && (opts->flags & MB_LOCATE_AUX);
-    b.checked = opts && (opts->flags & MB_CHECKED);
-    u64 *wc = count ? mb_work_counter_buf(st) : nullptr;
     KTimer kt("locate", st);
-    MB_TRY(locate_shared(I, (const mb_smem *)dsm, n_smem, nullptr, nullptr, dh, total, b, wc, count,
-                         opts ? opts->prefetch_depth : 0, &kt, st));
+    const u32 flags = opts ? opts->flags : 0u;
+    if (locate_is_direct(I, flags, total)) {
+        MB_TRY(bw.alloc(64 + direct_list(total) * 8, st));
+        b.err = bw.as<u32>() + 1;
+        MB_CK(cudaMemsetAsync(bw.p, 0, 64, st));
+        kt.start();
+        MB_TRY(locate_direct(I, (const mb_smem *)dsm, n_smem, nullptr, nullptr, dh, total,
+                             direct_bufs(bw.as<u64>() + 8, bw.as<u32>(), total), b.err, st));
+        kt.stop();
+    } else {
+        MB_TRY(share_alloc(bw, n_smem, total, I.n, locate_joins(I, flags), st, b));
+        b.aux = locate_aux(I, flags);
+        b.checked = opts && (opts->flags & MB_CHECKED);
+        u64 *wc = count ? mb_work_counter_buf(st) : nullptr;
+        MB_TRY(locate_shared(I, (const mb_smem *)dsm, n_smem, nullptr, nullptr, dh, total, b, wc, count,
+                             opts ? opts->prefetch_depth : 0, &kt, st));
+    }
     u32 err = 0;
     MB_CK(cudaMemcpyAsync(&err, b.err, 4, cudaMemcpyDeviceToHost, st));
     if (!hdev) MB_CK(cudaMemcpyAsync(hits, dh, total * 4, cudaMemcpyDeviceToHost, st));
@@ -2567,6 +2787,8 @@ struct mb_plan {
     u64 *counts = nullptr, *soff = nullptr, *misc = nullptr, *hitc = nullptr;
     u32 *ovf = nullptr, *rows = nullptr, *hits = nullptr;
     u32 *known = nullptr;   // per record: the hit position found while seeding, or NOPOS
+    bool is_direct = false; // locate hit by hit (DirectBufs), else with shared walks (ShareBufs)
+    DirectBufs direct;
     ShareBufs share;        // shared-walk locate: per-record arrays, positions of the walked rows
     mb_smem *out = nullptr;
     void *tmp = nullptr;
@@ -2592,35 +2814,37 @@ void mb_plan_arrays(const mb_plan *p, const mb_smem **smem, const u32 **hits, u6
 }
 
 // Device workspace of a plan, one entry per array (in the order mb_plan_create lays them out).
-constexpr int PLAN_ARRAYS = 28;
-// A plan locates with walks that join (their arrays sized by the index's n rows) when the options
-// say MB_LOCATE_JOIN without MB_CHECKED or MB_LOCATE_AUX and the plan holds hits to locate (not a
-// seeding-only plan).
-static bool plan_joins(const mb_opts *opts, u64 max_hits) {
-    return opts && (opts->flags & MB_LOCATE_JOIN) && !(opts->flags & (MB_CHECKED | MB_LOCATE_AUX)) && max_hits > 1;
+constexpr int PLAN_ARRAYS = 29;
+static u32 plan_flags(const mb_opts *opts) { return opts ? opts->flags & ~(u32)MB_COUNT : 0u; }
+static bool plan_direct(const DevIndex &I, const mb_opts *opts, u64 max_hits) {
+    return locate_is_direct(I, plan_flags(opts), max_hits);
 }
-static void plan_sizes(const mb_opts *opts, u64 n, u32 max_reads, u64 max_bases, u64 max_smem, u64 max_hits,
+static bool plan_joins(const DevIndex &I, const mb_opts *opts, u64 max_hits) {   // (not a seeding-only plan)
+    return max_hits > 1 && locate_joins(I, plan_flags(opts)) && !plan_direct(I, opts, max_hits);
+}
+static void plan_sizes(const DevIndex &I, const mb_opts *opts, u32 max_reads, u64 max_bases, u64 max_smem, u64 max_hits,
                        size_t sizes[PLAN_ARRAYS]) {
     const size_t nr = max_reads, ms = max_smem ? max_smem : 1, mh = max_hits ? max_hits : 1;
+    const bool direct = plan_direct(I, opts, max_hits), join = plan_joins(I, opts, max_hits);
+    const size_t sr = direct ? 0 : ms, sh = direct ? 0 : mh;   // shared walks: their records and rows
     size_t tb = scan_tmp_bytes(nr > ms ? nr : ms);
-    const size_t sb = share_tmp_bytes(ms, mh);
+    const size_t sb = direct ? 0 : share_tmp_bytes(ms, mh);
     if (sb > tb) tb = sb;
-    const bool join = plan_joins(opts, max_hits);
-    const size_t nw = join ? join_words(n) : 0, nc = join ? join_coarse(n) : 0, nt = join ? join_tiles(mh) : 0;
+    const size_t nw = join ? join_words(I.n) : 0, nc = join ? join_coarse(I.n) : 0, nt = join ? join_tiles(mh) : 0;
     const size_t z[PLAN_ARRAYS] = {slots_total(max_bases, max_reads) * sizeof(SlotRec), nr * 8, nr * 8, 256, ms * 8,
-                                   nr * 4, mh * 4, mh * 4, ms * sizeof(mb_smem), tb, ms * 4,
-                                   ms * 8, ms * 8, ms * 8, ms * 4, ms * 4, ms * 4, ms * 4, mh * 4,
+                                   nr * 4, sh * 4, mh * 4, ms * sizeof(mb_smem), tb, ms * 4,
+                                   sr * 8, sr * 8, sr * 8, sr * 4, sr * 4, sr * 4, sr * 4, sh * 4,
                                    nw * sizeof(WalkBlk), nc * 16, nw * 4, join ? 8u : 0u,
                                    join ? JOIN_PASSES * nt * 4 + 4 : 0, join ? mh * 4 : 0,
                                    join ? (size_t)(JOIN_PASSES + 1) * 8 : 0, join ? (size_t)JOIN_PASSES * 4 : 0,
-                                   SplitRoom(max_bases, max_reads).bytes()};
+                                   SplitRoom(max_bases, max_reads).bytes(), direct ? direct_list(mh) * 8 : 0};
     for (int i = 0; i < PLAN_ARRAYS; ++i) sizes[i] = z[i];
 }
 
-size_t mb_plan_workspace_bytes(const mb_opts *opts, u64 n, u32 max_reads, u64 max_bases, u64 max_smem,
+size_t mb_plan_workspace_bytes(const mb_index *idx, const mb_opts *opts, u32 max_reads, u64 max_bases, u64 max_smem,
                                u64 max_hits) {
     size_t sizes[PLAN_ARRAYS], total = 0;
-    plan_sizes(opts, n, max_reads, max_bases, max_smem, max_hits, sizes);
+    plan_sizes(mb_dev_index(idx), opts, max_reads, max_bases, max_smem, max_hits, sizes);
     for (size_t z : sizes) total += align_up(z);
     return total;
 }
@@ -2649,8 +2873,8 @@ extern "C" int mb_plan_create(const mb_index *idx, const mb_opts *opts, uint32_t
     P->max_hits = max_hits ? max_hits : 1;
     P->nslots = slots_total(max_bases, max_reads);
     size_t sizes[PLAN_ARRAYS];
-    const u64 n_rows = mb_dev_index(idx).n;
-    plan_sizes(opts, n_rows, max_reads, max_bases, max_smem, max_hits, sizes);
+    const DevIndex I = mb_dev_index(idx);
+    plan_sizes(I, opts, max_reads, max_bases, max_smem, max_hits, sizes);
     size_t total = 0;
     for (size_t z : sizes) total += align_up(z);
     if (cudaMalloc(&P->mem, total) != cudaSuccess) {
@@ -2669,7 +2893,8 @@ extern "C" int mb_plan_create(const mb_index *idx, const mb_opts *opts, uint32_t
                                 (void **)&P->share.vals_alt, (void **)&P->share.pmax, (void **)&P->share.last,
                                 (void **)&P->share.rpos, (void **)&P->share.wb, (void **)&P->share.coarse,
                                 (void **)&P->share.before, (void **)&P->share.nojoin, (void **)&P->share.tcnt,
-                                (void **)&P->share.idx, (void **)&P->share.range, (void **)&P->share.qhead, &split_mem};
+                                (void **)&P->share.idx, (void **)&P->share.range, (void **)&P->share.qhead, &split_mem,
+                                (void **)&P->direct.list};
     for (int i = 0; i < PLAN_ARRAYS; ++i) {
         *ptrs[i] = sizes[i] ? (void *)m : nullptr;
         m += align_up(sizes[i]);
@@ -2682,8 +2907,10 @@ extern "C" int mb_plan_create(const mb_index *idx, const mb_opts *opts, uint32_t
     P->share.err = plan_err(P);
     P->share.lq = (u32 *)(P->misc + 6);
     P->share.checked = (P->flags & MB_CHECKED) != 0;
-    P->share.join = plan_joins(opts, max_hits);
-    P->share.aux = (P->flags & MB_LOCATE_AUX) != 0;
+    P->share.join = plan_joins(I, opts, max_hits);
+    P->is_direct = plan_direct(I, opts, max_hits);
+    P->direct = direct_bufs(P->direct.list, (u32 *)(P->misc + 10), P->max_hits);
+    P->share.aux = locate_aux(I, plan_flags(opts));
     *out = P;
     return MB_OK;
 }
@@ -2747,9 +2974,11 @@ extern "C" int mb_plan_run(mb_plan *P, const uint8_t *seq, const uint64_t *off, 
     cudaStream_t st = (cudaStream_t)stream;
     MB_TRY(plan_seed(P, seq, off, n_reads, mate, st));
     if (n_reads == 0) return MB_OK;
-    MB_TRY(locate_shared(mb_dev_index(P->idx), P->out, P->max_smem, P->misc, P->known, P->hits, P->max_hits,
-                         P->share, nullptr, false, P->depth, nullptr, st));
-    return MB_OK;
+    if (P->is_direct)
+        return locate_direct(mb_dev_index(P->idx), P->out, P->max_smem, P->misc, P->known, P->hits, P->max_hits,
+                             P->direct, P->share.err, st);
+    return locate_shared(mb_dev_index(P->idx), P->out, P->max_smem, P->misc, P->known, P->hits, P->max_hits,
+                         P->share, nullptr, false, P->depth, nullptr, st);
 }
 
 extern "C" int mb_plan_result(mb_plan *P, void *stream, const mb_smem **smem, uint64_t *n_smem, const uint32_t **hits,

@@ -196,9 +196,7 @@ void free_slot(Slot &s) {
 }
 
 size_t slot_device_bytes(const mb_index *idx, const mb_opts *o) {
-    u64 n = 0, prim = 0, rl = 0;
-    mb_index_info(idx, &n, &prim, &rl);
-    return mb_plan_workspace_bytes(o, n, SLOT_READS, SLOT_BASES, SLOT_SMEM, SLOT_HITS) + SLOT_BASES + 16 +
+    return mb_plan_workspace_bytes(idx, o, SLOT_READS, SLOT_BASES, SLOT_SMEM, SLOT_HITS) + SLOT_BASES + 16 +
            (SLOT_READS + 2) * 8;
 }
 
