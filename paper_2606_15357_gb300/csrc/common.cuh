@@ -295,7 +295,7 @@ const u32 *mb_plan_known(const mb_plan *p);
 // except out.
 int mb_seed_device(const mb_index *idx, const u8 *dseq, const u64 *doff, u32 n_reads, const u8 *dmate,
                    const u32 *dlc, u64 o0, u64 o1, const mb_opts *opts, cudaStream_t st, mb_smem *out, u64 cap,
-                   u64 *n_out, u64 *n_hits);
+                   u64 *n_out, u64 *n_hits, const uint2 *winfo = nullptr);
 // Locate of device records (their hits at their hit offsets) with the walk form of the options
 // (null: the defaults); workspace allocated in stream order.
 int mb_locate_records(const mb_index *idx, const mb_smem *sm, u64 n_smem, const u32 *known, u32 *hits, u64 n_hits,
