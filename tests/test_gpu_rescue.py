@@ -70,3 +70,38 @@ def test_periodic_pairs_and_empty_batch(mb):
     assert len(e) == 0
     with pytest.raises(mb.MbError):
         mb.mb_rescue_prefilter(P, np.array([0, 200], np.uint64), W, np.array([0, 800], np.uint64), q=16)
+
+
+@pytest.mark.parametrize("m", [6, 31, 32, 33, 64, 96, 97, 128, 160, 161, 256, 257])
+def test_word_edges(mb, m):
+    """Read and window lengths around the 32-base words of the register form (reads up to 256 bases) and
+    past it, unaligned in memory, q at and off 7, matches up to both ends of the window."""
+    rng = np.random.default_rng(m)
+    reads, wins = [rng.integers(0, 4, 1).astype(np.uint8)], [rng.integers(0, 4, 3).astype(np.uint8)]
+    for w in (m, m + 1, 31, 32, 33, 63, 64, 65, 600, 1023, 1025):
+        for at in (0, 1):
+            W = rng.integers(0, 2, w).astype(np.uint8)
+            P = np.resize(W[:m] if at == 0 else W[max(0, w - m):], m) if w else W
+            P = np.where(rng.random(m) < 0.02, 4, P).astype(np.uint8)
+            reads.append(P)
+            wins.append(W)
+    ro = np.concatenate([[0], np.cumsum([len(x) for x in reads])]).astype(np.uint64)
+    wo = np.concatenate([[0], np.cumsum([len(x) for x in wins])]).astype(np.uint64)
+    r, w = np.concatenate(reads), np.concatenate(wins)
+    for q in (7, 8, 15, 1):
+        want = oracle.qmer_diag_max_batch(r, ro, w, wo, q)
+        got = torch.empty(len(want), dtype=torch.int32, device="cuda")
+        mb.mb_rescue_prefilter(dev(r), dev(ro), dev(w), dev(wo), q=q, best=got)
+        assert np.array_equal(got.cpu().numpy().view(np.uint32), want), q
+        assert np.array_equal(mb.mb_rescue_prefilter(r, ro, w, wo, q=q), want), q
+
+
+def test_decreasing_offsets_are_refused(mb):
+    r, w = np.zeros(300, np.uint8), np.zeros(900, np.uint8)
+    good, bad = np.array([0, 100, 200, 300], np.uint64), np.array([0, 100, 90, 300], np.uint64)
+    wo = np.array([0, 300, 600, 900], np.uint64)
+    for ro, wins in ((bad, wo), (good, np.array([0, 300, 900, 600], np.uint64))):
+        for f in (lambda a: a, dev):
+            with pytest.raises(mb.MbError) as e:
+                mb.mb_rescue_prefilter(f(r), f(ro), f(w), f(wins))
+            assert e.value.code == -1 and b"decrease" in mb.lib().mb_last_error()
