@@ -3,7 +3,7 @@
 // Section 2.4 sampled suffix array, Section 2.5 k-mer ds-interval table).
 //
 //   T = R . revcomp(R) . $            (bisulfite: R -> CT(R) . GA(R), Section 2.9)
-//   S = suffix array of T             prefix doubling: sort by the first 27 symbols, then
+//   S = suffix array of T             prefix doubling: sort by the first 21 symbols, then
 //                                     repeatedly re-sort the suffixes whose 2h-prefix is still
 //                                     shared by (rank of the h-prefix, rank of the h-prefix at +h)
 //   B[i] = T[S(i) - 1], T[-1] = $     written straight into 32-byte occurrence blocks
@@ -62,7 +62,11 @@ u32 mb_index_flags(const mb_index *x) { return x->flags; }
 namespace {
 
 constexpr u64 GOLDEN = 0x9E3779B97F4A7C15ULL;
-constexpr int KEY_SYMS = 27;   // 5^27 < 2^63: the first 27 symbols of a suffix in base 5 ($ = 0)
+// Sort key of a suffix: its first 21 symbols, two bits each, the first highest, $ and what follows it as
+// A; then in 5 bits how many of them come before $ (21 at most), which puts a suffix that ends early
+// before those that go on with A's, as $ < A asks.  47 bits: six passes of the sort (27 symbols in base 5
+// took eight); random texts of 2^32 symbols leave a thousandth of their suffixes tied.
+constexpr int KEY_SYMS = 21, KEY_REM_BITS = 5, KEY_BITS = 2 * KEY_SYMS + KEY_REM_BITS;
 
 __device__ __forceinline__ u8 ref_base(const u8 *__restrict__ R, u64 x, u64 seed) {
     u8 b = R[x];
@@ -90,16 +94,19 @@ __global__ void k_pack_text(const u8 *__restrict__ R, u64 m, u64 seed, int bs3, 
     }
 }
 
-__global__ void k_init_keys(const u8 *__restrict__ T, u64 n, u64 *__restrict__ keys, u32 *__restrict__ vals) {
+// Sixteen symbols of the packed text with the first one in the high bits.
+__device__ __forceinline__ u32 high_first(u32 w) {
+    w = __brev(w);
+    return ((w >> 1) & 0x55555555u) | ((w & 0x55555555u) << 1);
+}
+__global__ void k_init_keys(const u32 *__restrict__ t2, u64 words, u64 n, u64 *__restrict__ keys, u32 *__restrict__ vals) {
     for (u64 i = blockIdx.x * (u64)blockDim.x + threadIdx.x; i < n; i += (u64)gridDim.x * blockDim.x) {
-        u64 v = 0;
-#pragma unroll
-        for (int q = 0; q < KEY_SYMS; ++q) {
-            u64 p = i + q;
-            u32 s = p < n - 1 ? (u32)T[p] + 1u : 0u;
-            v = v * 5 + s;
-        }
-        keys[i] = v;
+        const u64 w = i >> 4;
+        const u32 a = high_first(t2[w]), b = high_first(t2[w + 1]), c = w + 2 < words ? high_first(t2[w + 2]) : 0u;
+        const u32 sh = 2 * (u32)(i & 15);
+        const u64 v = ((u64)__funnelshift_l(b, a, sh) << 32) | __funnelshift_l(c, b, sh);
+        const u64 rem = n - 1 - i;
+        keys[i] = ((v >> (64 - 2 * KEY_SYMS)) << KEY_REM_BITS) | (rem < KEY_SYMS ? rem : KEY_SYMS);
         vals[i] = (u32)i;
     }
 }
@@ -150,7 +157,9 @@ __global__ void k_scatter_sa(const u32 *__restrict__ act, u64 A, const u32 *__re
 
 // One warp per 128 rows, i.e. two 64-row blocks: symbols B[x] = T[S(x)-1] packed 2 bits each
 // ($ stored as A), per-block counts of A,C,G,T (excluding $) to bcnt[a * nblocks + b].
-__global__ void k_bwt_blocks(const u8 *__restrict__ T, const u32 *__restrict__ SA, u64 n, OccBlock *__restrict__ occ,
+// The symbols come from the packed text, a quarter of T, which stays in L2 up to some 200 Mbp (2.6 -> 0.8
+// ms at 100 Mbp).
+__global__ void k_bwt_blocks(const u32 *__restrict__ t2, const u32 *__restrict__ SA, u64 n, OccBlock *__restrict__ occ,
                              u64 nblocks, u64 *__restrict__ bcnt, u64 *__restrict__ primary) {
     const int lane = threadIdx.x & 31;
     const u64 warps = (u64)gridDim.x * (blockDim.x >> 5);
@@ -167,7 +176,7 @@ __global__ void k_bwt_blocks(const u8 *__restrict__ T, const u32 *__restrict__ S
                     *primary = x;
                     s = 0;
                 } else {
-                    s = T[p - 1];
+                    s = (__ldg(t2 + ((p - 1) >> 4)) >> (2 * ((p - 1) & 15))) & 3u;
                     c[s] += 1;
                 }
                 lob |= (s & 1u) << j;
@@ -221,12 +230,11 @@ __global__ void k_text2(const u8 *__restrict__ T, u64 n, u32 *__restrict__ t2, u
     }
 }
 
-// isa[p / r] = the row of the suffix at text position p, for p a multiple of r
-__global__ void k_sample_isa(const u32 *__restrict__ SA, u64 n, u32 r, u32 *__restrict__ isa) {
-    for (u64 i = blockIdx.x * (u64)blockDim.x + threadIdx.x; i < n; i += (u64)gridDim.x * blockDim.x) {
-        const u32 p = SA[i];
-        if (p % r == 0) isa[p / r] = (u32)i;
-    }
+// isa[x] = the row of the suffix at text position x * r (rank: the row of every suffix)
+__global__ void k_sample_isa(const u32 *__restrict__ rank, u64 n, u32 r, u32 *__restrict__ isa) {
+    const u64 m = (n + r - 1) / r;
+    for (u64 x = blockIdx.x * (u64)blockDim.x + threadIdx.x; x < m; x += (u64)gridDim.x * blockDim.x)
+        isa[x] = rank[x * r];
 }
 
 // ds-interval of every k-mer by k BackwardExt steps from the empty string (0, 0, n).  The
@@ -467,49 +475,49 @@ static int make_sa_ref(mb_index *x) {
     return cudaMemcpy(x->sa_ref, &x->sa, sizeof(u32 *), cudaMemcpyHostToDevice) == cudaSuccess ? MB_OK : MB_ERR_CUDA;
 }
 
-// Suffix array of T (device, n symbols) by prefix doubling.  SA (device, n) receives it.
-static int build_sa(const u8 *T, u64 n, u32 *SA, cudaStream_t st) {
-    // 25 bytes per suffix: keys and the sort's spare keys (8 + 8), values and spare values (4 + 4),
-    // ranks (4), two active lists (4 + 4); the run heads and flags (4 + 4) live in the spare keys,
-    // which are free whenever they are used.
-    DevBuf bk, bka, bv, bva, btmp, brank, bact, bact2, berr, bcount;
+// Suffix array of the packed text t2 (device, n symbols with $) by prefix doubling.  SA and rank (device,
+// n each) receive it and its inverse.
+static int build_sa(const u32 *t2, u64 t2words, u64 n, u32 *SA, u32 *rank, cudaStream_t st) {
+    // 20 bytes per suffix: keys and the sort's spare keys (8 + 8) and spare values (4; SA holds the
+    // values); the run heads and flags (4 + 4) live in the spare keys, which are free whenever they are
+    // used.  The rounds add 12 bytes per suffix still active (two active lists, values).
+    DevBuf bk, bka, bva, btmp, bact, bact2, bv, berr, bcount;
     MB_TRY(bk.alloc(n * 8, st));
     MB_TRY(bka.alloc(n * 8, st));
-    MB_TRY(bv.alloc(n * 4, st));
     MB_TRY(bva.alloc(n * 4, st));
     size_t tb = radix_tmp_bytes(n);
     size_t sb = scan_tmp_bytes(n);
     MB_TRY(btmp.alloc(tb > sb ? tb : sb, st));
-    MB_TRY(brank.alloc(n * 4, st));
-    MB_TRY(bact.alloc(n * 4, st));
-    MB_TRY(bact2.alloc(n * 4, st));
     MB_TRY(berr.alloc(8, st));
     MB_TRY(bcount.alloc(8, st));
     u64 *keys = bk.as<u64>(), *keys_alt = bka.as<u64>();
-    u32 *vals = bv.as<u32>(), *vals_alt = bva.as<u32>();
-    u32 *rank = brank.as<u32>(), *hv = bka.as<u32>(), *flag = bka.as<u32>() + n;
-    u32 *act = bact.as<u32>(), *act2 = bact2.as<u32>();
+    u32 *vals_alt = bva.as<u32>();
+    u32 *hv = bka.as<u32>(), *flag = bka.as<u32>() + n;
     u32 *err = berr.as<u32>(), *count = bcount.as<u32>();
     MB_CK(cudaMemsetAsync(err, 0, 4, st));
     const unsigned B = 256;
 
-    // round 0: the first 27 symbols
-    k_init_keys<<<grid_for(n, B), B, 0, st>>>(T, n, keys, vals);
+    // round 0: the first 21 symbols
+    k_init_keys<<<grid_for(n, B), B, 0, st>>>(t2, t2words, n, keys, SA);
     MB_KCHECK();
-    BitRange r0[1] = {{0, 63}};
-    MB_TRY(radix_sort_pairs(keys, vals, keys_alt, vals_alt, n, r0, 1, btmp.p, st));
-    MB_CK(cudaMemcpyAsync(SA, vals, n * 4, cudaMemcpyDeviceToDevice, st));
+    BitRange r0[1] = {{0, KEY_BITS}};
+    MB_TRY(radix_sort_pairs(keys, SA, keys_alt, vals_alt, n, r0, 1, btmp.p, st));
     k_heads<<<grid_for(n, B), B, 0, st>>>(keys, nullptr, n, hv, flag);
     MB_KCHECK();
     MB_TRY(scan_inclusive_max_u32(hv, hv, n, btmp.p, st));
-    k_set_rank<<<grid_for(n, B), B, 0, st>>>(vals, hv, n, rank);
+    k_set_rank<<<grid_for(n, B), B, 0, st>>>(SA, hv, n, rank);
     MB_KCHECK();
     MB_TRY(scan_exclusive_u32(flag, hv, n, count, btmp.p, st));   // hv reused as positions
-    k_compact<<<grid_for(n, B), B, 0, st>>>(flag, hv, nullptr, n, act);
-    MB_KCHECK();
     u32 A = 0;
     MB_CK(cudaMemcpyAsync(&A, count, 4, cudaMemcpyDeviceToHost, st));
     MB_CK(cudaStreamSynchronize(st));
+    if (A == 0) return MB_OK;
+    MB_TRY(bact.alloc((size_t)A * 4, st));
+    MB_TRY(bact2.alloc((size_t)A * 4, st));
+    MB_TRY(bv.alloc((size_t)A * 4, st));
+    u32 *act = bact.as<u32>(), *act2 = bact2.as<u32>(), *vals = bv.as<u32>();
+    k_compact<<<grid_for(n, B), B, 0, st>>>(flag, hv, nullptr, n, act);
+    MB_KCHECK();
 
     const int nb = nbits(n);
     BitRange rr[2] = {{0, nb}, {32, 32 + nb}};
@@ -579,15 +587,29 @@ extern "C" int mb_index_build(const uint8_t *ref, uint64_t len, const mb_opts *o
     cudaGetDevice(&X->device);
     int rc = MB_OK;
     do {
-        DevBuf bref, bT, bcnt, btmp, bprim, btot;
+        DevBuf bref, bT, bcnt, btmp, bprim, btot, brank, bt2;
         const void *dref = nullptr;
         if ((rc = mb_stage_in(ref, len, st, bref, &dref)) != MB_OK) break;
         if ((rc = bT.alloc(n, st)) != MB_OK) break;
         k_pack_text<<<grid_for(n, 256), 256, 0, st>>>((const u8 *)dref, len, n_seed, bs3, bT.as<u8>(), n);
         if (cudaGetLastError() != cudaSuccess) { rc = MB_ERR_CUDA; break; }
         bref.release();
+        // the text packed (kept with the auxiliary arrays), its suffix array and ranks
+        const u64 tw = text2_words(n);
+        u32 *t2 = nullptr;
+        if (flags & MB_NO_AUX) {
+            if ((rc = bt2.alloc(tw * 4, st)) != MB_OK) break;
+            t2 = bt2.as<u32>();
+        } else {
+            if (cudaMalloc(&X->text2, tw * 4) != cudaSuccess) { rc = MB_ERR_NOMEM; break; }
+            t2 = X->text2;
+        }
+        k_text2<<<grid_for(tw, 256), 256, 0, st>>>(bT.as<u8>(), n, t2, tw);
+        if (cudaGetLastError() != cudaSuccess) { rc = MB_ERR_CUDA; break; }
+        bT.release();
         if (cudaMalloc(&X->sa, n * 4) != cudaSuccess) { rc = MB_ERR_NOMEM; break; }
-        if ((rc = build_sa(bT.as<u8>(), n, X->sa, st)) != MB_OK) break;
+        if ((rc = brank.alloc(n * 4, st)) != MB_OK) break;
+        if ((rc = build_sa(t2, tw, n, X->sa, brank.as<u32>(), st)) != MB_OK) break;
 
         // BWT in occurrence blocks
         X->nblocks = n / BLK_ROWS + 1;
@@ -598,7 +620,7 @@ extern "C" int mb_index_build(const uint8_t *ref, uint64_t len, const mb_opts *o
         if ((rc = btmp.alloc(scan_tmp_bytes(nbk), st)) != MB_OK) break;
         if ((rc = bprim.alloc(8, st)) != MB_OK) break;
         if ((rc = btot.alloc(4 * 8, st)) != MB_OK) break;
-        k_bwt_blocks<<<grid_for((nbk + 1) / 2 * 32, 256), 256, 0, st>>>(bT.as<u8>(), X->sa, n, X->occ, nbk, bcnt.as<u64>(),
+        k_bwt_blocks<<<grid_for((nbk + 1) / 2 * 32, 256), 256, 0, st>>>(t2, X->sa, n, X->occ, nbk, bcnt.as<u64>(),
                                                               bprim.as<u64>());
         if (cudaGetLastError() != cudaSuccess) { rc = MB_ERR_CUDA; break; }
         for (int a = 0; a < 4 && rc == MB_OK; ++a)
@@ -626,13 +648,14 @@ extern "C" int mb_index_build(const uint8_t *ref, uint64_t len, const mb_opts *o
         k_kmer_table<<<grid_for(nk, 256), 256, 0, st>>>(mb_dev_index(X), kk, X->kmer);
         if (cudaGetLastError() != cudaSuccess) { rc = MB_ERR_CUDA; break; }
         if (!(flags & MB_NO_AUX)) {
-            // packed text and dense SA / ISA samples for extending unique matches by comparison
-            const u64 tw = text2_words(n), na = aux_count(n);
-            if (cudaMalloc(&X->text2, tw * 4) != cudaSuccess || cudaMalloc(&X->sa_aux, na * 4) != cudaSuccess ||
-                cudaMalloc(&X->isa_aux, na * 4) != cudaSuccess) { rc = MB_ERR_NOMEM; break; }
-            k_text2<<<grid_for(tw, 256), 256, 0, st>>>(bT.as<u8>(), n, X->text2, tw);
+            // dense SA / ISA samples for extending unique matches by comparison
+            const u64 na = aux_count(n);
+            if (cudaMalloc(&X->sa_aux, na * 4) != cudaSuccess || cudaMalloc(&X->isa_aux, na * 4) != cudaSuccess) {
+                rc = MB_ERR_NOMEM;
+                break;
+            }
             k_sample_sa<<<grid_for(na, 256), 256, 0, st>>>(X->sa, n, AUX_RATE, X->sa_aux);
-            k_sample_isa<<<grid_for(n, 256), 256, 0, st>>>(X->sa, n, AUX_RATE, X->isa_aux);
+            k_sample_isa<<<grid_for(na, 256), 256, 0, st>>>(brank.as<u32>(), n, AUX_RATE, X->isa_aux);
             if (cudaGetLastError() != cudaSuccess) { rc = MB_ERR_CUDA; break; }
         }
         if (cudaStreamSynchronize(st) != cudaSuccess) { rc = MB_ERR_CUDA; break; }
