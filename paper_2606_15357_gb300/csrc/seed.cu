@@ -3211,13 +3211,13 @@ __global__ void k_win_build(const mb_smem *__restrict__ sm, u64 nsm, const u64 *
         wmate[w] = mate ? mate[x.read] : 0;
     }
 }
-// Bases of every window, one warp per window, four at a time: each aligned word of the copy from the two
-// aligned words of the read that hold its bytes (byte by byte it took 0.23 ms for 1M windows).
+// Bases of every window, eight lanes per window, four bases at a time: each aligned word of the copy from
+// the two aligned words of the read that hold its bytes.
 __global__ void k_win_copy(const u8 *__restrict__ seq, const u64 *__restrict__ off, const uint2 *__restrict__ winfo,
                            const u64 *__restrict__ woff, u64 nw, u8 *__restrict__ wseq) {
-    const u32 lane = threadIdx.x & 31;
-    const u64 nwarps = ((u64)gridDim.x * blockDim.x) >> 5;
-    for (u64 w = (blockIdx.x * (u64)blockDim.x + threadIdx.x) >> 5; w < nw; w += nwarps) {
+    const u32 lane = threadIdx.x & 7;
+    const u64 nteams = ((u64)gridDim.x * blockDim.x) >> 3;
+    for (u64 w = (blockIdx.x * (u64)blockDim.x + threadIdx.x) >> 3; w < nw; w += nteams) {
         const u64 b = woff[w];
         const u32 len = (u32)(woff[w + 1] - b);
         const u8 *src = seq + off[winfo[w].x] + winfo[w].y;
@@ -3227,11 +3227,12 @@ __global__ void k_win_copy(const u8 *__restrict__ seq, const u64 *__restrict__ o
         const u32 words = (len - head) / 4, sh = 8 * (u32)((uintptr_t)(src + head) & 3);
         const u32 *s4 = reinterpret_cast<const u32 *>((uintptr_t)(src + head) & ~(uintptr_t)3);
         u32 *const d4 = reinterpret_cast<u32 *>(dst + head);
-        for (u32 q = lane; q < words; q += 32) {
+#pragma unroll 4
+        for (u32 q = lane; q < words; q += 8) {
             const u32 lo = __ldg(s4 + q);
             d4[q] = sh ? __funnelshift_r(lo, __ldg(s4 + q + 1), sh) : lo;
         }
-        const u32 rest = len - 4 * words;   // the bytes before and after the words
+        const u32 rest = len - 4 * words;   // the bytes before and after the words (six at most)
         if (lane < rest) {
             const u32 t = lane < head ? lane : lane + 4 * words;
             dst[t] = src[t];
@@ -3296,7 +3297,7 @@ extern "C" int mb_reseed(const mb_index *idx, const uint8_t *seq, const uint64_t
     MB_CK(cudaMemcpyAsync(&wbases, bwoff.as<u64>() + nw, 8, cudaMemcpyDeviceToHost, st));
     MB_CK(cudaStreamSynchronize(st));
     MB_TRY(bwseq.alloc(wbases + 16, st));
-    k_win_copy<<<grid_for(nw * 32, 256), 256, 0, st>>>((const u8 *)dseq, (const u64 *)doff, binfo.as<uint2>(),
+    k_win_copy<<<grid_for(nw * 8, 256), 256, 0, st>>>((const u8 *)dseq, (const u64 *)doff, binfo.as<uint2>(),
                                                        bwoff.as<u64>(), nw, bwseq.as<u8>());
     MB_KCHECK();
     // the seeding pipeline on the windows, each with its own (l', c'); window bases are copied
