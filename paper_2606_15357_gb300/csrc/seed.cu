@@ -1288,19 +1288,6 @@ __global__ void k_set_hitoff(const u64 *__restrict__ hoff, u64 m, const u64 *__r
 }
 
 // ---------------------------------------------------------------------------- locate
-// Largest record index m with hit_off <= h (records with no hits share the offset of the next
-// record that has hits, so the last such record is the one owning hit h).
-__device__ __forceinline__ u64 owner_of(const mb_smem *__restrict__ sm, u64 nsm, u64 h) {
-    u64 a = 0, b = nsm;   // invariant: hit_off[a] <= h, answer in [a, b)
-    while (b - a > 1) {
-        u64 mid = (a + b) >> 1;
-        if (__ldg(&sm[mid].hit_off) <= h) a = mid;
-        else b = mid;
-    }
-    return a;
-}
-
-
 // ---------------------------------------------------------------------------- shared walks
 // The records of a batch repeat rows: reads that cover the same repeat give the same or nested SA
 // intervals (two strings' intervals are nested when one is a prefix of the other, else
@@ -2006,20 +1993,6 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-__global__ void k_bs_filter(const mb_smem *__restrict__ sm, u64 nsm, const u8 *__restrict__ mate,
-                            const u32 *__restrict__ hits, u64 nhits, u64 M, u8 *__restrict__ keep) {
-    for (u64 h = blockIdx.x * (u64)blockDim.x + threadIdx.x; h < nhits; h += (u64)gridDim.x * blockDim.x) {
-        u64 m = owner_of(sm, nsm, h);
-        u64 len = sm[m].qend - sm[m].qbeg;
-        u8 mt = mate ? mate[sm[m].read] : 0;
-        u64 pos = hits[h];
-        u64 seg = pos / M;
-        bool whole = (pos + len - 1) / M == seg;
-        bool ok = mt == 1 ? (seg == 0 || seg == 2) : mt == 2 ? (seg == 1 || seg == 3) : true;
-        keep[h] = (whole && ok) ? 1 : 0;
-    }
-}
-
 void opts_defaults(const mb_opts *o, u32 &l, u32 &c, u32 &max_occ, u32 &flags) {
     l = o && o->min_len ? o->min_len : 19;
     c = o && o->min_occ ? o->min_occ : 1;
@@ -2594,39 +2567,6 @@ extern "C" int mb_locate(const mb_index *idx, const mb_smem *smem, uint64_t n_sm
                      (err & DEVCHK_RECORD) ? "a record's rows [k, k+s) leave the text" : "a row outside the text");
         return MB_ERR_DEVICE_CHECK;
     }
-    return MB_OK;
-}
-
-extern "C" int mb_bs_filter(const mb_index *idx, const mb_smem *smem, uint64_t n_smem, const uint8_t *mate,
-                            const uint32_t *hits, uint64_t n_hits, void *stream, uint8_t *keep) {
-    if (!idx || (n_hits && (!smem || !hits || !keep))) return MB_ERR_ARG;
-    if (n_hits == 0) return MB_OK;
-    cudaStream_t st = (cudaStream_t)stream;
-    DevBuf bsm, bmate, bhits, bkeep;
-    const void *dsm = nullptr, *dmate = nullptr, *dhits = nullptr;
-    MB_TRY(mb_stage_in(smem, n_smem * sizeof(mb_smem), st, bsm, &dsm));
-    if (mate) {
-        mb_smem last;
-        MB_CK(cudaMemcpyAsync(&last, (const mb_smem *)dsm + n_smem - 1, sizeof last, cudaMemcpyDeviceToHost, st));
-        MB_CK(cudaStreamSynchronize(st));
-        MB_TRY(mb_stage_in(mate, (size_t)last.read + 1, st, bmate, &dmate));
-    }
-    MB_TRY(mb_stage_in(hits, n_hits * 4, st, bhits, &dhits));
-    u8 *dk = keep;
-    const bool kdev = mb_is_device_ptr(keep);
-    if (!kdev) {
-        MB_TRY(bkeep.alloc(n_hits, st));
-        dk = bkeep.as<u8>();
-    }
-    u64 M = 0, n = 0, prim = 0;
-    mb_index_info(idx, &n, &prim, &M);
-    // the 3-base index holds four copies of |R| = M/2 bases
-    u64 quarter = M / 2;
-    k_bs_filter<<<grid_for(n_hits, 256), 256, 0, st>>>((const mb_smem *)dsm, n_smem, (const u8 *)dmate,
-                                                       (const u32 *)dhits, n_hits, quarter, dk);
-    MB_KCHECK();
-    if (!kdev) MB_CK(cudaMemcpyAsync(keep, dk, n_hits, cudaMemcpyDeviceToHost, st));
-    MB_CK(cudaStreamSynchronize(st));
     return MB_OK;
 }
 
