@@ -89,11 +89,11 @@ __global__ void k_scan_apply(const T *in, T *out, size_t n, const T *__restrict_
 size_t level_blocks(size_t n) { return (n + SCAN_TILE - 1) / SCAN_TILE; }
 
 template <class T, class Op, bool INCL>
-int scan_impl(const T *in, T *out, size_t n, void *tmp, cudaStream_t st, Op op) {
+int scan_impl(const T *in, T *out, size_t n, T *total, void *tmp, cudaStream_t st, Op op) {
     if (n == 0) return MB_OK;
     size_t nb = level_blocks(n);
     if (nb == 1) {
-        k_scan_apply<T, Op, INCL><<<1, SCAN_T, 0, st>>>(in, out, n, nullptr, nullptr, op);
+        k_scan_apply<T, Op, INCL><<<1, SCAN_T, 0, st>>>(in, out, n, nullptr, total, op);
         MB_KCHECK();
         return MB_OK;
     }
@@ -102,35 +102,20 @@ int scan_impl(const T *in, T *out, size_t n, void *tmp, cudaStream_t st, Op op) 
     k_scan_reduce<T, Op><<<(unsigned)nb, SCAN_T, 0, st>>>(in, n, part, op);
     MB_KCHECK();
     // exclusive scan of the tile sums gives each tile's carry
-    MB_TRY((scan_impl<T, Op, false>(part, part, nb, rest, st, op)));
-    k_scan_apply<T, Op, INCL><<<(unsigned)nb, SCAN_T, 0, st>>>(in, out, n, part, nullptr, op);
+    MB_TRY((scan_impl<T, Op, false>(part, part, nb, nullptr, rest, st, op)));
+    k_scan_apply<T, Op, INCL><<<(unsigned)nb, SCAN_T, 0, st>>>(in, out, n, part, total, op);
     MB_KCHECK();
     return MB_OK;
 }
 
-template <class T>
-__global__ void k_copy_one(const T *src, T *dst) { *dst = *src; }
-template <class T>
-__global__ void k_add_one(const T *src, T *dst) { *dst += *src; }
-
-// exclusive sum; total = last input + last output (the last input is saved first so that the
-// scan may run in place)
+// exclusive sum; total: of all inputs (written by the last tile)
 template <class T>
 int scan_excl_total(const T *in, T *out, size_t n, T *total, void *tmp, cudaStream_t st) {
     if (n == 0) {
         if (total) MB_CK(cudaMemsetAsync(total, 0, sizeof(T), st));
         return MB_OK;
     }
-    if (total) {
-        k_copy_one<T><<<1, 1, 0, st>>>(in + n - 1, total);
-        MB_KCHECK();
-    }
-    MB_TRY((scan_impl<T, OpSum, false>(in, out, n, tmp, st, OpSum())));
-    if (total) {
-        k_add_one<T><<<1, 1, 0, st>>>(out + n - 1, total);
-        MB_KCHECK();
-    }
-    return MB_OK;
+    return scan_impl<T, OpSum, false>(in, out, n, total, tmp, st, OpSum());
 }
 
 }  // namespace
@@ -154,7 +139,7 @@ int scan_exclusive_u32(const u32 *in, u32 *out, size_t n, u32 *total, void *tmp,
 }
 
 int scan_inclusive_max_u32(const u32 *in, u32 *out, size_t n, void *tmp, cudaStream_t st) {
-    return scan_impl<u32, OpMax, true>(in, out, n, tmp, st, OpMax());
+    return scan_impl<u32, OpMax, true>(in, out, n, nullptr, tmp, st, OpMax());
 }
 
 // ============================================================================ radix sort

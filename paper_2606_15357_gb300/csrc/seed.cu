@@ -2247,7 +2247,7 @@ int locate_shared(const DevIndex &I, const mb_smem *sm, u64 cap, const u64 *nsm_
     return MB_OK;
 }
 
-// The hits of records sm[0, min(cap, *nsm_dev)) by k_locate_direct.
+// The hits of records sm[0, min(cap, *nsm_dev)) by k_locate_direct (*D.n and *err zero before).
 int locate_direct(const DevIndex &I, const mb_smem *sm, u64 cap, const u64 *nsm_dev, const u32 *known, u32 *hits,
                   u64 hits_cap, const DirectBufs &D, u32 *err, cudaStream_t st) {
     if (cap == 0) return MB_OK;
@@ -2256,7 +2256,6 @@ int locate_direct(const DevIndex &I, const mb_smem *sm, u64 cap, const u64 *nsm_
         L.ssa = I.sa_aux;
         L.r = AUX_RATE;
     }
-    MB_CK(cudaMemsetAsync(D.n, 0, 4, st));
     const unsigned g = resident_grid((const void *)k_locate_direct<false>, 256, cap);
     k_locate_direct<false><<<g, 256, 0, st>>>(L, sm, cap, nsm_dev, known, hits, hits_cap, D, err);
     MB_KCHECK();
@@ -2289,15 +2288,20 @@ bool locate_joins(const DevIndex &I, u32 flags) {
 }
 
 // The SMEM kernel in the requested shape: work counters, work queue, threads per block.
-int launch_smem(const SmemArgs &a, bool count, bool queue, int block, cudaStream_t st) {
+// With `items` the items of cut reads too (launch_items), which a caller may also do later.
+constexpr u32 LATE_ITEMS = 65536;   // mb_seed_device: reads up to which it does
+int launch_items(const SmemArgs &a, cudaStream_t st) {
+    if (!a.sp.items_cap) return MB_OK;
+    MB_TRY(launch_slots<true>(a, 256, st));
+    k_split_sum<<<32, 128, 0, st>>>(a.sp, a.counts, a.ovf_list, a.ovf_n);
+    MB_KCHECK();
+    return MB_OK;
+}
+int launch_smem(const SmemArgs &a, bool count, bool queue, int block, bool items, cudaStream_t st) {
     if (count) return launch_smem_t<true, false, 256>(a, st);
     if (!a.one_loop) {
         MB_TRY(launch_slots<false>(a, block, st));
-        if (!a.sp.items_cap) return MB_OK;
-        MB_TRY(launch_slots<true>(a, 256, st));
-        k_split_sum<<<32, 128, 0, st>>>(a.sp, a.counts, a.ovf_list, a.ovf_n);
-        MB_KCHECK();
-        return MB_OK;
+        return items ? launch_items(a, st) : MB_OK;
     }
     if (queue) {
         if (block == 128) return launch_smem_t<false, true, 128>(a, st);
@@ -2324,48 +2328,56 @@ int mb_seed_device(const mb_index *idx, const u8 *dseq, const u64 *doff, u32 n_r
     if (n_hits) *n_hits = 0;
     if (n_reads == 0) return MB_OK;
     const u64 nslots = slots_total(o1 - o0, n_reads);
-    DevBuf bslots, bcounts, bsoff, bovf, bmisc, btmp, bsplit;
     const SplitRoom room(o1 - o0, n_reads);
-    MB_TRY(bsplit.alloc(room.bytes(), st));
-    MB_TRY(bslots.alloc(nslots * sizeof(SlotRec), st));
-    MB_TRY(bcounts.alloc((size_t)n_reads * 8, st));
-    MB_TRY(bsoff.alloc((size_t)n_reads * 8, st));
-    MB_TRY(bovf.alloc((size_t)n_reads * 4, st));
-    MB_TRY(bmisc.alloc(128, st));
-    u64 *dtotal = bmisc.as<u64>(), *dhtotal = bmisc.as<u64>() + 1;
-    u32 *dovf_n = (u32 *)(bmisc.as<u64>() + 2), *dqhead = (u32 *)(bmisc.as<u64>() + 3);
-    u32 *derr = (u32 *)(bmisc.as<u64>() + 4);
-    MB_CK(cudaMemsetAsync(bmisc.p, 0, 128, st));
-    const SplitBufs split = room.bufs(bsplit.p, (u32 *)(bmisc.as<u64>() + 8));
+    // one allocation: counters, per-read counts and record offsets, overflow list, scan scratch, slots,
+    // and the room for cut reads and the pool
+    const size_t z[7] = {128, (size_t)n_reads * 8, (size_t)n_reads * 8, (size_t)n_reads * 4, scan_tmp_bytes(n_reads),
+                         nslots * sizeof(SlotRec), room.bytes()};
+    size_t at[7], bytes = 0;
+    for (int i = 0; i < 7; ++i) {
+        at[i] = bytes;
+        bytes += align_up(z[i]);
+    }
+    DevBuf bw;
+    MB_TRY(bw.alloc(bytes, st));
+    char *const w = (char *)bw.p;
+    u64 *misc = (u64 *)w, *counts = (u64 *)(w + at[1]), *soff = (u64 *)(w + at[2]);
+    u64 *dtotal = misc, *dhtotal = misc + 1;
+    u32 *ovf = (u32 *)(w + at[3]), *dovf_n = (u32 *)(misc + 2), *dqhead = (u32 *)(misc + 3), *derr = (u32 *)(misc + 4);
+    SlotRec *slots = (SlotRec *)(w + at[5]);
+    MB_CK(cudaMemsetAsync(misc, 0, 128, st));
+    const SplitBufs split = room.bufs(w + at[6], (u32 *)(misc + 8));
 
     const DevIndex I = mb_dev_index(idx);
     const unsigned B = 256;
     const unsigned G = (unsigned)((n_reads + B - 1) / B);
     KTimer kt("smem", st);   // reported after the stream is synchronized below
-    const bool kmer = !(flags & MB_NO_KMER) && l >= mb_dev_index(idx).kmer_k;
+    const bool kmer = !(flags & MB_NO_KMER) && l >= I.kmer_k;
+    const bool count = (flags & MB_COUNT) != 0;
+    SmemArgs sa{I, dseq, doff, n_reads, dmate, bs, l, c, kmer, slots, nslots, counts, ovf, dovf_n, dqhead,
+                count ? mb_work_counter_buf(st) : nullptr, dlc, I.text2 && !(flags & MB_STEP_ONLY)};
+    smem_tuning(opts, sa);
+    sa.sp = split;
+    sa.err = derr;
+    sa.chk = (flags & MB_CHECKED) ? derr : nullptr;
+    // a small batch learns first whether any read was cut: most have none, and two launches less
+    const bool later = n_reads <= LATE_ITEMS && !count && !sa.one_loop;
     {
-        const bool count = (flags & MB_COUNT) != 0;
-        const bool queue = !count && (flags & MB_BATCHED);
-        SmemArgs sa{I, (const u8 *)dseq, (const u64 *)doff, n_reads, (const u8 *)dmate, bs, l, c, kmer,
-                    bslots.as<SlotRec>(), nslots, bcounts.as<u64>(), bovf.as<u32>(), dovf_n,
-                    dqhead, count ? mb_work_counter_buf(st) : nullptr, dlc,
-                    I.text2 && !(flags & MB_STEP_ONLY)};
-        smem_tuning(opts, sa);
-        sa.sp = split;
-        sa.err = derr;
-        sa.chk = (flags & MB_CHECKED) ? derr : nullptr;
         const int blk = opts && (opts->block_size == 128 || opts->block_size == 512) ? (int)opts->block_size : 256;
         kt.start();
-        MB_TRY(launch_smem(sa, count, queue, blk, st));
+        MB_TRY(launch_smem(sa, count, !count && (flags & MB_BATCHED), blk, !later, st));
         kt.stop();
     }
-    MB_TRY(btmp.alloc(scan_tmp_bytes(n_reads), st));
-    MB_TRY(scan_exclusive_u64(bcounts.as<u64>(), bsoff.as<u64>(), n_reads, dtotal, btmp.p, st));
-    u64 total = 0;
-    u32 err = 0;
-    MB_CK(cudaMemcpyAsync(&total, dtotal, 8, cudaMemcpyDeviceToHost, st));
-    MB_CK(cudaMemcpyAsync(&err, derr, 4, cudaMemcpyDeviceToHost, st));
-    MB_CK(cudaStreamSynchronize(st));
+    u64 v[10];   // the counters: records, hits, overflow, queue, error word; from 8 on SplitBufs::n
+    for (int pass = 0;; ++pass) {
+        MB_TRY(scan_exclusive_u64(counts, soff, n_reads, dtotal, w + at[4], st));
+        MB_CK(cudaMemcpyAsync(v, misc, sizeof v, cudaMemcpyDeviceToHost, st));
+        MB_CK(cudaStreamSynchronize(st));
+        if (!later || pass || (u32)v[8] == 0) break;
+        MB_TRY(launch_items(sa, st));
+    }
+    const u64 total = v[0];
+    const u32 err = (u32)v[4], over = (u32)v[2], pooled = (u32)v[9];
     if (err) {
         mb_set_error("mb_seed_batch: device check failed (0x%x): %s", err,
                      (err & DEVCHK_OFFSETS) ? "read offsets decrease or leave [off[0], off[n_reads]]"
@@ -2382,32 +2394,54 @@ int mb_seed_device(const mb_index *idx, const u8 *dseq, const u64 *doff, u32 n_r
         return MB_ERR_ARG;
     }
     MB_TRY(mb_check_span(out, total * sizeof(mb_smem), "mb_seed_batch: out"));
-    DevBuf bout, bhitc, bhtmp;
+    DevBuf bout, bhit;
     mb_smem *dout = out;
     if (!out_dev) {
         MB_TRY(bout.alloc(total * sizeof(mb_smem), st));
         dout = bout.as<mb_smem>();
     }
-    MB_TRY(bhitc.alloc(total * 8, st));
-    k_gather<<<G, B, 0, st>>>((const u64 *)doff, n_reads, bslots.as<SlotRec>(), nslots, bcounts.as<u64>(),
-                              bsoff.as<u64>(), max_occ, dout, bhitc.as<u64>(), total);
+    MB_TRY(bhit.alloc(align_up(total * 8) + scan_tmp_bytes(total), st));
+    u64 *hitc = bhit.as<u64>();
+    k_gather<<<G, B, 0, st>>>(doff, n_reads, slots, nslots, counts, soff, max_occ, dout, hitc, total);
     MB_KCHECK();
-    k_pool_write<<<152, 256, 0, st>>>(split, bsoff.as<u64>(), max_occ, dout, bhitc.as<u64>(), total);
-    MB_KCHECK();
-    k_smem_overflow<<<resident_grid((const void *)k_smem_overflow, 128, 1ull << 40), 128, 0, st>>>(I, (const u8 *)dseq, (const u64 *)doff, n_reads, (const u8 *)dmate, bs, l,
-                                         c, kmer,
-                                         bovf.as<u32>(), dovf_n, bsoff.as<u64>(), max_occ, dout, bhitc.as<u64>(),
-                                         total, dlc);
-    MB_KCHECK();
-    MB_TRY(bhtmp.alloc(scan_tmp_bytes(total), st));
-    MB_TRY(scan_exclusive_u64(bhitc.as<u64>(), bhitc.as<u64>(), total, dhtotal, bhtmp.p, st));
-    k_set_hitoff<<<grid_for(total, 256), 256, 0, st>>>(bhitc.as<u64>(), total, nullptr, dout, winfo);
+    if (pooled) {
+        k_pool_write<<<152, 256, 0, st>>>(split, soff, max_occ, dout, hitc, total);
+        MB_KCHECK();
+    }
+    if (over) {
+        k_smem_overflow<<<resident_grid((const void *)k_smem_overflow, 128, 1ull << 40), 128, 0, st>>>(
+            I, dseq, doff, n_reads, dmate, bs, l, c, kmer, ovf, dovf_n, soff, max_occ, dout, hitc, total, dlc);
+        MB_KCHECK();
+    }
+    MB_TRY(scan_exclusive_u64(hitc, hitc, total, dhtotal, (char *)bhit.p + align_up(total * 8), st));
+    k_set_hitoff<<<grid_for(total, 256), 256, 0, st>>>(hitc, total, nullptr, dout, winfo);
     MB_KCHECK();
     u64 ht = 0;
     MB_CK(cudaMemcpyAsync(&ht, dhtotal, 8, cudaMemcpyDeviceToHost, st));
     if (!out_dev) MB_CK(cudaMemcpyAsync(out, dout, total * sizeof(mb_smem), cudaMemcpyDeviceToHost, st));
     MB_CK(cudaStreamSynchronize(st));
     if (n_hits) *n_hits = ht;
+    return MB_OK;
+}
+
+// off[0] and off[n] on the host: read there, or both copied at once.
+static int off_ends(const u64 *off, u64 n, cudaStream_t st, u64 *o0, u64 *o1) {
+    u64 v[2];
+    if (mb_is_device_ptr(off)) {
+        if (n < (1u << 27)) {   // the pitch has to stay below 2 GB
+            MB_CK(cudaMemcpy2DAsync(v, 8, off, n * 8, 8, 2, cudaMemcpyDeviceToHost, st));
+        } else {
+            MB_CK(cudaMemcpyAsync(v, off, 8, cudaMemcpyDeviceToHost, st));
+            MB_CK(cudaMemcpyAsync(v + 1, off + n, 8, cudaMemcpyDeviceToHost, st));
+        }
+        MB_CK(cudaStreamSynchronize(st));
+    } else {
+        MB_CK(cudaStreamSynchronize(st));   // what the stream still writes there
+        v[0] = off[0];
+        v[1] = off[n];
+    }
+    *o0 = v[0];
+    *o1 = v[1];
     return MB_OK;
 }
 
@@ -2428,9 +2462,7 @@ extern "C" int mb_seed_batch(const mb_index *idx, const uint8_t *seq, const uint
     const void *doff = nullptr, *dseq = nullptr, *dmate = nullptr;
     u64 o0 = 0, o1 = 0;
     MB_TRY(mb_check_span(off, (size_t)(n_reads + 1) * 8, "mb_seed_batch: off"));
-    MB_CK(cudaMemcpyAsync(&o0, off, 8, cudaMemcpyDefault, st));
-    MB_CK(cudaMemcpyAsync(&o1, off + n_reads, 8, cudaMemcpyDefault, st));
-    MB_CK(cudaStreamSynchronize(st));
+    MB_TRY(off_ends(off, n_reads, st, &o0, &o1));
     if (o1 < o0) {
         mb_set_error("mb_seed_batch: offsets decrease");
         return MB_ERR_ARG;
@@ -2679,7 +2711,7 @@ extern "C" int mb_seed_batch_noalloc(const mb_index *idx, const uint8_t *seq, co
         smem_tuning(opts, sa);
         sa.err = derr;
         sa.chk = (flags & MB_CHECKED) ? derr : nullptr;
-        MB_TRY(launch_smem(sa, false, false, 256, st));
+        MB_TRY(launch_smem(sa, false, false, 256, true, st));
     }
     MB_TRY(scan_exclusive_u64(counts, soff, nr, dtotal, S + o_tmp, st));
     u64 total = 0;
@@ -2895,7 +2927,7 @@ static int plan_seed(mb_plan *P, const uint8_t *seq, const uint64_t *off, uint32
     sa.per_warp = P->per_warp;
     sa.err = err;
     sa.chk = (P->flags & MB_CHECKED) ? err : nullptr;
-    MB_TRY(launch_smem(sa, false, P->queue, P->block, st));
+    MB_TRY(launch_smem(sa, false, P->queue, P->block, true, st));
     MB_TRY(scan_exclusive_u64(P->counts, P->soff, n_reads, n_smem, P->tmp, st));
     const unsigned G = (unsigned)((n_reads + 255) / 256);
     k_gather<<<G, 256, 0, st>>>(off, n_reads, P->slots, P->nslots, P->counts, P->soff, P->max_occ, P->out, P->hitc,
@@ -3194,9 +3226,7 @@ extern "C" int mb_reseed(const mb_index *idx, const uint8_t *seq, const uint64_t
     DevBuf boff, bseq, bmate, bsm;
     const void *doff = nullptr, *dseq = nullptr, *dmate = nullptr, *dsm = nullptr;
     u64 o0 = 0, o1 = 0;
-    MB_CK(cudaMemcpyAsync(&o0, off, 8, cudaMemcpyDefault, st));
-    MB_CK(cudaMemcpyAsync(&o1, off + n_reads, 8, cudaMemcpyDefault, st));
-    MB_CK(cudaStreamSynchronize(st));
+    MB_TRY(off_ends(off, n_reads, st, &o0, &o1));
     MB_TRY(mb_stage_in(off, (size_t)(n_reads + 1) * 8, st, boff, &doff));
     if (mb_is_device_ptr(seq)) dseq = seq;
     else {
