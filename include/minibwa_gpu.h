@@ -94,7 +94,9 @@ typedef struct {
     uint32_t sa_rate;         /* r, suffix array sample rate (default 32, Section 2.4) */
     uint32_t kmer_k;          /* k of the k-mer ds-interval table (default 10, Section 2.5), <= 16;
                                  the table takes 12 * 4^k bytes (3.2 GB at k = 14, 51.5 GB at
-                                 k = 16) */
+                                 k = 16).  Where 4^(k+1) <= n / 2 the index keeps a deeper table
+                                 beside it for seeding, of 1.5 to 6 bytes per text position, if the
+                                 device has room (built with the index, also on load; not in files) */
     uint32_t flags;           /* MB_* flags above */
     uint32_t chunk_reads;     /* mb_seed_locate: reads per pipelined chunk (0 = 2^22) */
     uint32_t prefetch_depth;  /* tuning: LF-walks in flight per lane in locate, 1/2/4/8/16 (0 = 1) */

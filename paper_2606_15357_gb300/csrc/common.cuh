@@ -134,6 +134,8 @@ struct DevIndex {
     const u32 *sa_aux;  // S(x * AUX_RATE)
     const u32 *isa_aux; // row of the suffix at text position p * AUX_RATE
     const u32 *const *sa_ref;   // device word: the full suffix array, or null once it was dropped
+    const u32 *kmer2;   // a deeper k-mer table for seeding (null: none), of 4^kmer2_k entries
+    u32 kmer2_k;
     bool has_sa;        // the array is there now (it may be dropped later: kernels go by sa_ref)
 };
 // Sample rate of the auxiliary SA / ISA samples used to extend unique matches by comparison.

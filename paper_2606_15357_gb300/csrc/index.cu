@@ -30,6 +30,8 @@ struct mb_index {
     u32 *text2 = nullptr;         // T[0, n-1) at 2 bits per base, 16 per word, first in the low bits
     u32 *sa_aux = nullptr;        // S(x * AUX_RATE)
     u32 *isa_aux = nullptr;       // row of the suffix at text position p * AUX_RATE
+    u32 *kmer2 = nullptr;         // deeper k-mer table (build_kmer2), and its k
+    u32 kmer2_k = 0;
     const u32 **sa_ref = nullptr; // device word holding sa, null once it is dropped: kernels (also those
                                   // of graphs captured before) read it at every launch
     int device = 0;
@@ -53,6 +55,8 @@ DevIndex mb_dev_index(const mb_index *x) {
     I.sa_aux = x->sa_aux;
     I.isa_aux = x->isa_aux;
     I.sa_ref = x->sa_ref;
+    I.kmer2 = x->kmer2;
+    I.kmer2_k = x->kmer2_k;
     I.has_sa = x->sa != nullptr;
     return I;
 }
@@ -251,6 +255,32 @@ __global__ void k_kmer_table(DevIndex I, u32 k, u32 *__restrict__ out) {
         out[3 * w + 0] = p;
         out[3 * w + 1] = q;
         out[3 * w + 2] = s;
+    }
+}
+
+// The table of k + 1 from the one of k: entry 4w + a is a BackwardExt by a of entry w, and the four
+// read the same two blocks.
+__global__ void k_kmer_deeper(DevIndex I, u32 k, const u32 *__restrict__ in, uint4 *__restrict__ out) {
+    const u64 nk = 1ULL << (2 * k);
+    for (u64 w = blockIdx.x * (u64)blockDim.x + threadIdx.x; w < nk; w += (u64)gridDim.x * blockDim.x) {
+        const u32 p = in[3 * w], q = in[3 * w + 1], s = in[3 * w + 2];
+        u32 v[12];
+        if (s) {
+            const Blk b0 = load_blk(I.occ + (p >> BLK_SHIFT)), b1 = load_blk(I.occ + ((p + s) >> BLK_SHIFT));
+#pragma unroll
+            for (u32 a = 0; a < 4; ++a) {
+                const Ext e = extend_blocks(I, b0, b1, p, q, s, a);
+                v[3 * a] = e.p;
+                v[3 * a + 1] = e.q;
+                v[3 * a + 2] = e.s;
+            }
+        } else {   // absent: never read past s
+#pragma unroll
+            for (int t = 0; t < 12; ++t) v[t] = 0;
+        }
+        out[3 * w] = make_uint4(v[0], v[1], v[2], v[3]);
+        out[3 * w + 1] = make_uint4(v[4], v[5], v[6], v[7]);
+        out[3 * w + 2] = make_uint4(v[8], v[9], v[10], v[11]);
     }
 }
 
@@ -466,6 +496,7 @@ static void free_index(mb_index *x) {
     if (x->sa_aux) cudaFree(x->sa_aux);
     if (x->isa_aux) cudaFree(x->isa_aux);
     if (x->sa_ref) cudaFree(x->sa_ref);
+    if (x->kmer2) cudaFree(x->kmer2);
     delete x;
 }
 
@@ -473,6 +504,42 @@ static void free_index(mb_index *x) {
 static int make_sa_ref(mb_index *x) {
     if (cudaMalloc(&x->sa_ref, sizeof(u32 *)) != cudaSuccess) return MB_ERR_NOMEM;
     return cudaMemcpy(x->sa_ref, &x->sa, sizeof(u32 *), cudaMemcpyHostToDevice) == cudaSuccess ? MB_OK : MB_ERR_CUDA;
+}
+
+// Seeding's own k-mer table, as deep as 4^k <= n / 2 (13 at 100 Mbp, 14 at 1 Gbp), where the index's
+// table (k = 10 by default, Section 2.5, sized for a CPU cache) is shallower: every further base is an
+// extension less per lookup, of a wide interval and so of two blocks.  Same SMEMs with any k.  It takes
+// 1.5 to 6 bytes per text position; without room for it seeding uses the index's own.
+static int build_kmer2(mb_index *x, cudaStream_t st) {
+    u32 k = x->kmer_k;
+    while (k < 16 && (1ULL << (2 * k + 2)) <= x->n / 2) ++k;
+    if (k == x->kmer_k) return MB_OK;
+    const DevIndex I = mb_dev_index(x);
+    u32 *t = nullptr;
+    if (cudaMalloc(&t, (12ULL << (2 * k))) != cudaSuccess) {
+        cudaGetLastError();
+        return MB_OK;
+    }
+    // the levels between, each a quarter of the next one, take turns at the two ends of a buffer
+    DevBuf b;
+    const size_t quarter = 12ULL << (2 * (k - 1)), sixteenth = 12ULL << (2 * (k - 2));
+    int rc = k - x->kmer_k > 1 ? b.alloc(quarter + sixteenth, st) : MB_OK;
+    const u32 *in = x->kmer;
+    for (u32 i = x->kmer_k; i < k && rc == MB_OK; ++i) {
+        // level k - 1 goes to the buffer's start, k - 2 behind it, k - 3 to the start, ...
+        u32 *out = i + 1 == k ? t : (u32 *)((char *)b.p + ((k - 1 - (i + 1)) & 1 ? quarter : 0));
+        k_kmer_deeper<<<grid_for(1ULL << (2 * i), 256), 256, 0, st>>>(I, i, in, (uint4 *)out);
+        if (cudaGetLastError() != cudaSuccess) rc = MB_ERR_CUDA;
+        in = out;
+    }
+    if (rc != MB_OK) {
+        cudaStreamSynchronize(st);
+        cudaFree(t);
+        return rc == MB_ERR_NOMEM ? MB_OK : rc;
+    }
+    x->kmer2 = t;
+    x->kmer2_k = k;
+    return MB_OK;
 }
 
 // Suffix array of the packed text t2 (device, n symbols with $) by prefix doubling.  SA and rank (device,
@@ -647,6 +714,7 @@ extern "C" int mb_index_build(const uint8_t *ref, uint64_t len, const mb_opts *o
         if (cudaMalloc(&X->kmer, nk * 12) != cudaSuccess) { rc = MB_ERR_NOMEM; break; }
         k_kmer_table<<<grid_for(nk, 256), 256, 0, st>>>(mb_dev_index(X), kk, X->kmer);
         if (cudaGetLastError() != cudaSuccess) { rc = MB_ERR_CUDA; break; }
+        if ((rc = build_kmer2(X, st)) != MB_OK) break;
         if (!(flags & MB_NO_AUX)) {
             // dense SA / ISA samples for extending unique matches by comparison
             const u64 na = aux_count(n);
@@ -924,6 +992,11 @@ extern "C" int mb_index_load(const char *path, void *stream, mb_index **out) {
         cudaStreamSynchronize(st) != cudaSuccess) {
         free_index(X);
         mb_set_error("mb_index_load: copy to device failed");
+        return MB_ERR_CUDA;
+    }
+    if (build_kmer2(X, st) != MB_OK || cudaStreamSynchronize(st) != cudaSuccess) {
+        free_index(X);
+        mb_set_error("mb_index_load: building the deeper k-mer table failed");
         return MB_ERR_CUDA;
     }
     if (make_sa_ref(X) != MB_OK) {

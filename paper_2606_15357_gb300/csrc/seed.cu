@@ -2027,8 +2027,13 @@ int launch_slots(const SmemArgs &a, int block, cudaStream_t st) {
     const unsigned g = resident_grid(f, block, ITEMS ? 1ull << 40 : (u64)a.nr * 32, smem);
     const u64 each = (a.nr + (u64)g * wpb - 1) / ((u64)g * wpb);
     const u32 most = a.per_warp && a.per_warp < (u32)SLOTS ? a.per_warp : (u32)SLOTS;
+    DevIndex I = a.I;
+    if (I.kmer2 && a.l >= I.kmer2_k) {   // (the windows of the second round ask for at least l)
+        I.kmer = I.kmer2;
+        I.kmer_k = I.kmer2_k;
+    }
     k_smem_slots<ITEMS><<<g, block, smem, st>>>(
-        a.I, a.seq, a.off, a.nr, a.mate, a.bs, a.l, a.c, a.kmer, a.slots, a.slot_total, a.counts, a.ovf_list, a.ovf_n,
+        I, a.seq, a.off, a.nr, a.mate, a.bs, a.l, a.c, a.kmer, a.slots, a.slot_total, a.counts, a.ovf_list, a.ovf_n,
         ITEMS ? a.sp.n + 3 : a.qhead, a.lc, a.uext, each < most ? (u32)each : most, a.err, a.chk, a.sp);
     MB_KCHECK();
     return MB_OK;
