@@ -50,13 +50,51 @@ __device__ __forceinline__ T block_excl(T v, T &total, Op op) {
     return op(warp_pre, ex);
 }
 
+// A thread's SCAN_I items of a full tile in 32-byte accesses (whole sectors; one item at a time, the lanes
+// of a load lie 64 or 128 bytes apart and each sector is asked for several times).
+template <class T>
+__device__ __forceinline__ void load_items(const T *p, T v[SCAN_I]) {
+    constexpr int PER = 32 / sizeof(T);
+#pragma unroll
+    for (int i = 0; i < SCAN_I / PER; ++i) {
+        u64 a, b, c, d;
+        asm volatile("ld.global.v4.u64 {%0,%1,%2,%3}, [%4];" : "=l"(a), "=l"(b), "=l"(c), "=l"(d) : "l"(p + PER * i));
+        const u64 x[4] = {a, b, c, d};
+#pragma unroll
+        for (int j = 0; j < PER; ++j)
+            v[PER * i + j] = sizeof(T) == 8 ? (T)x[j & 3] : (T)(x[(j / 2) & 3] >> (32 * (j & 1)));
+    }
+}
+template <class T>
+__device__ __forceinline__ void store_items(T *p, const T v[SCAN_I]) {
+    constexpr int PER = 32 / sizeof(T);
+#pragma unroll
+    for (int i = 0; i < SCAN_I / PER; ++i) {
+        u64 x[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            x[j] = sizeof(T) == 8 ? (u64)v[PER * i + j]
+                                  : (u64)(u32)v[PER * i + (2 * j) % PER] | ((u64)(u32)v[PER * i + (2 * j + 1) % PER] << 32);
+        asm volatile("st.global.v4.u64 [%0], {%1,%2,%3,%4};" ::"l"(p + PER * i), "l"(x[0]), "l"(x[1]), "l"(x[2]), "l"(x[3])
+                     : "memory");
+    }
+}
+__device__ __forceinline__ bool sectors(const void *p) { return ((uintptr_t)p & 31) == 0; }
+
 template <class T, class Op>
 __global__ void k_scan_reduce(const T *__restrict__ in, size_t n, T *__restrict__ part, Op op) {
     size_t base = blockIdx.x * SCAN_TILE + (size_t)threadIdx.x * SCAN_I;
     T acc = Op::template id<T>();
+    if (base + SCAN_I <= n && sectors(in)) {
+        T v[SCAN_I];
+        load_items(in + base, v);
 #pragma unroll
-    for (int i = 0; i < SCAN_I; ++i)
-        if (base + i < n) acc = op(acc, in[base + i]);
+        for (int i = 0; i < SCAN_I; ++i) acc = op(acc, v[i]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < SCAN_I; ++i)
+            if (base + i < n) acc = op(acc, in[base + i]);
+    }
     T tot;
     block_excl(acc, tot, op);
     if (threadIdx.x == 0) part[blockIdx.x] = tot;
@@ -68,20 +106,31 @@ __global__ void k_scan_apply(const T *in, T *out, size_t n, const T *__restrict_
     size_t base = blockIdx.x * SCAN_TILE + (size_t)threadIdx.x * SCAN_I;
     T v[SCAN_I];
     T acc = Op::template id<T>();
+    const bool full = base + SCAN_I <= n;
+    if (full && sectors(in)) {
+        load_items(in + base, v);
+    } else {
 #pragma unroll
-    for (int i = 0; i < SCAN_I; ++i) {
-        v[i] = base + i < n ? in[base + i] : Op::template id<T>();
-        acc = op(acc, v[i]);
+        for (int i = 0; i < SCAN_I; ++i) v[i] = base + i < n ? in[base + i] : Op::template id<T>();
     }
+#pragma unroll
+    for (int i = 0; i < SCAN_I; ++i) acc = op(acc, v[i]);
     T tot;
     T pre = block_excl(acc, tot, op);
     T c = carry ? carry[blockIdx.x] : Op::template id<T>();
     pre = op(c, pre);
 #pragma unroll
     for (int i = 0; i < SCAN_I; ++i) {
-        T nx = op(pre, v[i]);
-        if (base + i < n) out[base + i] = INCL ? nx : pre;
+        const T nx = op(pre, v[i]);
+        v[i] = INCL ? nx : pre;
         pre = nx;
+    }
+    if (full && sectors(out)) {
+        store_items(out + base, v);
+    } else {
+#pragma unroll
+        for (int i = 0; i < SCAN_I; ++i)
+            if (base + i < n) out[base + i] = v[i];
     }
     if (total && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *total = op(c, tot);
 }
