@@ -482,6 +482,14 @@ struct WarpRange {
 // to the left, whatever came before.  So only a match found at c0 - 1 itself may be no SMEM, and the
 // item leaves it out; it ends at the first start of c1 or later.  Together the items give the SMEMs
 // of the read, each once, in order.
+//
+// In a batch of at most LONG_BASES bases, reads of LONG_LEN bases or more are cut before their first step:
+// such a batch takes as long as its longest chains, not as its work (200,000 reads of 100 bp - 10 kb, 430
+// Mbases: 8.4 -> 7.4 ms; a served mix with a few long reads 7.1 -> 2.8 ms; the cut costs about 35 steps per item, so larger batches, which fill the chip,
+// keep their reads whole until `steps`).
+constexpr u64 LONG_BASES = 1ull << 29;
+constexpr int LONG_LEN = 1024;
+constexpr u32 STEPS_LONG = 0x3FFFFFu;   // in the step count: cut at once
 struct Item {
     u32 read;
     int c0, c1;
@@ -490,7 +498,7 @@ struct Item {
 struct HeavyRead {
     u32 read, first, n, cnt;   // its items and the records found before the cut (bit 31: one found no room)
 };
-constexpr u32 NO_ROOM = 1u << 31;
+constexpr u32 NO_ROOM = 1u << 31, NO_READ = ~0u;
 // A record that found no slot: its number within the read (or, bit 31 of `who` set, within an item).
 struct PoolRec {
     u32 who, idx;
@@ -779,6 +787,9 @@ __global__ void __launch_bounds__(512, 2)
     const u32 n = (u32)I.n, prim = (u32)I.primary;
     const int K = (int)I.kmer_k;
     const u64 o0 = off[0], o1 = off[nr];
+    // long reads are cut before their first step in batches that do not fill the chip anyway
+    const int long_len = o1 - o0 <= LONG_BASES ? LONG_LEN : INT_MAX;
+    const u32 long_starts = o1 - o0 <= LONG_BASES / 8 ? 256u : 512u;
     u32 ntodo = nr;
     if (ITEMS) {
         ntodo = sp.n[0] < sp.items_cap ? sp.n[0] : sp.items_cap;
@@ -1032,15 +1043,19 @@ __global__ void __launch_bounds__(512, 2)
                 if (!ITEMS && !fin && (meta >> M_STEP) > sp.steps && S.u >= 1 && S.u <= 3) {
                     // the starts left: after i once its match is recorded, else from i on
                     const int c = S.u == 3 ? S.i + 1 : S.i, left = S.L - (int)lr + 1 - c;
-                    const u32 k = left > 0 ? ((u32)left + sp.starts - 1) / sp.starts : 0u;
+                    const u32 starts = (meta >> M_STEP) == STEPS_LONG ? long_starts : sp.starts;
+                    const u32 k = left > 0 ? ((u32)left + starts - 1) / starts : 0u;
                     if (k > 1) {
-                        u32 q = sp.n[0], seen;   // room for k items, or none is taken
-                        while (q + k <= sp.items_cap && (seen = atomicCAS(sp.n, q, q + k)) != q) q = seen;
-                        if (q + k <= sp.items_cap) {
+                        // room for k items; what a read past the end of the room took of it holds none
+                        u32 q = *(volatile u32 *)sp.n;
+                        if (q < sp.items_cap) q = atomicAdd(sp.n, k);
+                        if (q < sp.items_cap && k > sp.items_cap - q)
+                            for (u32 t = q; t < sp.items_cap; ++t) sp.items[t] = Item{NO_READ, 0, 0, 0u};
+                        if (q < sp.items_cap && k <= sp.items_cap - q) {
                             cut = true;
                             for (u32 t = 0; t < k; ++t)
-                                sp.items[q + t] = Item{r, c + (int)(t * sp.starts),
-                                                       t + 1 < k ? c + (int)((t + 1) * sp.starts) : INT_MAX, 0u};
+                                sp.items[q + t] = Item{r, c + (int)(t * starts),
+                                                       t + 1 < k ? c + (int)((t + 1) * starts) : INT_MAX, 0u};
                             sp.heavy[atomicAdd(sp.n + 1, 1u)] = HeavyRead{r, q, k, cnt | (meta & M_DROP ? NO_ROOM : 0u)};
                             if (!ITEMS && cnt < cap) slots[sb + cnt].qend = 0;   // ends the read's slots
                             fin = true;
@@ -1055,6 +1070,7 @@ __global__ void __launch_bounds__(512, 2)
                 }
             }
             // finished reads give their slots to the next ones
+            bool uncut = false;   // a long read, to be cut in its next service
             const bool want = fin || (on && (meta & M_NEW));
             const u32 fm = __ballot_sync(FULL, want);
             if (fm) {
@@ -1068,7 +1084,9 @@ __global__ void __launch_bounds__(512, 2)
                     r = (u32)item;
                     Item it{r, 0, 0, 0u};
                     if (ITEMS) it = sp.items[r];
-                    u64 b = off[it.read], e = off[it.read + 1];
+                    const bool none = ITEMS && it.read == NO_READ;
+                    if (none) it.read = 0;
+                    u64 b = off[it.read], e = none ? b : off[it.read + 1];
                     if (b > e || b < o0 || e > o1) {   // offsets outside the batch or decreasing: nothing is read
                         atomicOr(err, (u32)DEVCHK_OFFSETS);
                         b = e = o0;
@@ -1092,6 +1110,10 @@ __global__ void __launch_bounds__(512, 2)
                     S.pos = 0;
                     restart();
                     wb = INT_MIN / 2;   // no window yet
+                    if (!ITEMS && S.u == 1 && S.L >= long_len) {
+                        uncut = true;
+                        meta |= STEPS_LONG << M_STEP;
+                    }
                     W.rd[x] = r;
                     W.at[x] = b;
                     W.L[x] = S.L;
@@ -1102,6 +1124,8 @@ __global__ void __launch_bounds__(512, 2)
             }
             if (on && cls != C_FREE) {
                 W.cnt[x] = cnt;
+            }
+            if (on && cls != C_FREE && !uncut) {
                 // stage changes up to the next memory action
                 if (S.u == 3 && S.j <= S.i) {           // back to stage 1 at the next start
                     S.u = 1;
@@ -2114,7 +2138,7 @@ constexpr u32 SPLIT_STEPS = 1024, SEG_STARTS = 256;
 struct SplitRoom {
     u32 items, heavy, pool;
     SplitRoom(u64 bases, u64 n_reads) {
-        const u64 it = n_reads / 8 + bases / 1024 + 4096, po = n_reads / 2 + bases / 256 + 16384;
+        const u64 it = n_reads / 8 + bases / (bases <= LONG_BASES ? 256 : 1024) + 4096, po = n_reads / 2 + bases / 256 + 16384;
         items = (u32)(it < (1u << 30) ? it : 1u << 30);
         heavy = items / 2 + 1;   // a cut read has at least two items
         pool = n_reads < NO_ROOM ? (u32)(po < (1u << 30) ? po : 1u << 30) : 0u;
