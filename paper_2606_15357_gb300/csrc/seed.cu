@@ -485,8 +485,8 @@ struct WarpRange {
 //
 // In a batch of at most LONG_BASES bases, reads of LONG_LEN bases or more are cut before their first step:
 // such a batch takes as long as its longest chains, not as its work (200,000 reads of 100 bp - 10 kb, 430
-// Mbases: 8.4 -> 7.4 ms; a served mix with a few long reads 7.1 -> 2.8 ms; the cut costs about 35 steps per item, so larger batches, which fill the chip,
-// keep their reads whole until `steps`).
+// Mbases: 8.4 -> 7.4 ms; a served mix with a few long reads 7.1 -> 2.8 ms).  A cut costs about 35 steps
+// per item, so larger batches, which fill the chip, keep their reads whole until `steps`.
 constexpr u64 LONG_BASES = 1ull << 29;
 constexpr int LONG_LEN = 1024;
 constexpr u32 STEPS_LONG = 0x3FFFFFu;   // in the step count: cut at once
@@ -789,7 +789,7 @@ __global__ void __launch_bounds__(512, 2)
     const u64 o0 = off[0], o1 = off[nr];
     // long reads are cut before their first step in batches that do not fill the chip anyway
     const int long_len = o1 - o0 <= LONG_BASES ? LONG_LEN : INT_MAX;
-    const u32 long_starts = o1 - o0 <= LONG_BASES / 8 ? 256u : 512u;
+    const u32 long_starts = o1 - o0 <= LONG_BASES / 8 ? 256u : 1024u;
     u32 ntodo = nr;
     if (ITEMS) {
         ntodo = sp.n[0] < sp.items_cap ? sp.n[0] : sp.items_cap;
