@@ -1109,7 +1109,7 @@ __global__ void __launch_bounds__(512, 2)
                     }
                     S.pos = 0;
                     restart();
-                    wb = INT_MIN / 2;   // no window yet
+                    W.wb[x] = wb = INT_MIN / 2;   // no window yet
                     if (!ITEMS && S.u == 1 && S.L >= long_len) {
                         uncut = true;
                         meta |= STEPS_LONG << M_STEP;

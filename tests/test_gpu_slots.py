@@ -1,6 +1,8 @@
 """The SMEM kernel's slot form at its edges, against the CPU oracle: reads cut into items (long reads
 inside tandem repeats), records past a read's slots (the pool, and the pass that recomputes a read
 when the pool is full), windows of read bases at every alignment, N, reads shorter than l."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -56,3 +58,25 @@ def test_slots_match_oracle(mb, tandem, l, c, shift, slots):
     assert psm.tobytes() == sm.tobytes()
     hits, _ = mb.mb_locate(G, sm, m, opts=o, cap=nh)
     assert np.array_equal(phits, hits)
+
+
+def test_long_reads_without_room_to_cut(mb, tandem):
+    """The no-allocation call has no items: long reads, meant to be cut at once, run whole in slots that
+    held other reads before."""
+    ref, seq, off, G, X = tandem
+    reps = 8
+    big = np.tile(seq, reps)
+    boff = np.concatenate([off[:-1] + i * off[-1] for i in range(reps)] + [[reps * off[-1]]]).astype(np.uint64)
+    n = len(boff) - 1
+    dseq, doff = torch.from_numpy(big).cuda(), torch.from_numpy(boff.view(np.int64)).cuda()
+    want, m, _ = mb.mb_seed_batch(G, big, boff)
+    out = torch.empty(m * 48, dtype=torch.uint8, device="cuda")
+    for slots in (1, 5, 0):
+        no, nh = ctypes.c_uint64(), ctypes.c_uint64()
+        o = mb.Opts(smem_reads_per_warp=slots)
+        rc = mb.lib().mb_seed_batch_noalloc(G.handle, ctypes.c_void_p(dseq.data_ptr()),
+                                            ctypes.c_void_p(doff.data_ptr()), n, None, ctypes.byref(o), None,
+                                            ctypes.c_void_p(out.data_ptr()), m, ctypes.byref(no), ctypes.byref(nh))
+        assert rc == 0 and no.value == m and out.cpu().numpy().tobytes() == want.tobytes()
+    osm = X.seed(seq, off, 19, 1, 500)[0]
+    assert m == reps * len(osm) and np.array_equal(want["qbeg"][:len(osm)], osm["qbeg"])
