@@ -258,12 +258,14 @@ __host__ __device__ __forceinline__ u64 mb_mix64(u64 z) {
 
 // ----------------------------------------------------------------------------- primitives
 // Exclusive prefix sum of n values (in place allowed).  *total (device, may be null) receives
-// the sum.  Uses `tmp` (device) of at least scan_tmp_bytes(n) bytes.
+// the sum.  Uses `tmp` (device) of at least scan_tmp_bytes(n) bytes.  With n_dev (device) only the first
+// min(n, *n_dev) values take part; the others are neither read nor written.
 size_t scan_tmp_bytes(size_t n);
-int scan_exclusive_u64(const u64 *in, u64 *out, size_t n, u64 *total, void *tmp, cudaStream_t st);
+int scan_exclusive_u64(const u64 *in, u64 *out, size_t n, u64 *total, void *tmp, cudaStream_t st,
+                       const u64 *n_dev = nullptr);
 int scan_exclusive_u32(const u32 *in, u32 *out, size_t n, u32 *total, void *tmp, cudaStream_t st);
 // Inclusive prefix maximum of u32 values (in place allowed).
-int scan_inclusive_max_u32(const u32 *in, u32 *out, size_t n, void *tmp, cudaStream_t st);
+int scan_inclusive_max_u32(const u32 *in, u32 *out, size_t n, void *tmp, cudaStream_t st, const u64 *n_dev = nullptr);
 
 // Stable LSD radix sort of (key, val) pairs by the key bits in [lo_bit, hi_bit) of each digit
 // range given.  Sorted output ends in (keys, vals); (keys_alt, vals_alt) are scratch of the

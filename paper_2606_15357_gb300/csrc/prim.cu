@@ -81,8 +81,15 @@ __device__ __forceinline__ void store_items(T *p, const T v[SCAN_I]) {
 }
 __device__ __forceinline__ bool sectors(const void *p) { return ((uintptr_t)p & 31) == 0; }
 
+// With n_dev (device) only the first min(n, *n_dev) items take part: tiles past them read and write
+// nothing but an identity partial.
 template <class T, class Op>
-__global__ void k_scan_reduce(const T *__restrict__ in, size_t n, T *__restrict__ part, Op op) {
+__global__ void k_scan_reduce(const T *__restrict__ in, size_t n, const u64 *n_dev, T *__restrict__ part, Op op) {
+    if (n_dev && *n_dev < n) n = (size_t)*n_dev;
+    if (blockIdx.x * SCAN_TILE >= n) {
+        if (threadIdx.x == 0) part[blockIdx.x] = Op::template id<T>();
+        return;
+    }
     size_t base = blockIdx.x * SCAN_TILE + (size_t)threadIdx.x * SCAN_I;
     T acc = Op::template id<T>();
     if (base + SCAN_I <= n && sectors(in)) {
@@ -102,7 +109,9 @@ __global__ void k_scan_reduce(const T *__restrict__ in, size_t n, T *__restrict_
 
 // Scans one tile; carry = scanned partial of this tile (exclusive), or identity for one tile.
 template <class T, class Op, bool INCL>
-__global__ void k_scan_apply(const T *in, T *out, size_t n, const T *__restrict__ carry, T *total, Op op) {
+__global__ void k_scan_apply(const T *in, T *out, size_t n, const u64 *n_dev, const T *__restrict__ carry, T *total, Op op) {
+    if (n_dev && *n_dev < n) n = (size_t)*n_dev;
+    if (blockIdx.x * SCAN_TILE >= n && !(total && blockIdx.x == gridDim.x - 1)) return;
     size_t base = blockIdx.x * SCAN_TILE + (size_t)threadIdx.x * SCAN_I;
     T v[SCAN_I];
     T acc = Op::template id<T>();
@@ -138,33 +147,33 @@ __global__ void k_scan_apply(const T *in, T *out, size_t n, const T *__restrict_
 size_t level_blocks(size_t n) { return (n + SCAN_TILE - 1) / SCAN_TILE; }
 
 template <class T, class Op, bool INCL>
-int scan_impl(const T *in, T *out, size_t n, T *total, void *tmp, cudaStream_t st, Op op) {
+int scan_impl(const T *in, T *out, size_t n, T *total, void *tmp, cudaStream_t st, Op op, const u64 *n_dev = nullptr) {
     if (n == 0) return MB_OK;
     size_t nb = level_blocks(n);
     if (nb == 1) {
-        k_scan_apply<T, Op, INCL><<<1, SCAN_T, 0, st>>>(in, out, n, nullptr, total, op);
+        k_scan_apply<T, Op, INCL><<<1, SCAN_T, 0, st>>>(in, out, n, n_dev, nullptr, total, op);
         MB_KCHECK();
         return MB_OK;
     }
     T *part = (T *)tmp;
     void *rest = (void *)((char *)tmp + ((nb * sizeof(u64) + 255) & ~(size_t)255));
-    k_scan_reduce<T, Op><<<(unsigned)nb, SCAN_T, 0, st>>>(in, n, part, op);
+    k_scan_reduce<T, Op><<<(unsigned)nb, SCAN_T, 0, st>>>(in, n, n_dev, part, op);
     MB_KCHECK();
     // exclusive scan of the tile sums gives each tile's carry
     MB_TRY((scan_impl<T, Op, false>(part, part, nb, nullptr, rest, st, op)));
-    k_scan_apply<T, Op, INCL><<<(unsigned)nb, SCAN_T, 0, st>>>(in, out, n, part, total, op);
+    k_scan_apply<T, Op, INCL><<<(unsigned)nb, SCAN_T, 0, st>>>(in, out, n, n_dev, part, total, op);
     MB_KCHECK();
     return MB_OK;
 }
 
 // exclusive sum; total: of all inputs (written by the last tile)
 template <class T>
-int scan_excl_total(const T *in, T *out, size_t n, T *total, void *tmp, cudaStream_t st) {
+int scan_excl_total(const T *in, T *out, size_t n, T *total, void *tmp, cudaStream_t st, const u64 *n_dev) {
     if (n == 0) {
         if (total) MB_CK(cudaMemsetAsync(total, 0, sizeof(T), st));
         return MB_OK;
     }
-    return scan_impl<T, OpSum, false>(in, out, n, total, tmp, st, OpSum());
+    return scan_impl<T, OpSum, false>(in, out, n, total, tmp, st, OpSum(), n_dev);
 }
 
 }  // namespace
@@ -179,16 +188,16 @@ size_t scan_tmp_bytes(size_t n) {
     return b + 256;
 }
 
-int scan_exclusive_u64(const u64 *in, u64 *out, size_t n, u64 *total, void *tmp, cudaStream_t st) {
-    return scan_excl_total<u64>(in, out, n, total, tmp, st);
+int scan_exclusive_u64(const u64 *in, u64 *out, size_t n, u64 *total, void *tmp, cudaStream_t st, const u64 *n_dev) {
+    return scan_excl_total<u64>(in, out, n, total, tmp, st, n_dev);
 }
 
 int scan_exclusive_u32(const u32 *in, u32 *out, size_t n, u32 *total, void *tmp, cudaStream_t st) {
-    return scan_excl_total<u32>(in, out, n, total, tmp, st);
+    return scan_excl_total<u32>(in, out, n, total, tmp, st, nullptr);
 }
 
-int scan_inclusive_max_u32(const u32 *in, u32 *out, size_t n, void *tmp, cudaStream_t st) {
-    return scan_impl<u32, OpMax, true>(in, out, n, nullptr, tmp, st, OpMax());
+int scan_inclusive_max_u32(const u32 *in, u32 *out, size_t n, void *tmp, cudaStream_t st, const u64 *n_dev) {
+    return scan_impl<u32, OpMax, true>(in, out, n, nullptr, tmp, st, OpMax(), n_dev);
 }
 
 // ============================================================================ radix sort

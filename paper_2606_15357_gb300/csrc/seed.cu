@@ -1412,18 +1412,16 @@ __global__ void k_share_flag(const mb_smem *__restrict__ sm, u64 cap, const u64 
                              const u32 *__restrict__ known, u32 *__restrict__ hits, u64 hits_cap,
                              u64 *__restrict__ flag, u64 n, u32 *err) {
     const u64 nsm = count_of(cap, nsm_dev);
-    for (u64 t = blockIdx.x * (u64)blockDim.x + threadIdx.x; t < cap; t += (u64)gridDim.x * blockDim.x) {
+    for (u64 t = blockIdx.x * (u64)blockDim.x + threadIdx.x; t < nsm; t += (u64)gridDim.x * blockDim.x) {
         u64 f = 0;
-        if (t < nsm) {
-            const u64 cnt = hits_of(sm, t);
-            if (rows_outside(sm, t, cnt, n)) {
-                atomicOr(err, (u32)DEVCHK_RECORD);
-            } else if (walks(cnt, known, t)) {
-                f = 1;
-            } else if (cnt == 1) {   // known position
-                const u64 ho = __ldg(&sm[t].hit_off);
-                if (ho < hits_cap) hits[ho] = known[t];
-            }
+        const u64 cnt = hits_of(sm, t);
+        if (rows_outside(sm, t, cnt, n)) {
+            atomicOr(err, (u32)DEVCHK_RECORD);
+        } else if (walks(cnt, known, t)) {
+            f = 1;
+        } else if (cnt == 1) {   // known position
+            const u64 ho = __ldg(&sm[t].hit_off);
+            if (ho < hits_cap) hits[ho] = known[t];
         }
         flag[t] = f;
     }
@@ -1445,22 +1443,18 @@ __global__ void k_share_compact(const mb_smem *__restrict__ sm, u64 cap, const u
 }
 
 // For sorted record t < nw: its s and hit offset in sorted order, and ends[t] = k + s (saturated
-// to 32 bits); ends = 0 past the records.
+// to 32 bits).
 __global__ void k_share_gather(const mb_smem *__restrict__ sm, const u64 *__restrict__ keys,
                                const u32 *__restrict__ vals, u64 cap, const u64 *__restrict__ nw_dev,
                                u32 *__restrict__ ss, u64 *__restrict__ sho, u32 *__restrict__ ends) {
     const u64 nw = count_of(cap, nw_dev);
-    for (u64 t = blockIdx.x * (u64)blockDim.x + threadIdx.x; t < cap; t += (u64)gridDim.x * blockDim.x) {
-        u32 e = 0;
-        if (t < nw) {
-            const u32 r = vals[t];
-            const u64 s = __ldg(&sm[r].s);
-            const u64 end = (keys[t] >> SHARE_S_BITS) + s;
-            ss[t] = (u32)s;
-            sho[t] = __ldg(&sm[r].hit_off);
-            e = end < 0xFFFFFFFFull ? (u32)end : 0xFFFFFFFFu;
-        }
-        ends[t] = e;
+    for (u64 t = blockIdx.x * (u64)blockDim.x + threadIdx.x; t < nw; t += (u64)gridDim.x * blockDim.x) {
+        const u32 r = vals[t];
+        const u64 s = __ldg(&sm[r].s);
+        const u64 end = (keys[t] >> SHARE_S_BITS) + s;
+        ss[t] = (u32)s;
+        sho[t] = __ldg(&sm[r].hit_off);
+        ends[t] = end < 0xFFFFFFFFull ? (u32)end : 0xFFFFFFFFu;
     }
 }
 
@@ -1470,16 +1464,14 @@ __global__ void k_share_mark(const u64 *__restrict__ keys, const u32 *__restrict
                              const u64 *__restrict__ nw_dev, const u32 *__restrict__ pmax, u64 *__restrict__ len,
                              u32 *__restrict__ last) {
     const u64 nw = count_of(cap, nw_dev);
-    for (u64 t = blockIdx.x * (u64)blockDim.x + threadIdx.x; t < cap; t += (u64)gridDim.x * blockDim.x) {
+    for (u64 t = blockIdx.x * (u64)blockDim.x + threadIdx.x; t < nw; t += (u64)gridDim.x * blockDim.x) {
         u64 l = 0;
         u32 lm = 0;
-        if (t < nw) {
-            const u64 end = (keys[t] >> SHARE_S_BITS) + ss[t];
-            const u32 e = end < 0xFFFFFFFFull ? (u32)end : 0xFFFFFFFFu;
-            if (t == 0 || e > pmax[t - 1]) {   // pmax[t - 1] >= 1 here, so the first record is maximal
-                l = ss[t];
-                lm = (u32)t;
-            }
+        const u64 end = (keys[t] >> SHARE_S_BITS) + ss[t];
+        const u32 e = end < 0xFFFFFFFFull ? (u32)end : 0xFFFFFFFFu;
+        if (t == 0 || e > pmax[t - 1]) {   // pmax[t - 1] >= 1 here, so the first record is maximal
+            l = ss[t];
+            lm = (u32)t;
         }
         len[t] = l;
         last[t] = lm;
@@ -2277,7 +2269,7 @@ int locate_shared(const DevIndex &I, const mb_smem *sm, u64 cap, const u64 *nsm_
     const unsigned G = grid_for(cap, 256);
     k_share_flag<<<G, 256, 0, st>>>(sm, cap, nsm_dev, known, hits, hits_cap, b.roff, I.n, b.err);
     MB_KCHECK();
-    MB_TRY(scan_exclusive_u64(b.roff, b.roff, cap, b.nwalk, b.tmp, st));
+    MB_TRY(scan_exclusive_u64(b.roff, b.roff, cap, b.nwalk, b.tmp, st, nsm_dev));
     k_share_compact<<<G, 256, 0, st>>>(sm, cap, nsm_dev, known, b.roff, b.keys, b.vals, I.n);
     MB_KCHECK();
     const BitRange r[1] = {{0, share_key_bits(I.n)}};
@@ -2286,11 +2278,11 @@ int locate_shared(const DevIndex &I, const mb_smem *sm, u64 cap, const u64 *nsm_
     u64 *sho = b.keys_alt;
     k_share_gather<<<G, 256, 0, st>>>(sm, b.keys, b.vals, cap, b.nwalk, ss, sho, b.pmax);
     MB_KCHECK();
-    MB_TRY(scan_inclusive_max_u32(b.pmax, b.pmax, cap, b.tmp, st));
+    MB_TRY(scan_inclusive_max_u32(b.pmax, b.pmax, cap, b.tmp, st, b.nwalk));
     k_share_mark<<<G, 256, 0, st>>>(b.keys, ss, cap, b.nwalk, b.pmax, b.roff, b.last);
     MB_KCHECK();
-    MB_TRY(scan_exclusive_u64(b.roff, b.roff, cap, b.nrows, b.tmp, st));
-    MB_TRY(scan_inclusive_max_u32(b.last, b.last, cap, b.tmp, st));
+    MB_TRY(scan_exclusive_u64(b.roff, b.roff, cap, b.nrows, b.tmp, st, b.nwalk));
+    MB_TRY(scan_inclusive_max_u32(b.last, b.last, cap, b.tmp, st, b.nwalk));
     k_share_rows<<<G, 256, 0, st>>>(b.keys, ss, b.last, b.roff, cap, b.nwalk, b.rows, hits_cap);
     MB_KCHECK();
     u32 *chk = b.checked ? b.err : nullptr;
@@ -3004,7 +2996,6 @@ static int plan_seed(mb_plan *P, const uint8_t *seq, const uint64_t *off, uint32
     const u32 bs = (P->flags & MB_BS3) ? 1u : 0u;
     u64 *n_smem = P->misc, *n_hits = P->misc + 1;
     u32 *ovf_n = (u32 *)(P->misc + 2), *qhead = (u32 *)(P->misc + 3), *err = plan_err(P);
-    MB_CK(cudaMemsetAsync(P->hitc, 0, P->max_smem * 8, st));   // zero tail for the fixed-length scan
     SmemArgs sa{I, seq, off, n_reads, mate, bs, P->l, P->c, P->kmer, P->slots, P->nslots, P->counts, P->ovf, ovf_n,
                 qhead, nullptr, nullptr, I.text2 && !(P->flags & MB_STEP_ONLY)};
     sa.sp = P->split;
@@ -3023,7 +3014,7 @@ static int plan_seed(mb_plan *P, const uint8_t *seq, const uint64_t *off, uint32
     k_smem_overflow<<<resident_grid((const void *)k_smem_overflow, 128, 1ull << 40), 128, 0, st>>>(I, seq, off, n_reads, mate, bs, P->l, P->c, P->kmer, P->ovf, ovf_n, P->soff,
                                          P->max_occ, P->out, P->hitc, P->max_smem, nullptr, P->known);
     MB_KCHECK();
-    MB_TRY(scan_exclusive_u64(P->hitc, P->hitc, P->max_smem, n_hits, P->tmp, st));
+    MB_TRY(scan_exclusive_u64(P->hitc, P->hitc, P->max_smem, n_hits, P->tmp, st, n_smem));
     k_set_hitoff<<<grid_for(P->max_smem, 256), 256, 0, st>>>(P->hitc, P->max_smem, n_smem, P->out);
     MB_KCHECK();
     return MB_OK;
