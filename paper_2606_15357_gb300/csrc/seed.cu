@@ -1260,22 +1260,27 @@ __global__ void __launch_bounds__(256)
     s_slot[w][lane] = sb - (incl - cnt);
     s_out[w][lane] = o - (incl - cnt);
     __syncwarp();
+    u32 ended = 32;   // the read, if any, that goes on into the next 32 slots but has ended before them
     for (u32 t0 = 0; t0 < total; t0 += 32) {
         const u32 t = t0 + lane;
-        u32 q = 0;
+        u32 q = 0, first = 0;   // the slot's read, and that read's first t
         bool ok = t < total;
         u64 m = 0;
+        SlotRec x{};
         if (ok) {
 #pragma unroll
             for (u32 b = 16; b; b >>= 1)
                 if (s_end[w][q + b - 1] <= t) q += b;
-            const u64 at = s_slot[w][q] + t;
-            const SlotRec x = slots[at];
+            first = q ? s_end[w][q - 1] : 0u;
+            x = slots[s_slot[w][q] + t];
             m = s_out[w][q] + t;
-            // a slot with qend = 0 ends its read; what lies behind it was never written
-            const u32 first = q ? s_end[w][q - 1] : 0u;
-            for (u64 b = s_slot[w][q] + first; ok && b <= at; ++b) ok = slots[b].qend != 0;
-            ok = ok && m < out_cap;
+        }
+        // a slot with qend = 0 ends its read; what lies behind it was never written
+        const u32 ends = __ballot_sync(FULL, ok && x.qend == 0), from_lane = first > t0 ? first - t0 : 0u;
+        ok = ok && !((ends & (FULL >> (31 - lane))) >> from_lane) && !(q == ended && first < t0);
+        ended = __shfl_sync(FULL, ok ? 32u : q, 31);
+        ok = ok && m < out_cap;
+        if (ok) {
             const bool over = x.s > max_occ;
             u64 *rec = s_rec[w] + 6 * lane;
             rec[0] = (u64)(u32)(r0 + q) | ((u64)x.qbeg << 32);
@@ -1284,10 +1289,8 @@ __global__ void __launch_bounds__(256)
             rec[3] = x.kr;
             rec[4] = x.s;
             rec[5] = 0;
-            if (ok) {
-                hitc[m] = over ? 0 : x.s;
-                if (known) known[m] = x.pos;
-            }
+            hitc[m] = over ? 0 : x.s;
+            if (known) known[m] = x.pos;
         }
         // the records as 64-bit words, neighbouring lanes neighbouring words
         const u32 mask = __ballot_sync(FULL, ok);
