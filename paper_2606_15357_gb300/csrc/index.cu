@@ -66,11 +66,13 @@ u32 mb_index_flags(const mb_index *x) { return x->flags; }
 namespace {
 
 constexpr u64 GOLDEN = 0x9E3779B97F4A7C15ULL;
-// Sort key of a suffix: its first 21 symbols, two bits each, the first highest, $ and what follows it as
-// A; then in 5 bits how many of them come before $ (21 at most), which puts a suffix that ends early
-// before those that go on with A's, as $ < A asks.  47 bits: six passes of the sort (27 symbols in base 5
-// took eight); random texts of 2^32 symbols leave a thousandth of their suffixes tied.
-constexpr int KEY_SYMS = 21, KEY_REM_BITS = 5, KEY_BITS = 2 * KEY_SYMS + KEY_REM_BITS;
+// Sort key of a suffix: its first 20 symbols, two bits each, the first highest, $ and what follows it as
+// A.  A suffix that ends within them is below every other one with its key ($ < A), and below a longer one
+// that ends within them: the sort is stable and starts from the shortest suffix, so they come first in that
+// order, and k_heads gives each its own run.  40 bits are five passes of the sort (21 symbols and the
+// symbols before $ in 5 more bits took six); random texts of 2^32 symbols leave a few thousandths of their
+// suffixes tied.
+constexpr int KEY_SYMS = 20, KEY_BITS = 2 * KEY_SYMS;
 
 __device__ __forceinline__ u8 ref_base(const u8 *__restrict__ R, u64 x, u64 seed) {
     u8 b = R[x];
@@ -104,25 +106,26 @@ __device__ __forceinline__ u32 high_first(u32 w) {
     return ((w >> 1) & 0x55555555u) | ((w & 0x55555555u) << 1);
 }
 __global__ void k_init_keys(const u32 *__restrict__ t2, u64 words, u64 n, u64 *__restrict__ keys, u32 *__restrict__ vals) {
-    for (u64 i = blockIdx.x * (u64)blockDim.x + threadIdx.x; i < n; i += (u64)gridDim.x * blockDim.x) {
-        const u64 w = i >> 4;
+    for (u64 t = blockIdx.x * (u64)blockDim.x + threadIdx.x; t < n; t += (u64)gridDim.x * blockDim.x) {
+        const u64 i = n - 1 - t, w = i >> 4;
         const u32 a = high_first(t2[w]), b = high_first(t2[w + 1]), c = w + 2 < words ? high_first(t2[w + 2]) : 0u;
         const u32 sh = 2 * (u32)(i & 15);
         const u64 v = ((u64)__funnelshift_l(b, a, sh) << 32) | __funnelshift_l(c, b, sh);
-        const u64 rem = n - 1 - i;
-        keys[i] = ((v >> (64 - 2 * KEY_SYMS)) << KEY_REM_BITS) | (rem < KEY_SYMS ? rem : KEY_SYMS);
-        vals[i] = (u32)i;
+        keys[t] = v >> (64 - KEY_BITS);
+        vals[t] = (u32)i;
     }
 }
 
 // hv[t] = (start of a new key run) ? pos(t) : 0, for a max-scan giving each item its run head.
-// flag[t] = item t is in a run of more than one key.
+// flag[t] = item t is in a run of more than one key.  With SA (the sorted suffixes of a text of n symbols) a
+// suffix that ends within its key is a run of its own.
 __global__ void k_heads(const u64 *__restrict__ keys, const u32 *__restrict__ pos, u64 A, u32 *__restrict__ hv,
-                        u32 *__restrict__ flag) {
+                        u32 *__restrict__ flag, const u32 *__restrict__ SA = nullptr, u64 n = 0) {
+    auto ends = [&](u64 t) { return SA && (u64)SA[t] + KEY_SYMS > n - 1; };
     for (u64 t = blockIdx.x * (u64)blockDim.x + threadIdx.x; t < A; t += (u64)gridDim.x * blockDim.x) {
         u64 k = keys[t];
-        bool head = t == 0 || keys[t - 1] != k;
-        bool last = t == A - 1 || keys[t + 1] != k;
+        bool head = t == 0 || keys[t - 1] != k || ends(t - 1) || ends(t);
+        bool last = t == A - 1 || keys[t + 1] != k || ends(t) || ends(t + 1);
         hv[t] = head ? (pos ? pos[t] : (u32)t) : 0u;
         flag[t] = (head && last) ? 0u : 1u;
     }
@@ -509,7 +512,8 @@ static int make_sa_ref(mb_index *x) {
 // Seeding's own k-mer table, as deep as 4^k <= n / 2 (13 at 100 Mbp, 14 at 1 Gbp), where the index's
 // table (k = 10 by default, Section 2.5, sized for a CPU cache) is shallower: every further base is an
 // extension less per lookup, of a wide interval and so of two blocks.  Same SMEMs with any k.  It takes
-// 1.5 to 6 bytes per text position; without room for it seeding uses the index's own.
+// 1.5 to 6 bytes per text position; without room for it seeding uses the index's own.  2M reads on
+// 100 Mbp (k = 10 -> 13), seeded and located: 3.36 -> 3.10 ms.
 static int build_kmer2(mb_index *x, cudaStream_t st) {
     u32 k = x->kmer_k;
     while (k < 16 && (1ULL << (2 * k + 2)) <= x->n / 2) ++k;
@@ -546,8 +550,8 @@ static int build_kmer2(mb_index *x, cudaStream_t st) {
 // n each) receive it and its inverse.
 static int build_sa(const u32 *t2, u64 t2words, u64 n, u32 *SA, u32 *rank, cudaStream_t st) {
     // 20 bytes per suffix: keys and the sort's spare keys (8 + 8) and spare values (4; SA holds the
-    // values); the run heads and flags (4 + 4) live in the spare keys, which are free whenever they are
-    // used.  The rounds add 12 bytes per suffix still active (two active lists, values).
+    // values); the run heads live in the spare keys and the flags in the spare values, which are free
+    // whenever they are used.  The rounds add 12 bytes per suffix still active (two active lists, values).
     DevBuf bk, bka, bva, btmp, bact, bact2, bv, berr, bcount;
     MB_TRY(bk.alloc(n * 8, st));
     MB_TRY(bka.alloc(n * 8, st));
@@ -559,21 +563,27 @@ static int build_sa(const u32 *t2, u64 t2words, u64 n, u32 *SA, u32 *rank, cudaS
     MB_TRY(bcount.alloc(8, st));
     u64 *keys = bk.as<u64>(), *keys_alt = bka.as<u64>();
     u32 *vals_alt = bva.as<u32>();
-    u32 *hv = bka.as<u32>(), *flag = bka.as<u32>() + n;
+    u32 *hv = bka.as<u32>(), *flag = vals_alt;
     u32 *err = berr.as<u32>(), *count = bcount.as<u32>();
     MB_CK(cudaMemsetAsync(err, 0, 4, st));
     const unsigned B = 256;
 
-    // round 0: the first 21 symbols
-    k_init_keys<<<grid_for(n, B), B, 0, st>>>(t2, t2words, n, keys, SA);
+    // round 0: the first KEY_SYMS symbols, from the spare arrays so that an odd number of passes ends in
+    // keys and SA
+    static_assert((KEY_BITS + 7) / 8 % 2 == 1, "the sort ends in the other arrays");
+    k_init_keys<<<grid_for(n, B), B, 0, st>>>(t2, t2words, n, keys_alt, vals_alt);
     MB_KCHECK();
     BitRange r0[1] = {{0, KEY_BITS}};
-    MB_TRY(radix_sort_pairs(keys, SA, keys_alt, vals_alt, n, r0, 1, btmp.p, st));
-    k_heads<<<grid_for(n, B), B, 0, st>>>(keys, nullptr, n, hv, flag);
+    bool moved = false;
+    MB_TRY(radix_sort_pairs(keys_alt, vals_alt, keys, SA, n, r0, 1, btmp.p, st, nullptr, &moved));
+    if (!moved) {   // one suffix: not sorted
+        MB_CK(cudaMemcpyAsync(keys, keys_alt, n * 8, cudaMemcpyDeviceToDevice, st));
+        MB_CK(cudaMemcpyAsync(SA, vals_alt, n * 4, cudaMemcpyDeviceToDevice, st));
+    }
+    k_heads<<<grid_for(n, B), B, 0, st>>>(keys, nullptr, n, hv, flag, SA, n);
     MB_KCHECK();
     MB_TRY(scan_inclusive_max_u32(hv, hv, n, btmp.p, st));
-    k_set_rank<<<grid_for(n, B), B, 0, st>>>(SA, hv, n, rank);
-    MB_KCHECK();
+    MB_TRY(permute_u32(SA, hv, n, nbits(n), rank, keys, keys_alt, btmp.p, st));
     MB_TRY(scan_exclusive_u32(flag, hv, n, count, btmp.p, st));   // hv reused as positions
     u32 A = 0;
     MB_CK(cudaMemcpyAsync(&A, count, 4, cudaMemcpyDeviceToHost, st));

@@ -210,7 +210,8 @@ constexpr size_t RS_TILE = (size_t)RS_T * RS_I;
 // count nothing and move nothing).
 __device__ __forceinline__ size_t items(size_t n, const u64 *n_dev) { return n_dev && *n_dev < n ? (size_t)*n_dev : n; }
 
-__global__ void __launch_bounds__(RS_T) k_radix_up(const u64 *__restrict__ keys, size_t n, const u64 *n_dev, int shift,
+template <class K>
+__global__ void __launch_bounds__(RS_T) k_radix_up(const K *__restrict__ keys, size_t n, const u64 *n_dev, int shift,
                                                    u32 mask, u32 *__restrict__ hist, size_t tiles) {
     __shared__ u32 h[256];
     n = items(n, n_dev);
@@ -232,18 +233,22 @@ __global__ void __launch_bounds__(RS_T) k_radix_up(const u64 *__restrict__ keys,
 // (iteration-major, lane-minor), warps keep theirs inside the tile, tiles theirs inside a digit: the
 // scatter is stable.  Bound: the copy of 12 bytes per item; writing each item from its lane instead
 // (partial sectors all over the digits) took 5 to 6 ms per pass of 200M items, this about 1.7 ms.
+// Without VALS an item is a word, its key in the high half and its value in the low one; with K = u32 such
+// words are made from keys and vals.
 struct RadixTile {
     u64 key[RS_TILE];
     u32 val[RS_TILE];
     u32 wh[RS_T / 32][256];   // per warp and digit: items, then their first place in the tile
     u32 to[256];              // per digit: where its run goes, less its first place in the tile
 };
-__global__ void __launch_bounds__(RS_T, 3) k_radix_down(const u64 *__restrict__ keys, const u32 *__restrict__ vals,
+template <class K, bool VALS>
+__global__ void __launch_bounds__(RS_T, 3) k_radix_down(const K *__restrict__ keys, const u32 *__restrict__ vals,
                                                         u64 *__restrict__ okeys, u32 *__restrict__ ovals, size_t n,
                                                         const u64 *n_dev, int shift, u32 mask,
                                                         const u32 *__restrict__ offs, size_t tiles) {
     extern __shared__ __align__(16) unsigned char smem[];
     RadixTile &S = *reinterpret_cast<RadixTile *>(smem);
+    constexpr bool JOIN = sizeof(K) == 4;
     n = items(n, n_dev);
     const size_t tile0 = blockIdx.x * RS_TILE;
     if (tile0 >= n) return;
@@ -253,7 +258,10 @@ __global__ void __launch_bounds__(RS_T, 3) k_radix_down(const u64 *__restrict__ 
     u64 k[RS_I];
     u32 rank[RS_I / 2];   // 16 bits each
 #pragma unroll
-    for (int it = 0; it < RS_I; ++it) k[it] = base + 32 * it < n ? keys[base + 32 * it] : 0;
+    for (int it = 0; it < RS_I; ++it) {
+        const size_t at = base + 32 * it;
+        k[it] = at < n ? (JOIN ? (u64)keys[at] << 32 | vals[at] : (u64)keys[at]) : 0;
+    }
     __syncthreads();
     const u32 lt = (1u << lane) - 1u;
 #pragma unroll
@@ -290,7 +298,7 @@ __global__ void __launch_bounds__(RS_T, 3) k_radix_down(const u64 *__restrict__ 
         if (base + 32 * it < n) {
             const u32 at = S.wh[warp][(u32)(k[it] >> shift) & mask] + ((rank[it / 2] >> (16 * (it & 1))) & 0xFFFFu);
             S.key[at] = k[it];
-            S.val[at] = vals[base + 32 * it];
+            if (VALS) S.val[at] = vals[base + 32 * it];
         }
     __syncthreads();
     const u32 cnt = (u32)(n - tile0 < RS_TILE ? n - tile0 : RS_TILE);
@@ -298,10 +306,69 @@ __global__ void __launch_bounds__(RS_T, 3) k_radix_down(const u64 *__restrict__ 
         const u64 x = S.key[i];
         const u32 at = S.to[(u32)(x >> shift) & mask] + i;
         okeys[at] = x;
-        ovals[at] = S.val[i];
+        if (VALS) ovals[at] = S.val[i];
     }
 }
+
+// out[at[t]] = v[t]
+__global__ void k_permute(const u32 *__restrict__ at, const u32 *__restrict__ v, size_t n, u32 *__restrict__ out) {
+    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x)
+        out[at[t]] = v[t];
+}
+// The same for words (place, value) of a permutation of [0, n), in order of place / PERM_WIN: window w of
+// `out` takes exactly the words of the same numbers, so a block puts them in place in shared memory.
+constexpr int PERM_BITS = 12;
+constexpr u32 PERM_WIN = 1u << PERM_BITS;
+__global__ void __launch_bounds__(256) k_permute_windows(const u64 *__restrict__ words, size_t n, u32 *__restrict__ out) {
+    __shared__ u32 win[PERM_WIN];
+    const size_t first = blockIdx.x * (size_t)PERM_WIN;
+    const u32 len = (u32)(n - first < PERM_WIN ? n - first : PERM_WIN);
+#pragma unroll 4
+    for (u32 t = threadIdx.x; t < len; t += 256) {
+        const u64 w = words[first + t];
+        win[(u32)(w >> 32) & (PERM_WIN - 1)] = (u32)w;
+    }
+    __syncthreads();
+    for (u32 t = threadIdx.x; t < len; t += 256) out[first + t] = win[t];
+}
 }  // namespace
+
+// out[at[t]] = v[t], `at` a permutation of [0, n), n <= 2^bits.  Single words written all over memory move a
+// sector each, or within what L2 holds a slot of its write rate each (200M ranks: 7.5 ms; after one radix pass
+// on the place 4.6 ms).  From 2^24 items on the items are therefore sorted by place down to windows that fit
+// shared memory, two passes up to 2^28 items and three above (200M ranks: 4.2 ms in all).
+// a, b: room for n words each (vals and `v` may lie in b), tmp: radix_tmp_bytes(n).
+int permute_u32(const u32 *at, const u32 *v, size_t n, int bits, u32 *out, u64 *a, u64 *b, void *tmp, cudaStream_t st) {
+    if (n < (size_t)1 << 24 || n >= (1ULL << 32)) {
+        k_permute<<<grid_for(n, 256), 256, 0, st>>>(at, v, n, out);
+        MB_KCHECK();
+        return MB_OK;
+    }
+    const size_t tiles = (n + RS_TILE - 1) / RS_TILE;
+    u32 *hist = (u32 *)tmp;
+    void *stmp = (char *)tmp + (((256 * tiles * sizeof(u32)) + 255) & ~(size_t)255);
+    MB_CK(cudaFuncSetAttribute(k_radix_down<u32, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RadixTile)));
+    MB_CK(cudaFuncSetAttribute(k_radix_down<u64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RadixTile)));
+    for (int sh = PERM_BITS; sh < bits; sh += 8) {
+        const u32 mask = bits - sh < 8 ? (1u << (bits - sh)) - 1u : 255u;
+        const bool first = sh == PERM_BITS;
+        if (first) k_radix_up<u32><<<(unsigned)tiles, RS_T, 0, st>>>(at, n, nullptr, sh, mask, hist, tiles);
+        else k_radix_up<u64><<<(unsigned)tiles, RS_T, 0, st>>>(b, n, nullptr, 32 + sh, mask, hist, tiles);
+        MB_KCHECK();
+        MB_TRY(scan_exclusive_u32(hist, hist, 256 * tiles, nullptr, stmp, st));
+        if (first)
+            k_radix_down<u32, false><<<(unsigned)tiles, RS_T, sizeof(RadixTile), st>>>(at, v, a, nullptr, n, nullptr, 32 + sh,
+                                                                                       mask, hist, tiles);
+        else
+            k_radix_down<u64, false><<<(unsigned)tiles, RS_T, sizeof(RadixTile), st>>>(b, nullptr, a, nullptr, n, nullptr,
+                                                                                       32 + sh, mask, hist, tiles);
+        MB_KCHECK();
+        u64 *t = a; a = b; b = t;
+    }
+    k_permute_windows<<<(unsigned)((n + PERM_WIN - 1) / PERM_WIN), 256, 0, st>>>(b, n, out);
+    MB_KCHECK();
+    return MB_OK;
+}
 
 size_t radix_tmp_bytes(size_t n) {
     size_t tiles = (n + RS_TILE - 1) / RS_TILE;
@@ -310,14 +377,15 @@ size_t radix_tmp_bytes(size_t n) {
 }
 
 int radix_sort_pairs(u64 *keys, u32 *vals, u64 *keys_alt, u32 *vals_alt, size_t n, const BitRange *ranges,
-                     int nranges, void *tmp, cudaStream_t st, const u64 *n_dev) {
+                     int nranges, void *tmp, cudaStream_t st, const u64 *n_dev, bool *in_alt) {
+    if (in_alt) *in_alt = false;
     if (n <= 1) return MB_OK;
     if (n >= (1ULL << 32)) {
         mb_set_error("radix_sort_pairs: %zu items exceed 2^32-1", n);
         return MB_ERR_ARG;
     }
     size_t tiles = (n + RS_TILE - 1) / RS_TILE;
-    MB_CK(cudaFuncSetAttribute(k_radix_down, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RadixTile)));
+    MB_CK(cudaFuncSetAttribute(k_radix_down<u64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RadixTile)));
     u32 *hist = (u32 *)tmp;
     void *stmp = (char *)tmp + (((256 * tiles * sizeof(u32)) + 255) & ~(size_t)255);
     u64 *ka = keys, *kb = keys_alt;
@@ -327,17 +395,19 @@ int radix_sort_pairs(u64 *keys, u32 *vals, u64 *keys_alt, u32 *vals_alt, size_t 
         for (int sh = ranges[r].lo; sh < ranges[r].hi; sh += 8) {
             int w = ranges[r].hi - sh < 8 ? ranges[r].hi - sh : 8;
             u32 mask = (1u << w) - 1u;
-            k_radix_up<<<(unsigned)tiles, RS_T, 0, st>>>(ka, n, n_dev, sh, mask, hist, tiles);
+            k_radix_up<u64><<<(unsigned)tiles, RS_T, 0, st>>>(ka, n, n_dev, sh, mask, hist, tiles);
             MB_KCHECK();
             MB_TRY(scan_exclusive_u32(hist, hist, 256 * tiles, nullptr, stmp, st));
-            k_radix_down<<<(unsigned)tiles, RS_T, sizeof(RadixTile), st>>>(ka, va, kb, vb, n, n_dev, sh, mask, hist, tiles);
+            k_radix_down<u64, true><<<(unsigned)tiles, RS_T, sizeof(RadixTile), st>>>(ka, va, kb, vb, n, n_dev, sh, mask, hist, tiles);
             MB_KCHECK();
             u64 *tk = ka; ka = kb; kb = tk;
             u32 *tv = va; va = vb; vb = tv;
             ++passes;
         }
     }
-    if (passes & 1) {
+    if (in_alt) {
+        *in_alt = passes & 1;
+    } else if (passes & 1) {
         MB_CK(cudaMemcpyAsync(keys, ka, n * sizeof(u64), cudaMemcpyDeviceToDevice, st));
         MB_CK(cudaMemcpyAsync(vals, va, n * sizeof(u32), cudaMemcpyDeviceToDevice, st));
     }
