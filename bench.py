@@ -815,9 +815,10 @@ def run_gpu(args):
     if args.locate_sweep:
         return locate_sweep(mb, torch, idx, out, m, hits, nh, opts)
 
-    # work counters of the chosen form (untimed pass with counting kernels)
+    # work counters of the chosen form (untimed pass with counting kernels): locate without the full
+    # suffix array walks to the rate-4 samples, each distinct row once at this many hits
     mb.profile_reset()
-    copts = dict(opts, flags=mb.MB_COUNT | (best.flags & mb.MB_LOCATE_JOIN))
+    copts = dict(opts, flags=mb.MB_COUNT | mb.MB_LOCATE_AUX)
     _, m, nh = mb.mb_seed_batch(idx, seq, off, opts=copts, out=out, cap=cap)
     mb.mb_locate(idx, out, m, opts=copts, hits=hits, cap=nh)
     wc = mb.work_counters()
@@ -889,8 +890,8 @@ def run_gpu(args):
                             "gpu_launches": graph_launches, "shape": mb.shape_of(best)},
              "reported": "graph_plan" if use_graph else "plain_launch"}
 
-    # the same graph with locate walks that stop at the index's rate-4 SA samples (MB_LOCATE_AUX):
-    # reported beside the headline, which locates through the rate-32 samples of Section 2.4
+    # the same graph with MB_LOCATE_AUX and 16 walks per lane: the walks of the headline (locate stops at
+    # the index's rate-4 SA samples by default), in another launch shape
     if not args.no_aux_form:
         aopts = dict(opts, flags=(best.flags & ~mb.MB_LOCATE_JOIN) | mb.MB_LOCATE_AUX, prefetch_depth=16)
         AP = mb.Plan(idx, n_reads, len(rd.seq), m + 1024, nh + 1024, opts=aopts)
@@ -914,8 +915,8 @@ def run_gpu(args):
         forms["graph_plan_locate_aux"] = {
             "reads_per_s": ws * args.steps * n_reads / (aux_ms / 1000.0), "ms_per_step": aux_ms / args.steps,
             "identical_output": bool(aux_same), "shape": mb.shape_of(mb.Opts(**aopts)),
-            "note": "locate walks stop at the rate-4 SA samples the index keeps for text extension "
-                    "(MB_LOCATE_AUX); not the headline, which uses the rate-32 samples"}
+            "note": "locate walks stop at the rate-4 SA samples the index keeps for text extension, as "
+                    "in the headline; 16 walks per lane"}
         log(f"graph form with MB_LOCATE_AUX: {aux_ms / args.steps:.1f} ms/step (identical: {aux_same})")
 
     # roofline of the dominant kernel: algorithmic bytes / its event-timed duration

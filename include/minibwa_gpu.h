@@ -98,7 +98,8 @@ typedef struct {
                                  beside it for seeding, of 1.5 to 6 bytes per text position, if the
                                  device has room (built with the index, also on load; not in files) */
     uint32_t flags;           /* MB_* flags above */
-    uint32_t chunk_reads;     /* mb_seed_locate: reads per pipelined chunk (0 = 2^22) */
+    uint32_t chunk_reads;     /* mb_seed_locate: reads per pipelined chunk (0 = 2^22; with host
+                                 inputs the first chunk is a quarter of the others) */
     uint32_t prefetch_depth;  /* tuning: LF-walks in flight per lane in locate, 1/2/4/8/16 (0 = 1) */
     uint32_t block_size;      /* tuning: threads per block (0 = default) */
     uint32_t smem_burst;      /* accepted, without effect: the slot form picks its steps itself */

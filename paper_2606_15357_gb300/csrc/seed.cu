@@ -710,10 +710,10 @@ __global__ void __launch_bounds__(BLOCK, BLOCK == 128 ? 6 : 1024 / BLOCK) k_smem
 // records are the same.
 //
 // What bounds it: latency of the random block reads, then their rate.  The form this replaced (one
-// read per lane, all kinds of step in one loop) had 9.6 active lanes per instruction and cost a read
-// 2,160 warp instructions; this one has 19-26 lanes in its block steps and about 900.  20M reads of
-// 150 bases on a 1 Gbp index (k = 14): 59.2 -> 45 ms, 36 -> 47 G random sectors/s, the rate the
-// random-read probe reaches; 2M reads on a 100 Mbp index 5.17 -> 2.9 ms.  More reads in flight help
+// read per lane, all kinds of step in one loop) had 9.8 active lanes per instruction and cost a read
+// 2,100 warp instructions (1 Gbp, k = 14); this one has 16.5 (19-26 in its block steps) and 1,370.  20M
+// reads of 150 bases there: 59.2 -> 45 ms (with 32-byte L2 fetches 54.5 -> 37.3), 36 -> 47 G random
+// sectors/s, the rate the random-read probe reaches; 2M reads on a 100 Mbp index 5.17 -> 2.6 ms.  More reads in flight help
 // (32 slots per warp instead of 64: 20% slower; 24 warps per SM instead of 32: 6%), so the table takes
 // the shared memory it can get: 64 slots x 32 warps x 89 bytes.  A lone read (a small batch's tail)
 // advances one extension per 0.7 us.

@@ -44,9 +44,9 @@ constexpr int MAX_SLOTS = 32;
 constexpr u64 RING_BYTES = 1ull << 30;         // pinned staging of submitted bases
 constexpr u64 RESERVE_MIN = 1ull << 30;        // free device memory left to other users (at least)
 constexpr double MEM_POLL_MS = 1.0;            // how often the worker may query free memory
-// A group takes as long as its longest read (Algorithm 3's steps on one read are sequential), so
-// requests with reads of at least LONG_READ bases are grouped apart from the others: a request of
-// short reads never waits for a long read of another request.
+// A group takes as long as its longest chain of steps (long reads are cut, but the steps of one piece stay
+// sequential), so requests with reads of at least LONG_READ bases are grouped apart from the others: a
+// request of short reads never waits for a long read of another request.
 constexpr u64 LONG_READ = 1000;
 constexpr double LONG_SLOT_SHARE = 0.5;
 
