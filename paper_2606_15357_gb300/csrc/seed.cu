@@ -712,8 +712,9 @@ __global__ void __launch_bounds__(BLOCK, BLOCK == 128 ? 6 : 1024 / BLOCK) k_smem
 // What bounds it: latency of the random block reads, then their rate.  The form this replaced (one
 // read per lane, all kinds of step in one loop) had 9.8 active lanes per instruction and cost a read
 // 2,100 warp instructions (1 Gbp, k = 14); this one has 16.5 (19-26 in its block steps) and 1,370.  20M
-// reads of 150 bases there: 59.2 -> 45 ms (with 32-byte L2 fetches 54.5 -> 37.3), 36 -> 47 G random
-// sectors/s, the rate the random-read probe reaches; 2M reads on a 100 Mbp index 5.17 -> 2.6 ms.  More reads in flight help
+// reads of 150 bases there: 54.5 -> 37.3 ms (331M hits; another genome, 605M hits: 59.2 -> 45), 36 -> 52 G
+// DRAM sectors/s with the sequential ones, the rate the random-read probe reaches; 2M reads on a 100
+// Mbp index 5.17 -> 2.6 ms.  More reads in flight help
 // (32 slots per warp instead of 64: 20% slower; 24 warps per SM instead of 32: 6%), so the table takes
 // the shared memory it can get: 64 slots x 32 warps x 89 bytes.  A lone read (a small batch's tail)
 // advances one extension per 0.7 us.
