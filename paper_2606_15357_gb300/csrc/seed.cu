@@ -2337,15 +2337,23 @@ int locate_shared(const DevIndex &I, const mb_smem *sm, u64 cap, const u64 *nsm_
     return MB_OK;
 }
 
+// The index with the samples at which a hit's own walk ends: its own where they hold every row or every
+// second one, else the rate-4 ones.  k_locate_direct reads the rate as a power of two, which 1, 2 and 4 are;
+// locate_is_direct lets no index in that would be left with another.
+DevIndex dense_samples(const DevIndex &I) {
+    DevIndex L = I;
+    if (I.sa_aux && I.r > 2) {
+        L.ssa = I.sa_aux;
+        L.r = AUX_RATE;
+    }
+    return L;
+}
+
 // The hits of records sm[0, min(cap, *nsm_dev)) by k_locate_direct (*D.n and *err zero before).
 int locate_direct(const DevIndex &I, const mb_smem *sm, u64 cap, const u64 *nsm_dev, const u32 *known, u32 *hits,
                   u64 hits_cap, const DirectBufs &D, u32 *err, cudaStream_t st) {
     if (cap == 0) return MB_OK;
-    DevIndex L = I;
-    if (I.sa_aux && I.r > AUX_RATE) {   // the denser samples
-        L.ssa = I.sa_aux;
-        L.r = AUX_RATE;
-    }
+    const DevIndex L = dense_samples(I);
     const unsigned g = resident_grid((const void *)k_locate_direct<false>, 256, cap);
     k_locate_direct<false><<<g, 256, 0, st>>>(L, sm, cap, nsm_dev, known, hits, hits_cap, D, err);
     MB_KCHECK();

@@ -1,0 +1,76 @@
+"""Calls on a nearly full device: an allocation that is refused gives its error (or, for the optional
+deeper k-mer table, none), and nothing of it is left for the next call to find."""
+import ctypes
+
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+MB = 1 << 20
+
+
+@pytest.fixture(scope="module")
+def mb():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_2606_15357_gb300 as m
+    m.lib()
+    return m
+
+
+@pytest.fixture(scope="module")
+def tiny(mb):
+    ref, rd, _ = synth.workload(1, scale=0.01)
+    G = mb.mb_index_build(ref)
+    return ref, rd, G, mb.seed(G, rd.seq, rd.off)
+
+
+def still_works(mb, tiny):
+    _, rd, G, want = tiny
+    sm, hits = mb.seed(G, rd.seq, rd.off)
+    assert sm.tobytes() == want[0].tobytes() and np.array_equal(hits, want[1])
+
+
+def leave(mb, tiny, room):
+    """The rest of the device taken but for `room` bytes; the library's pool given back first."""
+    mb.mb_index_build(tiny[0][:1000], opts=dict(kmer_k=4))   # a build ends by trimming the pool
+    torch.cuda.empty_cache()
+    free, _ = torch.cuda.mem_get_info()
+    return torch.empty(free - room, dtype=torch.uint8, device="cuda")
+
+
+def test_a_refused_call_leaves_no_error_behind(mb, tiny):
+    _, rd, G, _ = tiny
+    sm = np.zeros(1, dtype=mb.SMEM_DTYPE)
+    sm["s"] = 1 << 38   # a terabyte of hits, staged on the device for a host array
+    hits, nh, o = np.zeros(4, np.uint32), ctypes.c_uint64(), mb.Opts(max_occ=1)
+    rc = mb.lib().mb_locate(G.handle, mb._ptr(sm), 1, ctypes.byref(o), None, mb._ptr(hits), 1 << 40, ctypes.byref(nh))
+    assert rc == -2 and nh.value == 1 << 38
+    still_works(mb, tiny)
+
+
+def test_load_with_little_room(mb, tiny, tmp_path):
+    """20 Mbp at k = 4: 115 MB of index, a deeper table of 201 MB and 63 MB to make it with.  At every room
+    the load succeeds from the index's own size on, and calls after it (or after its refusal) work."""
+    ref = np.random.default_rng(3).integers(0, 4, 20_000_000).astype(np.uint8)
+    G = mb.mb_index_build(ref, opts=dict(kmer_k=4))
+    G.save(str(tmp_path / "i.mbi"))
+    G.free()
+    loaded = []
+    for room in range(64 * MB, 480 * MB, 24 * MB):
+        rest = leave(mb, tiny, room)
+        try:
+            X, rc = mb.mb_index_load(str(tmp_path / "i.mbi")), 0
+        except mb.MbError as e:
+            X, rc = None, e.code
+        del rest
+        torch.cuda.empty_cache()
+        still_works(mb, tiny)
+        if X is not None:
+            X.free()
+        assert rc in (0, -2)
+        loaded.append(rc == 0)
+    assert loaded[-1] and not loaded[0] and loaded == sorted(loaded)

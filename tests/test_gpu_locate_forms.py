@@ -97,3 +97,30 @@ def test_many_hits_share_their_walks(mb, small):
         out.zero_()
         mb.mb_locate(G, dsm, len(sm), opts=dict(flags=flags), hits=out, cap=len(rows))
         assert torch.equal(out, want)
+
+
+@pytest.mark.parametrize("rate", [1, 2, 3, 4, 5, 6, 7, 12, 33])
+@pytest.mark.parametrize("aux", [True, False])
+def test_every_rate_dropped_and_loaded(mb, small, tmp_path, rate, aux):
+    """Sample rates on both sides of the rate-4 samples, powers of two and not, without the full array:
+    after it was dropped, and on an index read back from its file (which never has it); mb_locate, a plan
+    and the pipelined call."""
+    ref, rd, S = small
+    G = mb.mb_index_build(ref, opts=dict(sa_rate=rate, flags=0 if aux else mb.MB_NO_AUX))
+    G.save(str(tmp_path / "i.mbi"))
+    G.drop_sa()
+    r = np.random.default_rng(rate)
+    sm, rows = records(mb, G.n, np.concatenate([r.integers(0, 40, 400), [5000, 1]]), rate)
+    want_sm, _, _ = mb.mb_seed_batch(G, rd.seq, rd.off)
+    cnt = np.where(want_sm["flags"] & mb.MB_SMEM_OVER_MAX_OCC, 0, want_sm["s"]).astype(np.int64)
+    want = S[np.concatenate([np.arange(int(k), int(k) + int(c)) for k, c in zip(want_sm["k"], cnt)])]
+    seq, off = torch.from_numpy(rd.seq).cuda(), torch.from_numpy(rd.off.view(np.int64)).cuda()
+    for X in (G, mb.mb_index_load(str(tmp_path / "i.mbi"))):
+        hits, nh = mb.mb_locate(X, sm, len(sm), cap=len(rows))
+        assert nh == len(rows) and np.array_equal(hits, S[rows])
+        P = mb.Plan(X, rd.n, len(rd.seq), len(want_sm) + 8, len(want) + 8)
+        P.run(seq, off)
+        psm, phits = P.result()
+        assert psm.tobytes() == want_sm.tobytes() and np.array_equal(phits, want)
+        lsm, lhits = mb.seed_locate(X, rd.seq, rd.off)
+        assert lsm.tobytes() == want_sm.tobytes() and np.array_equal(lhits, want)
