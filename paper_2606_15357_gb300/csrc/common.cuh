@@ -10,11 +10,14 @@ typedef uint32_t u32;
 typedef uint8_t u8;
 
 // ----------------------------------------------------------------------------- error plumbing
+// A CUDA error that a call has reported (or, for memory it can do without, passed over) is taken out of
+// the runtime's last error: the launch checks of a later call would find it there and fail for it.
 void mb_set_error(const char *fmt, ...);
 #define MB_CK(call)                                                                           \
     do {                                                                                      \
         cudaError_t e_ = (call);                                                              \
         if (e_ != cudaSuccess) {                                                              \
+            cudaGetLastError();                                                               \
             mb_set_error("%s:%d %s: %s", __FILE__, __LINE__, #call, cudaGetErrorString(e_));  \
             return e_ == cudaErrorMemoryAllocation ? MB_ERR_NOMEM : MB_ERR_CUDA;              \
         }                                                                                     \
@@ -47,6 +50,7 @@ struct DevBuf {
         cudaError_t e = cudaMallocAsync(&p, b, s);
         if (e != cudaSuccess) {
             p = nullptr;
+            cudaGetLastError();
             mb_set_error("cudaMallocAsync(%zu): %s", b, cudaGetErrorString(e));
             return e == cudaErrorMemoryAllocation ? MB_ERR_NOMEM : MB_ERR_CUDA;
         }

@@ -491,6 +491,7 @@ int mb_stage_in(const void *src, size_t bytes, cudaStream_t st, DevBuf &buf, con
 
 static void free_index(mb_index *x) {
     if (!x) return;
+    cudaGetLastError();   // of a build or load that ends here
     if (x->occ) cudaFree(x->occ);
     if (x->ssa) cudaFree(x->ssa);
     if (x->kmer) cudaFree(x->kmer);

@@ -3129,7 +3129,10 @@ extern "C" int mb_plan_capture(mb_plan *P, const uint8_t *seq, const uint64_t *o
         else if (g) cudaGraphDestroy(g);
     }
     cudaStreamDestroy(s);
-    if (rc != MB_OK) mb_set_error("mb_plan_capture: graph capture failed");
+    if (rc != MB_OK) {
+        cudaGetLastError();
+        mb_set_error("mb_plan_capture: graph capture failed");
+    }
     return rc;
 }
 

@@ -23,33 +23,36 @@ def mb():
 
 @pytest.fixture(scope="module")
 def tiny(mb):
-    ref, rd, _ = synth.workload(1, scale=0.01)
-    G = mb.mb_index_build(ref)
-    return ref, rd, G, mb.seed(G, rd.seq, rd.off)
+    """A small index with one record and its hits on the device."""
+    ref, _, _ = synth.workload(1, scale=0.01)
+    sm = np.zeros(1, dtype=mb.SMEM_DTYPE)
+    sm["qend"], sm["s"] = 20, 100
+    return dict(ref=ref, G=mb.mb_index_build(ref), sm=torch.from_numpy(sm.view(np.uint8)).cuda(),
+                hits=torch.zeros(100, dtype=torch.int32, device="cuda"),
+                keep=torch.zeros(100, dtype=torch.uint8, device="cuda"))
 
 
-def still_works(mb, tiny):
-    _, rd, G, want = tiny
-    sm, hits = mb.seed(G, rd.seq, rd.off)
-    assert sm.tobytes() == want[0].tobytes() and np.array_equal(hits, want[1])
+def next_call(mb, t):
+    """The call that follows: one kernel, no allocation, and nothing that would drop an earlier error."""
+    return mb.lib().mb_bs_filter(t["G"].handle, mb._ptr(t["sm"]), 1, None, mb._ptr(t["hits"]), 100, None,
+                                 mb._ptr(t["keep"]))
 
 
 def leave(mb, tiny, room):
     """The rest of the device taken but for `room` bytes; the library's pool given back first."""
-    mb.mb_index_build(tiny[0][:1000], opts=dict(kmer_k=4))   # a build ends by trimming the pool
+    mb.mb_index_build(tiny["ref"][:1000], opts=dict(kmer_k=4))   # a build ends by trimming the pool
     torch.cuda.empty_cache()
     free, _ = torch.cuda.mem_get_info()
     return torch.empty(free - room, dtype=torch.uint8, device="cuda")
 
 
 def test_a_refused_call_leaves_no_error_behind(mb, tiny):
-    _, rd, G, _ = tiny
     sm = np.zeros(1, dtype=mb.SMEM_DTYPE)
     sm["s"] = 1 << 38   # a terabyte of hits, staged on the device for a host array
     hits, nh, o = np.zeros(4, np.uint32), ctypes.c_uint64(), mb.Opts(max_occ=1)
-    rc = mb.lib().mb_locate(G.handle, mb._ptr(sm), 1, ctypes.byref(o), None, mb._ptr(hits), 1 << 40, ctypes.byref(nh))
-    assert rc == -2 and nh.value == 1 << 38
-    still_works(mb, tiny)
+    rc = mb.lib().mb_locate(tiny["G"].handle, mb._ptr(sm), 1, ctypes.byref(o), None, mb._ptr(hits), 1 << 40, ctypes.byref(nh))
+    after = next_call(mb, tiny)
+    assert rc == -2 and nh.value == 1 << 38 and after == 0 and bool(tiny["keep"].all())
 
 
 def test_load_with_little_room(mb, tiny, tmp_path):
@@ -66,11 +69,11 @@ def test_load_with_little_room(mb, tiny, tmp_path):
             X, rc = mb.mb_index_load(str(tmp_path / "i.mbi")), 0
         except mb.MbError as e:
             X, rc = None, e.code
-        del rest
-        torch.cuda.empty_cache()
-        still_works(mb, tiny)
+        after = next_call(mb, tiny)
+        assert rc in (0, -2) and after == 0, (room, rc, after)
         if X is not None:
             X.free()
-        assert rc in (0, -2)
+        del rest
+        torch.cuda.empty_cache()
         loaded.append(rc == 0)
     assert loaded[-1] and not loaded[0] and loaded == sorted(loaded)
