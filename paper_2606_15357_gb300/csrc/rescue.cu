@@ -297,6 +297,7 @@ extern "C" int mb_rescue_prefilter(const uint8_t *reads, const uint64_t *read_of
     MB_TRY(mb_stage_in(read_off, ((size_t)n_pairs + 1) * 8, st, bro, &dro));
     MB_TRY(mb_stage_in(win_off, ((size_t)n_pairs + 1) * 8, st, bwo, &dwo));
     if (!rdev && !wdev) {
+        MB_CK(cudaStreamSynchronize(st));   // what the stream still writes there: the staged copies have it
         for (u32 p = 0; p < n_pairs && bad == n_pairs; ++p) {
             if (read_off[p + 1] < read_off[p] || win_off[p + 1] < win_off[p]) bad = p;
             else {

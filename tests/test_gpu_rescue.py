@@ -105,3 +105,27 @@ def test_decreasing_offsets_are_refused(mb):
             with pytest.raises(mb.MbError) as e:
                 mb.mb_rescue_prefilter(f(r), f(ro), f(w), f(wins))
             assert e.value.code == -1 and b"decrease" in mb.lib().mb_last_error()
+
+
+def test_host_offsets_that_the_stream_still_writes(mb):
+    """Pinned offsets that hold a small batch's values until earlier work of the call's stream replaces them:
+    the sizes of the launch are those of the new values."""
+    rng = np.random.default_rng(8)
+    lens, wlens = rng.integers(100, 251, 400), rng.integers(300, 3000, 400)
+    ro, wo = (np.concatenate([[0], np.cumsum(x)]) for x in (lens, wlens))
+    r, w = rng.integers(0, 4, ro[-1]).astype(np.uint8), rng.integers(0, 4, wo[-1]).astype(np.uint8)
+    for p in range(0, 400, 2):   # half of the reads come from their window
+        r[ro[p]:ro[p + 1]] = w[wo[p] + 20:wo[p] + 20 + lens[p]]
+    want = oracle.qmer_diag_max_batch(r, ro.astype(np.uint64), w, wo.astype(np.uint64), 7)
+    new = [torch.from_numpy(x).cuda() for x in (ro, wo)]
+    pinned = [torch.from_numpy(np.arange(401) * k).pin_memory() for k in (8, 16)]
+    dr, dw = dev(r), dev(w)
+    best = torch.empty(400, dtype=torch.int32, device="cuda")
+    st = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(st):
+        torch.cuda._sleep(100_000_000)   # about 50 ms before the new offsets arrive
+        for a, b in zip(pinned, new):
+            a.copy_(b, non_blocking=True)
+        mb.mb_rescue_prefilter(dr, pinned[0], dw, pinned[1], best=best, stream=st.cuda_stream)
+    assert np.array_equal(best.cpu().numpy().view(np.uint32), want)
