@@ -172,6 +172,8 @@ extern "C" int mb_seed_locate(const mb_index *idx, const uint8_t *seq, const uin
         MB_CK(cudaMemcpyAsync(hoff_copy.data(), off, hoff_copy.size() * 8, cudaMemcpyDeviceToHost, ust));
         MB_CK(cudaStreamSynchronize(ust));
         hoff = hoff_copy.data();
+    } else {
+        MB_CK(cudaStreamSynchronize(ust));   // what the stream still writes there: the chunks are cut by it
     }
     if (hoff[n_reads] < hoff[0]) {
         mb_set_error("mb_seed_locate: offsets decrease");

@@ -215,3 +215,23 @@ def test_edge_reads_and_empty_batch(mb):
         check_oracle(sm, hits, oracle.Index(ref), seq, off)
     sm, hits = mb.seed_locate(G, seq, off[:1])
     assert len(sm) == 0 and len(hits) == 0
+
+
+def test_host_offsets_that_the_stream_still_writes(mb, repeat_rich):
+    """Pinned offsets that hold shorter reads' values until earlier work of the call's stream replaces them:
+    chunks and buffers are sized by the new values."""
+    ref, rd, G = repeat_rich
+    want_sm, want_hits = mb.seed(G, rd.seq, rd.off)
+    seq = torch.from_numpy(rd.seq).pin_memory()
+    off = torch.arange(rd.n + 1, dtype=torch.int64).pin_memory()
+    new = dev(rd.off)
+    out, hits = np.zeros(len(want_sm), mb.SMEM_DTYPE), np.zeros(len(want_hits), np.uint32)
+    st = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(st):
+        torch.cuda._sleep(100_000_000)   # about 50 ms before the new offsets arrive
+        off.copy_(new, non_blocking=True)
+        m, nh = mb.seed_locate(G, seq, off, opts=dict(chunk_reads=4096), stream=st.cuda_stream, out=out, cap=len(out),
+                               hits=hits, hits_cap=len(hits))
+    assert (m, nh) == (len(want_sm), len(want_hits))
+    assert out.tobytes() == want_sm.tobytes() and np.array_equal(hits, want_hits)
