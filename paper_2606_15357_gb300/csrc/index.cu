@@ -725,7 +725,6 @@ extern "C" int mb_index_build(const uint8_t *ref, uint64_t len, const mb_opts *o
         if (cudaMalloc(&X->kmer, nk * 12) != cudaSuccess) { rc = MB_ERR_NOMEM; break; }
         k_kmer_table<<<grid_for(nk, 256), 256, 0, st>>>(mb_dev_index(X), kk, X->kmer);
         if (cudaGetLastError() != cudaSuccess) { rc = MB_ERR_CUDA; break; }
-        if ((rc = build_kmer2(X, st)) != MB_OK) break;
         if (!(flags & MB_NO_AUX)) {
             // dense SA / ISA samples for extending unique matches by comparison
             const u64 na = aux_count(n);
@@ -737,8 +736,9 @@ extern "C" int mb_index_build(const uint8_t *ref, uint64_t len, const mb_opts *o
             k_sample_isa<<<grid_for(na, 256), 256, 0, st>>>(brank.as<u32>(), n, AUX_RATE, X->isa_aux);
             if (cudaGetLastError() != cudaSuccess) { rc = MB_ERR_CUDA; break; }
         }
-        if (cudaStreamSynchronize(st) != cudaSuccess) { rc = MB_ERR_CUDA; break; }
         if ((rc = make_sa_ref(X)) != MB_OK) break;
+        if ((rc = build_kmer2(X, st)) != MB_OK) break;   // last: it may take only what all others leave
+        if (cudaStreamSynchronize(st) != cudaSuccess) { rc = MB_ERR_CUDA; break; }
     } while (0);
     {
         // give the build's temporaries (tens of GB at 1 Gbp) back to the device
@@ -1005,15 +1005,15 @@ extern "C" int mb_index_load(const char *path, void *stream, mb_index **out) {
         mb_set_error("mb_index_load: copy to device failed");
         return MB_ERR_CUDA;
     }
-    if (build_kmer2(X, st) != MB_OK || cudaStreamSynchronize(st) != cudaSuccess) {
-        free_index(X);
-        mb_set_error("mb_index_load: building the deeper k-mer table failed");
-        return MB_ERR_CUDA;
-    }
     if (make_sa_ref(X) != MB_OK) {
         free_index(X);
         mb_set_error("mb_index_load: device allocation failed");
         return MB_ERR_NOMEM;
+    }
+    if (build_kmer2(X, st) != MB_OK || cudaStreamSynchronize(st) != cudaSuccess) {
+        free_index(X);
+        mb_set_error("mb_index_load: building the deeper k-mer table failed");
+        return MB_ERR_CUDA;
     }
     *out = X;
     return MB_OK;

@@ -77,3 +77,22 @@ def test_load_with_little_room(mb, tiny, tmp_path):
         torch.cuda.empty_cache()
         loaded.append(rc == 0)
     assert loaded[-1] and not loaded[0] and loaded == sorted(loaded)
+
+
+def test_more_room_never_builds_less(mb, tiny):
+    """The optional table takes no array's room: from the smallest room in which a build succeeds on, every
+    larger one does too."""
+    ref = np.random.default_rng(4).integers(0, 4, 20_000_000).astype(np.uint8)
+    built = []
+    for room in range(1000 * MB, 1660 * MB, 60 * MB):
+        rest = leave(mb, tiny, room)
+        try:
+            mb.mb_index_build(ref, opts=dict(kmer_k=4)).free()
+            rc = 0
+        except mb.MbError as e:
+            rc = e.code
+        assert next_call(mb, tiny) == 0 and rc in (0, -2)
+        del rest
+        torch.cuda.empty_cache()
+        built.append(rc == 0)
+    assert built[-1] and not built[0] and built == sorted(built)
