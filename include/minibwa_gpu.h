@@ -56,7 +56,8 @@ enum {
                               or walk and the call returns MB_ERR_DEVICE_CHECK.  Without the flag the kernels still check every
                               read's offsets and every record's rows (MB_ERR_DEVICE_CHECK), and the
                               host checks every device buffer against its allocation (MB_ERR_ARG) */
-#define MB_NO_KMER  0x8u   /* seeding: do not use the k-mer ds-interval table */
+#define MB_NO_KMER  0x8u   /* seeding: do not use the k-mer ds-interval table; index: without the deeper
+                              table that kmer_k describes (nor when loaded from its file) */
 #define MB_COUNT    0x10u  /* seeding/locate: also count the work done (mb_work_counters) */
 #define MB_NO_AUX   0x20u  /* index: build without the packed text and the rate-4 SA / ISA samples
                               (2.25 bytes per text position) that let seeding extend unique matches
@@ -96,7 +97,8 @@ typedef struct {
                                  the table takes 12 * 4^k bytes (3.2 GB at k = 14, 51.5 GB at
                                  k = 16).  Where 4^(k+1) <= n / 2 the index keeps a deeper table
                                  beside it for seeding, of 1.5 to 6 bytes per text position, if the
-                                 device has room (built with the index, also on load; not in files) */
+                                 device has room (built with the index, also on load; not in files;
+                                 MB_NO_KMER declines it) */
     uint32_t flags;           /* MB_* flags above */
     uint32_t chunk_reads;     /* mb_seed_locate: reads per pipelined chunk (0 = 2^22; with host
                                  inputs the first chunk is a quarter of the others) */
@@ -122,7 +124,7 @@ typedef struct {
  *   ref      host or device, `len` base codes; codes > 3 (ambiguous) are replaced by
  *            random bases: bits 63..62 of splitmix64's output function of
  *            (n_seed + (pos+1) * 0x9E3779B97F4A7C15)  (Section 2.1, "random bases").
- *   opts     sa_rate, kmer_k, flags & MB_BS3 are used.
+ *   opts     sa_rate, kmer_k and flags & (MB_BS3 | MB_NO_AUX | MB_NO_KMER) are used.
  *   stream   stream for the build.
  *   out      receives the new index (free with mb_index_free).
  * Builds T, its suffix array by prefix doubling, the BWT in occurrence blocks (Section 2.2;

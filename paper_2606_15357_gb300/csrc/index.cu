@@ -516,6 +516,7 @@ static int make_sa_ref(mb_index *x) {
 // 1.5 to 6 bytes per text position; without room for it seeding uses the index's own.  2M reads on
 // 100 Mbp (k = 10 -> 13), seeded and located: 3.36 -> 3.10 ms.
 static int build_kmer2(mb_index *x, cudaStream_t st) {
+    if (x->flags & MB_NO_KMER) return MB_OK;   // declined at the build (kept in the file's flags)
     u32 k = x->kmer_k;
     while (k < 16 && (1ULL << (2 * k + 2)) <= x->n / 2) ++k;
     if (k == x->kmer_k) return MB_OK;
@@ -661,7 +662,7 @@ extern "C" int mb_index_build(const uint8_t *ref, uint64_t len, const mb_opts *o
     X->rlen = M;
     X->sa_rate = r;
     X->kmer_k = kk;
-    X->flags = flags & MB_BS3;
+    X->flags = flags & (MB_BS3 | MB_NO_KMER);
     cudaGetDevice(&X->device);
     int rc = MB_OK;
     do {

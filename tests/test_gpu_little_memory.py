@@ -96,3 +96,28 @@ def test_more_room_never_builds_less(mb, tiny):
         torch.cuda.empty_cache()
         built.append(rc == 0)
     assert built[-1] and not built[0] and built == sorted(built)
+
+
+def test_the_deeper_table_can_be_declined(mb, tiny, tmp_path):
+    """MB_NO_KMER at the build: 201 MB less at 20 Mbp and k = 4, also after a load; the same records."""
+    ref = np.random.default_rng(5).integers(0, 4, 20_000_000).astype(np.uint8)
+    rd = synth.reads(ref, 2000, 6, mode=1, read_len=150, sub_lo=0.001, sub_hi=0.01, indel=0.0001)
+    used, recs = [], []
+    for flags in (0, mb.MB_NO_KMER):
+        for load in (False, True):
+            torch.cuda.empty_cache()
+            before = torch.cuda.mem_get_info()[0]
+            if load:
+                G = mb.mb_index_load(str(tmp_path / f"{flags}.mbi"))
+            else:
+                G = mb.mb_index_build(ref, opts=dict(kmer_k=4, flags=flags))
+                G.save(str(tmp_path / f"{flags}.mbi"))
+                G.drop_sa()
+            mb.mb_index_build(tiny["ref"][:1000], opts=dict(kmer_k=4)).free()   # trims the pool
+            used.append(before - torch.cuda.mem_get_info()[0])
+            recs.append(mb.mb_seed_batch(G, rd.seq, rd.off)[0].tobytes())
+            G.free()
+            mb.mb_index_build(tiny["ref"][:1000], opts=dict(kmer_k=4)).free()
+    table = 12 * 4 ** 12
+    assert abs(used[0] - used[2] - table) < 8 * MB and abs(used[1] - used[3] - table) < 8 * MB
+    assert len(set(recs)) == 1
