@@ -455,9 +455,11 @@ int mb_set_l2_fetch_granularity(int bytes, int *now);
 int mb_device_extent(const void *p, uint64_t *base, uint64_t *size);
 /* L2 persistence for the k-mer ds-interval table (Section 2.5 keeps it in a CPU cache): sets an
  * access-policy window on `stream` over the first min(max_bytes, table bytes, the device's window
- * and persisting-L2 limits) bytes of the table, hits persisting, and sets this context's
- * persisting-L2 limit to that size (*window receives it).  Kernels later launched on `stream`
- * keep those table lines in L2.  max_bytes = 0 removes the window and resets persisting lines.
+ * and persisting-L2 limits) bytes of the table that seeding reads (the deeper one where the index has
+ * it), hits persisting, and sets this context's persisting-L2 limit to that size (*window receives it).
+ * Kernels later launched on `stream` keep those table lines in L2.  max_bytes = 0 removes the window and
+ * resets persisting lines.  Seeding with min_len below the deeper table's k, MB_SMEM_ONE_LOOP or MB_COUNT
+ * reads the table of kmer_k, outside the window.
  * Like mb_set_l2_fetch_granularity this changes only the calling process's context.  No
  * counterpart in the paper. */
 int mb_index_l2_persist(const mb_index *idx, void *stream, uint64_t max_bytes, uint64_t *window);

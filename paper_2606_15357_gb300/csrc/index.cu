@@ -1056,12 +1056,12 @@ extern "C" int mb_index_l2_persist(const mb_index *idx, void *stream, uint64_t m
         int max_win = 0, max_persist = 0;
         MB_CK(cudaDeviceGetAttribute(&max_win, cudaDevAttrMaxAccessPolicyWindowSize, dev));
         MB_CK(cudaDeviceGetAttribute(&max_persist, cudaDevAttrMaxPersistingL2CacheSize, dev));
-        w = (1ULL << (2 * idx->kmer_k)) * 12;
+        w = (1ULL << (2 * (idx->kmer2 ? idx->kmer2_k : idx->kmer_k))) * 12;
         if (w > max_bytes) w = max_bytes;
         if (w > (u64)max_win) w = (u64)max_win;
         if (w > (u64)max_persist) w = (u64)max_persist;
         MB_CK(cudaDeviceSetLimit(cudaLimitPersistingL2CacheSize, (size_t)w));
-        v.accessPolicyWindow.base_ptr = idx->kmer;
+        v.accessPolicyWindow.base_ptr = idx->kmer2 ? idx->kmer2 : idx->kmer;   // the one the SMEM kernel reads
         v.accessPolicyWindow.num_bytes = (size_t)w;
         v.accessPolicyWindow.hitRatio = 1.0f;
         v.accessPolicyWindow.hitProp = cudaAccessPropertyPersisting;
