@@ -2273,6 +2273,18 @@ size_t share_tmp_bytes(u64 cap, u64 rows_cap) {
 // bytes of the per-record arrays (keys, keys_alt, roff: u64; vals, vals_alt, pmax, last: u32)
 constexpr size_t SHARE_BYTES_PER_RECORD = 3 * 8 + 4 * 4;
 
+// The index with the samples that short walks end at: its own where they hold every row or every second
+// one, else the rate-4 ones.  k_locate_direct reads the rate as a power of two, which 1, 2 and 4 are;
+// locate_is_direct lets no index in that would be left with another.
+DevIndex dense_samples(const DevIndex &I) {
+    DevIndex L = I;
+    if (I.sa_aux && I.r > 2) {
+        L.ssa = I.sa_aux;
+        L.r = AUX_RATE;
+    }
+    return L;
+}
+
 // Locate of the records sm[0, nsm), nsm = min(cap, *nsm_dev): every hit of every record without
 // MB_SMEM_OVER_MAX_OCC, written at the record's hit offset (hits_cap bounds every write).  Each
 // distinct row is walked once (see the shared-walk kernels); kt, when given, times the walks.
@@ -2324,8 +2336,15 @@ int locate_shared(const DevIndex &I, const mb_smem *sm, u64 cap, const u64 *nsm_
     } else {
         DevIndex L = I;
         if (aux) {   // short walks to the rate-4 samples: four per lane at least (2: 20% slower)
-            L.ssa = I.sa_aux;
-            L.r = AUX_RATE;
+            // (a walk takes 3 steps on average to a row of rate 4, 1 or none at rates 2 and 1, so there the
+            // index's own: 40M distinct rows 0.96 ms at rate 4, 0.45 and 0.15; MB_COUNT counts the walks that
+            // its flags name)
+            if (count) {
+                L.ssa = I.sa_aux;
+                L.r = AUX_RATE;
+            } else {
+                L = dense_samples(I);
+            }
             if (depth < 4) depth = 4;
         }
         if (kt) kt->start();
@@ -2335,18 +2354,6 @@ int locate_shared(const DevIndex &I, const mb_smem *sm, u64 cap, const u64 *nsm_
     k_share_copy<<<G, 256, 0, st>>>(b.keys, ss, sho, b.last, b.roff, cap, b.nwalk, b.rpos, hits_cap, hits, hits_cap);
     MB_KCHECK();
     return MB_OK;
-}
-
-// The index with the samples at which a hit's own walk ends: its own where they hold every row or every
-// second one, else the rate-4 ones.  k_locate_direct reads the rate as a power of two, which 1, 2 and 4 are;
-// locate_is_direct lets no index in that would be left with another.
-DevIndex dense_samples(const DevIndex &I) {
-    DevIndex L = I;
-    if (I.sa_aux && I.r > 2) {
-        L.ssa = I.sa_aux;
-        L.r = AUX_RATE;
-    }
-    return L;
 }
 
 // The hits of records sm[0, min(cap, *nsm_dev)) by k_locate_direct (*D.n and *err zero before).

@@ -124,3 +124,43 @@ def test_every_rate_dropped_and_loaded(mb, small, tmp_path, rate, aux):
         assert psm.tobytes() == want_sm.tobytes() and np.array_equal(phits, want)
         lsm, lhits = mb.seed_locate(X, rd.seq, rd.off)
         assert lsm.tobytes() == want_sm.tobytes() and np.array_equal(lhits, want)
+
+
+@pytest.mark.parametrize("rate", [1, 2, 3, 4])
+def test_many_hits_at_dense_rates(mb, small, rate):
+    """More than 2^25 hits without the full array where the index's own samples are as dense as the rate-4
+    ones or denser, or not a power of two apart."""
+    ref, rd, S = small
+    G = mb.mb_index_build(ref, opts=dict(sa_rate=rate))
+    G.drop_sa()
+    sm, rows = records(mb, G.n, np.full(110, 400_000), rate)
+    assert len(rows) > 1 << 25
+    dsm = torch.from_numpy(sm.view(np.uint8)).cuda()
+    out = torch.empty(len(rows), dtype=torch.int32, device="cuda")
+    want = torch.from_numpy(S.astype(np.int32)).cuda()[torch.from_numpy(rows).cuda()]
+    for flags in (0, mb.MB_LOCATE_AUX, mb.MB_LOCATE_JOIN, mb.MB_CHECKED, mb.MB_COUNT, mb.MB_COUNT | mb.MB_LOCATE_AUX):
+        out.zero_()
+        mb.mb_locate(G, dsm, len(sm), opts=dict(flags=flags), hits=out, cap=len(rows))
+        assert torch.equal(out, want), flags
+
+
+def test_dense_own_samples_end_the_walks(mb):
+    """36M distinct rows without the full array: with every row sampled no walk takes a step (0.15 ms; 0.96 ms
+    to the rate-4 samples), so the walks take well under those of an index that has only the latter."""
+    ref = np.random.default_rng(2).integers(0, 4, 40_000_000).astype(np.uint8)
+    sm = np.zeros(400_000, dtype=mb.SMEM_DTYPE)
+    sm["s"], sm["k"], sm["hit_off"] = 90, np.arange(400_000) * 199, np.arange(400_000) * 90
+    dsm = torch.from_numpy(sm.view(np.uint8)).cuda()
+    out = torch.empty(36_000_000, dtype=torch.int32, device="cuda")
+    ms = {}
+    for rate in (1, 32):
+        G = mb.mb_index_build(ref, opts=dict(sa_rate=rate))
+        G.drop_sa()
+        for _ in range(6):
+            mb.profile_reset()
+            mb.profile_enable(True)
+            mb.mb_locate(G, dsm, len(sm), hits=out, cap=out.numel())
+            mb.profile_enable(False)
+            ms[rate] = min(ms.get(rate, 1e9), mb.profile_get("locate")[0])
+        G.free()
+    assert ms[1] < 0.5 * ms[32], ms
