@@ -2345,7 +2345,8 @@ int locate_shared(const DevIndex &I, const mb_smem *sm, u64 cap, const u64 *nsm_
             } else {
                 L = dense_samples(I);
             }
-            if (depth < 4) depth = 4;
+            // (not where the longer chunks of four walks would pass the queue's 32-bit positions)
+            if (depth < 4 && hits_cap < (1ull << 32) - (1ull << 24)) depth = 4;
         }
         if (kt) kt->start();
         MB_TRY(launch_locate(L, b.rows, hits_cap, b.nrows, b.rpos, b.lq, wc, count, depth, chk, st));

@@ -164,3 +164,22 @@ def test_dense_own_samples_end_the_walks(mb):
             ms[rate] = min(ms.get(rate, 1e9), mb.profile_get("locate")[0])
         G.free()
     assert ms[1] < 0.5 * ms[32], ms
+
+
+def test_hits_up_to_the_walk_queue_limit(mb, small):
+    """4,292M hits, under what one walk per lane can queue (2^32 less a chunk per warp), on a dropped array:
+    4,292 records of the same 1M rows, walked once."""
+    free, _ = torch.cuda.mem_get_info()
+    if free < 80 << 30:
+        pytest.skip("needs 80 GB of device memory")
+    ref, rd, S = small
+    G = mb.mb_index_build(ref)
+    G.drop_sa()
+    n = G.n
+    m = 4_292_300_000 // n
+    sm = np.zeros(m, dtype=mb.SMEM_DTYPE)
+    sm["s"], sm["hit_off"] = n, np.arange(m) * n
+    out = torch.zeros(m * n, dtype=torch.int32, device="cuda")
+    hits, nh = mb.mb_locate(G, torch.from_numpy(sm.view(np.uint8)).cuda(), m, hits=out, cap=m * n)
+    want = torch.from_numpy(S.astype(np.int32)).cuda()
+    assert nh == m * n and all(torch.equal(out[t * n:(t + 1) * n], want) for t in range(m))
