@@ -296,9 +296,9 @@ int mb_seed_locate(const mb_index *idx, const uint8_t *seq, const uint64_t *off,
  * slot form at smem_burst 2/4/8/16 x smem_wait 4/8/16, which no longer differ), with 16 plain locate
  * walks per lane; then, when the best is a slot form, smem_reads_per_warp 1/2/4/8/16; then, with
  * the best SMEM shape, locate walks per lane 1/2/4/8 plain and 1/2/4/8/16 with walks that join
- * (MB_LOCATE_JOIN) (92 points, 87 when the one-loop form wins).  mb_autotune_points does
- * the same and also returns every point tried with its time in ms (up to cap points; *n_points
- * receives the number tried).
+ * (MB_LOCATE_JOIN) (92 points, 87 when the one-loop form wins).  Points that launch the same kernels in the
+ * same form are run once and share their time.  mb_autotune_points does the same and also returns every
+ * point with its time in ms (up to cap points; *n_points receives their number).
  */
 typedef struct mb_plan mb_plan;
 int mb_plan_create(const mb_index *idx, const mb_opts *opts, uint32_t max_reads, uint64_t max_bases,

@@ -3151,15 +3151,35 @@ extern "C" int mb_plan_replay(mb_plan *P, void *stream) {
     return MB_OK;
 }
 
+// What a plan with these options launches, as far as the autotuner varies it: options with equal shapes run
+// the same kernels in the same form.
+struct RunShape {
+    u32 one_loop, queue, block, per_warp, walks;
+    bool operator==(const RunShape &o) const {
+        return one_loop == o.one_loop && queue == o.queue && block == o.block && per_warp == o.per_warp && walks == o.walks;
+    }
+};
+static RunShape run_shape(const DevIndex &I, const mb_opts &o, u64 max_hits) {
+    SmemArgs t{};
+    smem_tuning(&o, t);
+    const u32 fl = plan_flags(&o), depth = o.prefetch_depth ? o.prefetch_depth : 1u;
+    RunShape r{t.one_loop, t.one_loop && (fl & MB_BATCHED) ? 1u : 0u,
+               o.block_size == 128 || o.block_size == 512 ? o.block_size : 256u, t.one_loop ? 0u : t.per_warp, 0u};
+    if (!plan_direct(I, &o, max_hits))   // (hit by hit, no option changes the walks)
+        r.walks = plan_joins(I, &o, max_hits) ? 1024 + depth : (locate_aux(I, fl) && depth < 4 ? 4u : depth);
+    return r;
+}
+
 // Times launch shapes on this batch (all give the same output; tests check that), in stages:
 // (1) the SMEM kernel's shape, over threads per block {128, 256, 512} x work queue off/on x the
 // kernel form (the one-loop form, and the slot form at smem_burst {2, 4, 8, 16} x smem_wait
 // {4, 8, 16}, which no longer differ: programs expect the points), with 16 plain locate walks per
 // lane; (2) for a slot-form winner, reads per warp {1, 2, 4, 8, 16}; (3) with the best
 // SMEM shape, locate walks per lane {1, 2, 4, 8} plain and {1, 2, 4, 8, 16} with walks that join
-// (MB_LOCATE_JOIN).  Each point is the
-// best of two timed runs of mb_plan_run after one untimed run.  Every point tried is written to
-// points / points_ms when given (up to cap; *n_points receives the number tried).
+// (MB_LOCATE_JOIN).  Each point is the best of two timed runs of mb_plan_run after one untimed run; points
+// that launch the same (RunShape) are run once and share the time, so that the choice between them is not
+// noise (of the 92 points 14 differ where locate goes hit by hit).  Every point is written to points /
+// points_ms when given (up to cap; *n_points receives their number).
 static int autotune_impl(const mb_index *idx, const uint8_t *seq, const uint64_t *off, uint32_t n_reads,
                          const mb_opts *opts, cudaStream_t st, mb_opts *best, double *best_ms, mb_opts *points,
                          double *points_ms, uint32_t cap, uint32_t *n_points) {
@@ -3184,22 +3204,30 @@ static int autotune_impl(const mb_index *idx, const uint8_t *seq, const uint64_t
     u32 np = 0;
     double bms = 1e30;
     mb_opts bo = opts ? *opts : mb_opts{};
+    const DevIndex I = mb_dev_index(idx);
+    std::vector<std::pair<RunShape, double>> timed;
     auto time_point = [&](const mb_opts &o) -> int {
-        mb_plan *P = nullptr;
-        int rc = mb_plan_create(idx, &o, n_reads, o1 - o0, n_smem, n_hits, &P);
-        if (rc != MB_OK) return rc;
+        const RunShape shape = run_shape(I, o, n_hits);
         double t_best = 1e30;
-        for (int rep = 0; rep < 3 && rc == MB_OK; ++rep) {
-            cudaEventRecord(a, st);
-            rc = mb_plan_run(P, seq, off, n_reads, nullptr, st);
-            cudaEventRecord(b, st);
-            if (cudaEventSynchronize(b) != cudaSuccess) rc = MB_ERR_CUDA;
-            float ms = 0;
-            cudaEventElapsedTime(&ms, a, b);
-            if (rep > 0 && ms < t_best) t_best = ms;   // the first run warms up
+        for (const auto &t : timed)
+            if (t.first == shape) t_best = t.second;
+        if (t_best == 1e30) {
+            mb_plan *P = nullptr;
+            int rc = mb_plan_create(idx, &o, n_reads, o1 - o0, n_smem, n_hits, &P);
+            if (rc != MB_OK) return rc;
+            for (int rep = 0; rep < 3 && rc == MB_OK; ++rep) {
+                cudaEventRecord(a, st);
+                rc = mb_plan_run(P, seq, off, n_reads, nullptr, st);
+                cudaEventRecord(b, st);
+                if (cudaEventSynchronize(b) != cudaSuccess) rc = MB_ERR_CUDA;
+                float ms = 0;
+                cudaEventElapsedTime(&ms, a, b);
+                if (rep > 0 && ms < t_best) t_best = ms;   // the first run warms up
+            }
+            mb_plan_free(P);
+            if (rc != MB_OK) return rc;
+            timed.push_back({shape, t_best});
         }
-        mb_plan_free(P);
-        if (rc != MB_OK) return rc;
         if (points && np < cap) {
             points[np] = o;
             if (points_ms) points_ms[np] = t_best;

@@ -146,3 +146,24 @@ def test_autotune_picks_a_supported_shape(mb, mixed):
     P.run(dev(rd.seq), dev(rd.off))
     psm, phits = P.result()
     assert psm.tobytes() == sm.tobytes() and np.array_equal(phits, hits)
+
+
+@pytest.mark.parametrize("aux", [True, False])
+def test_autotune_times_equal_runs_once(mb, mixed, aux):
+    """Points that launch the same share one time: slot-form points of one block size and reads per warp
+    (with the same walks), whatever their burst, wait and queue flag; with the rate-4 samples all walk
+    options too, without them each number of walks, plain or joining, has its own."""
+    ref, rd, G, sm, hits = mixed
+    if not aux:
+        G = mb.mb_index_build(dev(ref), opts=dict(flags=mb.MB_NO_AUX))
+    best, ms, grid = mb.autotune(G, dev(rd.seq), dev(rd.off), points=True)
+    slots, other = {}, set()
+    for o, t in grid:
+        if o.flags & mb.MB_SMEM_ONE_LOOP:
+            other.add((o.block_size, o.flags, o.prefetch_depth, t))
+            continue
+        walks = () if aux else (o.prefetch_depth, o.flags & mb.MB_LOCATE_JOIN)
+        slots.setdefault((o.block_size, o.smem_reads_per_warp) + walks, set()).add(t)
+    assert len(grid) in (87, 92) and len(other) >= 6
+    assert all(len(v) == 1 for v in slots.values()), slots
+    assert len(slots) >= 3 and min(t for _, t in grid) == ms
