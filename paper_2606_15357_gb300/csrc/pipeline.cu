@@ -91,11 +91,11 @@ struct Pipeline {
     }
 };
 
-// the options that shape a plan (chunk_reads only sizes the chunks)
+// the options that shape a plan (chunk_reads only sizes the chunks; smem_burst, smem_wait and smem_warps have
+// no effect)
 bool same_plan_opts(const mb_opts &a, const mb_opts &b) {
     return a.min_len == b.min_len && a.min_occ == b.min_occ && a.max_occ == b.max_occ && a.flags == b.flags &&
-           a.prefetch_depth == b.prefetch_depth && a.block_size == b.block_size && a.smem_burst == b.smem_burst &&
-           a.smem_wait == b.smem_wait && a.smem_warps == b.smem_warps &&
+           a.prefetch_depth == b.prefetch_depth && a.block_size == b.block_size &&
            a.smem_reads_per_warp == b.smem_reads_per_warp;
 }
 

@@ -235,3 +235,13 @@ def test_host_offsets_that_the_stream_still_writes(mb, repeat_rich):
                                hits=hits, hits_cap=len(hits))
     assert (m, nh) == (len(want_sm), len(want_hits))
     assert out.tobytes() == want_sm.tobytes() and np.array_equal(hits, want_hits)
+
+
+def test_kept_workspace_serves_options_without_effect(mb, repeat_rich):
+    """A second call that differs only in smem_burst, smem_wait and smem_warps takes the kept workspace."""
+    ref, rd, G = repeat_rich
+    sm, hits = mb.seed_locate(G, rd.seq, rd.off)
+    free = torch.cuda.mem_get_info()[0]
+    sm2, hits2 = mb.seed_locate(G, rd.seq, rd.off, opts=dict(smem_burst=4, smem_wait=16, smem_warps=40))
+    assert torch.cuda.mem_get_info()[0] == free
+    assert sm2.tobytes() == sm.tobytes() and np.array_equal(hits2, hits)
