@@ -86,6 +86,7 @@ struct KTimer {
     const char *name;
     cudaStream_t st;
     cudaEvent_t a = nullptr, b = nullptr;
+    bool timed = false;   // a launch was timed (stop() was reached)
     KTimer(const char *n, cudaStream_t s);
     void start();
     void stop();

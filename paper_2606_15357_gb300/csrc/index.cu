@@ -334,12 +334,12 @@ void KTimer::start() {
     if (a) cudaEventRecord(a, st);
 }
 void KTimer::stop() {
-    if (b) cudaEventRecord(b, st);
+    timed = b && cudaEventRecord(b, st) == cudaSuccess;
 }
 KTimer::~KTimer() {
     if (!a) return;
     float ms = 0;
-    if (cudaEventSynchronize(b) == cudaSuccess && cudaEventElapsedTime(&ms, a, b) == cudaSuccess) {
+    if (timed && cudaEventSynchronize(b) == cudaSuccess && cudaEventElapsedTime(&ms, a, b) == cudaSuccess) {
         std::lock_guard<std::mutex> g(g_err_mu);
         KStat &k = g_kstat[name];
         k.ms += ms;

@@ -2457,7 +2457,7 @@ int mb_seed_device(const mb_index *idx, const u8 *dseq, const u64 *doff, u32 n_r
     const DevIndex I = mb_dev_index(idx);
     const unsigned B = 256;
     const unsigned G = (unsigned)((n_reads + B - 1) / B);
-    KTimer kt("smem", st);   // reported after the stream is synchronized below
+    KTimer kt("smem", st), kt_items("smem", st);   // reported after the stream is synchronized below
     const bool kmer = !(flags & MB_NO_KMER) && l >= I.kmer_k;
     const bool count = (flags & MB_COUNT) != 0;
     SmemArgs sa{I, dseq, doff, n_reads, dmate, bs, l, c, kmer, slots, nslots, counts, ovf, dovf_n, dqhead,
@@ -2480,7 +2480,9 @@ int mb_seed_device(const mb_index *idx, const u8 *dseq, const u64 *doff, u32 n_r
         MB_CK(cudaMemcpyAsync(v, misc, sizeof v, cudaMemcpyDeviceToHost, st));
         MB_CK(cudaStreamSynchronize(st));
         if (!later || pass || (u32)v[8] == 0) break;
+        kt_items.start();
         MB_TRY(launch_items(sa, st));
+        kt_items.stop();
     }
     const u64 total = v[0];
     const u32 err = (u32)v[4], over = (u32)v[2], pooled = (u32)v[9];

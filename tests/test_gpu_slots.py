@@ -80,3 +80,17 @@ def test_long_reads_without_room_to_cut(mb, tandem):
         assert rc == 0 and no.value == m and out.cpu().numpy().tobytes() == want.tobytes()
     osm = X.seed(seq, off, 19, 1, 500)[0]
     assert m == reps * len(osm) and np.array_equal(want["qbeg"][:len(osm)], osm["qbeg"])
+
+
+def test_profile_counts_the_items_of_cut_reads(mb, tandem):
+    """A small batch with cut reads runs the SMEM kernel twice, for the reads and for the items: both are timed;
+    a batch without cut reads runs it once."""
+    ref, seq, off, G, X = tandem
+    short = synth.reads(ref, 50, 3, mode=1, read_len=100)
+    for s, o, launches in ((seq, off, 2), (short.seq, short.off, 1)):
+        mb.profile_reset()
+        mb.profile_enable(True)
+        mb.mb_seed_batch(G, s, o)
+        mb.profile_enable(False)
+        ms, n = mb.profile_get("smem")
+        assert n == launches and ms > 0
