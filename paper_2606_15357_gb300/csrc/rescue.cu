@@ -248,11 +248,13 @@ __global__ void k_pair_sizes(const u64 *__restrict__ roff, const u64 *__restrict
 
 template <int NP>
 int launch_words(const u8 *reads, const u64 *roff, const u8 *wins, const u64 *woff, u32 npairs, u32 q, u64 wmax, int sms,
-                 u32 *best, cudaStream_t st) {
+                 int smem_max, u32 *best, cudaStream_t st) {
     const u32 words = (u32)((wmax + 31) / 32) + NP + 2;
     const size_t smem = 8 * 3 * (size_t)words * 4;
     const void *f = q == 7 ? (const void *)k_qmer_words<NP, true> : (const void *)k_qmer_words<NP, false>;
-    if (smem > 48 * 1024) MB_CK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // (always the device's maximum: the attribute is the kernel's, and another thread's call with smaller windows
+    // must not lower it before this launch)
+    if (smem > 48 * 1024) MB_CK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, 256, smem) != cudaSuccess || per_sm < 1) {
         cudaGetLastError();
@@ -345,7 +347,7 @@ extern "C" int mb_rescue_prefilter(const uint8_t *reads, const uint64_t *read_of
     int warps = (int)std::min<size_t>(8, (size_t)smem_max / per_warp);
     const size_t smem = per_warp * warps;
     if (smem > 48 * 1024)
-        MB_CK(cudaFuncSetAttribute(k_qmer_diag_max, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        MB_CK(cudaFuncSetAttribute(k_qmer_diag_max, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_qmer_diag_max, warps * 32, smem) != cudaSuccess ||
         per_sm < 1) {
@@ -370,11 +372,11 @@ extern "C" int mb_rescue_prefilter(const uint8_t *reads, const uint64_t *read_of
     if (words <= 8 && 8 * 3 * ((wmax + 31) / 32 + 10) * 4 <= (u64)smem_max) {
         const u8 *xr = (const u8 *)dr, *xw = (const u8 *)dw;
         const u64 *xo = (const u64 *)dro, *yo = (const u64 *)dwo;
-        if (words <= 2) MB_TRY(launch_words<2>(xr, xo, xw, yo, n_pairs, q, wmax, sms, db, st));
-        else if (words == 3) MB_TRY(launch_words<3>(xr, xo, xw, yo, n_pairs, q, wmax, sms, db, st));
-        else if (words == 4) MB_TRY(launch_words<4>(xr, xo, xw, yo, n_pairs, q, wmax, sms, db, st));
-        else if (words == 5) MB_TRY(launch_words<5>(xr, xo, xw, yo, n_pairs, q, wmax, sms, db, st));
-        else MB_TRY(launch_words<8>(xr, xo, xw, yo, n_pairs, q, wmax, sms, db, st));
+        if (words <= 2) MB_TRY(launch_words<2>(xr, xo, xw, yo, n_pairs, q, wmax, sms, smem_max, db, st));
+        else if (words == 3) MB_TRY(launch_words<3>(xr, xo, xw, yo, n_pairs, q, wmax, sms, smem_max, db, st));
+        else if (words == 4) MB_TRY(launch_words<4>(xr, xo, xw, yo, n_pairs, q, wmax, sms, smem_max, db, st));
+        else if (words == 5) MB_TRY(launch_words<5>(xr, xo, xw, yo, n_pairs, q, wmax, sms, smem_max, db, st));
+        else MB_TRY(launch_words<8>(xr, xo, xw, yo, n_pairs, q, wmax, sms, smem_max, db, st));
     } else {
         k_qmer_diag_max<<<(unsigned)blocks, warps * 32, smem, st>>>((const u8 *)dr, (const u64 *)dro, (const u8 *)dw,
                                                                     (const u64 *)dwo, n_pairs, q, (u32)slice, db);

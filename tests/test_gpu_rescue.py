@@ -129,3 +129,36 @@ def test_host_offsets_that_the_stream_still_writes(mb):
             a.copy_(b, non_blocking=True)
         mb.mb_rescue_prefilter(dr, pinned[0], dw, pinned[1], best=best, stream=st.cuda_stream)
     assert np.array_equal(best.cpu().numpy().view(np.uint32), want)
+
+
+@pytest.mark.parametrize("m", [100, 300])
+def test_calls_of_several_threads(mb, m):
+    """Threads whose windows need 60 to 210 kB of shared memory per block, each on its own stream (reads in the
+    register form, and past it)."""
+    import threading
+    rng = np.random.default_rng(m)
+    work, errors = [], []
+    for w in (18_000, 30_000, 42_000, 55_000):
+        ro, wo = np.arange(9, dtype=np.uint64) * m, np.arange(9, dtype=np.uint64) * w
+        r, x = rng.integers(0, 4, 8 * m).astype(np.uint8), rng.integers(0, 4, 8 * w).astype(np.uint8)
+        want = torch.from_numpy(oracle.qmer_diag_max_batch(r, ro, x, wo, 7).view(np.int32)).cuda()
+        work.append((dev(r), dev(ro), dev(x), dev(wo), want, torch.cuda.Stream()))
+    torch.cuda.synchronize()
+
+    def calls(r, ro, x, wo, want, st):
+        try:
+            best = torch.empty(8, dtype=torch.int32, device="cuda")
+            for _ in range(150):
+                mb.mb_rescue_prefilter(r, ro, x, wo, best=best, stream=st.cuda_stream)
+                st.synchronize()
+            with torch.cuda.stream(st):
+                assert torch.equal(best, want)
+        except Exception as e:   # noqa: BLE001 - reported by the test
+            errors.append(e)
+
+    threads = [threading.Thread(target=calls, args=a) for a in work]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
