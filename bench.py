@@ -6,8 +6,9 @@ batch of reads.  Default workload: 1 Gbp repeat-rich synthetic reference (45% re
 0.5% N runs) and 10M 2x150 bp pairs (20M reads), min_len 19, max_occ 500, SA rate 32.
 The index build is timed separately and is not part of the step.
 
-Prints one JSON line.  `--impl reference` times the CPU oracle (the plain reference
-implementation of the same stage) on the host cores instead.
+Prints one JSON line of a few kilobytes on stdout (short_line); the whole report, with the autotuner's
+grid and every form's details, goes to stderr as another.  `--impl reference` times the CPU oracle
+(the plain reference implementation of the same stage) on the host cores instead.
 """
 from __future__ import annotations
 
@@ -740,6 +741,45 @@ def bench_bisulfite(mb, torch, dev, ref, opts, reps: int = 3):
     return res
 
 
+# --------------------------------------------------------------------------------- report
+SHORT_MAX = 3800   # bytes of the line on stdout: readers that keep the end of a log keep all of it
+SHORT_KEYS = {     # of the report's parts, what the line on stdout keeps
+    "roofline": ("bound", "kernel", "achieved", "peak", "unit", "frac", "peak_kind", "traffic", "dram_GBps",
+                 "random_read_ceiling_GBps", "frac_of_random_read_ceiling", "frac_of_random_read_ceiling_basis"),
+    "cpu_baseline": ("value", "unit", "cores", "kind", "sample"),
+    "e2e": ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "call", "identical_output"),
+    "batched": ("reads", "plain_ms", "batched_ms", "speedup", "identical_output"),
+    "rescue_prefilter": ("pairs_per_s", "kernel_ms"),
+    "served": ("requests", "capacity_requests_per_s", "capacity_reads_per_s", "offered_load", "served_reads_per_s",
+               "served_p50_ms", "served_p95_ms", "served_p99_ms", "sequential_plain_p50_ms", "sequential_plain_p99_ms"),
+    "bisulfite": ("reads", "hits", "ms", "whole_bs_path_reads_per_s"),
+}
+
+
+def rounded(x):
+    """Measured values to six digits (counts and texts as they are)."""
+    if isinstance(x, float):
+        return float(f"{x:.6g}")
+    if isinstance(x, dict):
+        return {k: rounded(v) for k, v in x.items()}
+    return x
+
+
+def short_line(line: dict) -> dict:
+    """The report's headline keys whole, of its parts the few values that sum them up."""
+    out = dict(line)
+    for part, keep in SHORT_KEYS.items():
+        if line.get(part):
+            out[part] = rounded({k: line[part][k] for k in keep if k in line[part]})
+    if line.get("roofline"):
+        out["roofline"]["kernels_ms"] = rounded({k: v["ms_per_launch"] for k, v in line["roofline"]["kernels"].items()})
+    if line.get("cpu_baseline") and line["cpu_baseline"].get("batched_prefetch"):
+        out["cpu_baseline"]["batched_prefetch_reads_per_s"] = rounded(line["cpu_baseline"]["batched_prefetch"]["value"])
+    if line.get("forms"):
+        out["forms"] = rounded({k: v if isinstance(v, str) else v["ms_per_step"] for k, v in line["forms"].items()})
+    return out
+
+
 # --------------------------------------------------------------------------------- GPU side
 def run_gpu(args):
     import torch
@@ -1101,7 +1141,8 @@ def run_gpu(args):
         "bisulfite": bisulfite,
         "clocks": clk.summary(),
     }
-    print(json.dumps(line), flush=True)
+    log("report: " + json.dumps(line))
+    print(json.dumps(short_line(line)), flush=True)
     return 0
 
 
