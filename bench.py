@@ -400,24 +400,6 @@ def bench_batched(mb, torch, dev, reps: int = 3):
     batched_s = e0.elapsed_time(e1) / 1000 / reps
     bsm, bhits = BP.result()
     BP.free()
-    # the fastest shape with the device work queue (reads handed out in read order), as its own
-    # replayed graph: reported beside the autotuner's choice, output compared
-    qo, _ = min(((o, t) for o, t in grid if o.flags & mb.MB_BATCHED), key=lambda p: p[1])
-    QP = mb.Plan(G, rd.n, len(rd.seq), n_smem + 64, n_hits + 64, opts=qo)
-    QP.capture(seq, off)
-    QP.replay()
-    torch.cuda.synchronize()
-    e0.record(st)
-    for _ in range(reps):
-        QP.replay()
-    e1.record(st)
-    torch.cuda.synchronize()
-    queue_s = e0.elapsed_time(e1) / 1000 / reps
-    qsm, qhits = QP.result()
-    QP.free()
-    queue_same = qsm.tobytes() == bsm.tobytes() and np.array_equal(qhits, bhits)
-    if not queue_same:
-        raise SystemExit("bench: the work-queue form disagrees with the autotuned form")
     # identity with the per-bucket launches, put back in read order
     rec, hl = [], []
     for ids, s_, o_, P, m, nh in buckets:
@@ -439,11 +421,9 @@ def bench_batched(mb, torch, dev, reps: int = 3):
             "plain_per_bucket_reads_per_s": rd.n / plain_s, "batched_graph_reads_per_s": rd.n / batched_s,
             "plain_per_bucket_bases_per_s": len(rd.seq) / plain_s, "batched_graph_bases_per_s": len(rd.seq) / batched_s,
             "speedup": plain_s / batched_s, "identical_output": bool(same),
-            "autotuned": mb.shape_of(best), "autotuned_ms": tune_ms,
+            "autotuned": mb.run_shape(best), "autotuned_ms": tune_ms,
             "autotune_grid": [dict(mb.shape_of(o), ms=round(ms, 3)) for o, ms in grid],
-            "plain_ms": plain_s * 1000, "batched_ms": batched_s * 1000,
-            "work_queue_best": dict(mb.shape_of(qo), graph_reads_per_s=rd.n / queue_s, ms=queue_s * 1000,
-                                    identical_output=bool(queue_same))}
+            "plain_ms": plain_s * 1000, "batched_ms": batched_s * 1000}
 
 
 def serve_requests(ref, n, seed):
@@ -676,10 +656,9 @@ def bench_bisulfite(mb, torch, dev, ref, opts, reps: int = 3):
     _, m, nh = mb.mb_seed_batch(G, seq, off, mate=mate, opts=o, out=out, cap=cap)
     hits = torch.empty(max(nh, 1), dtype=torch.int32, device=dev)
     keep = torch.empty(max(nh, 1), dtype=torch.uint8, device=dev)
-    # locate form for this batch: plain walks (16 per lane) or walks that join (2 per lane), the
-    # faster of the two on one timed call each (the join's per-call setup scales with the index)
-    forms = {"plain": dict(o, flags=o["flags"] & ~mb.MB_LOCATE_JOIN, prefetch_depth=16),
-             "join": dict(o, flags=o["flags"] | mb.MB_LOCATE_JOIN, prefetch_depth=2)}
+    # walks per lane for this batch (shared walks to the rate-4 samples, which hold four at least): the
+    # fastest of one timed call each
+    forms = {d: dict(o, flags=o["flags"] & ~mb.MB_LOCATE_JOIN, prefetch_depth=d) for d in (4, 8, 16)}
     st = torch.cuda.current_stream()
     form_ms = {}
     for name, fo in forms.items():
@@ -732,7 +711,7 @@ def bench_bisulfite(mb, torch, dev, ref, opts, reps: int = 3):
                        "30% CpG conversion) on the 3-base index of the 1 Gbp reference",
            "n": int(G.n), "index_build_s": build_s, "reads": rd.n, "smems": m, "hits": nh,
            "kept_hits": int(keep[:nh].sum().item()), "pieces": npieces, "ms": ms,
-           "locate_form": loc_form, "locate_form_ms": form_ms,
+           "locate_walks_per_lane": loc_form, "locate_ms_by_walks_per_lane": form_ms,
            "seed_locate_reads_per_s": rd.n / ((ms["seed"] + ms["locate"]) / 1000.0),
            "whole_bs_path_reads_per_s": rd.n / (total / 1000.0)}
     del out, hits, keep, seq, off, mate, ref_d, pieces
@@ -839,18 +818,15 @@ def run_gpu(args):
     ns = min(n_reads, 1_000_000)
     if args.autotune:
         best, tune_ms = mb.autotune(idx, seq[:int(rd.off[ns])], off[:ns + 1], opts=opts)
-        log(f"autotuned on {ns} reads: {mb.shape_of(best)}")
+        log(f"autotuned on {ns} reads: {mb.run_shape(best)}")
     else:
         best = mb.Opts(block_size=args.block, prefetch_depth=args.locate_walks,
                        flags=(mb.MB_BATCHED if args.queue else 0) | (mb.MB_SMEM_ONE_LOOP if args.one_loop else 0) |
-                       (mb.MB_LOCATE_JOIN if args.locate_join else 0),
-                       smem_burst=args.smem_burst, smem_wait=args.smem_wait, smem_warps=args.smem_warps)
+                       (mb.MB_LOCATE_JOIN if args.locate_join else 0))
     opts["block_size"] = best.block_size
     opts["prefetch_depth"] = best.prefetch_depth
     opts["flags"] = best.flags
-    opts["smem_burst"] = best.smem_burst
-    opts["smem_wait"] = best.smem_wait
-    opts["smem_warps"] = best.smem_warps
+    opts["smem_reads_per_warp"] = best.smem_reads_per_warp
 
     if args.locate_sweep:
         return locate_sweep(mb, torch, idx, out, m, hits, nh, opts)
@@ -927,7 +903,7 @@ def run_gpu(args):
              "graph_plan": {"reads_per_s": ws * args.steps * n_reads / (graph_ms / 1000.0),
                             "bases_per_s": ws * args.steps * n_bases / (graph_ms / 1000.0),
                             "ms_per_step": graph_ms / args.steps, "identical_output": bool(same),
-                            "gpu_launches": graph_launches, "shape": mb.shape_of(best)},
+                            "gpu_launches": graph_launches, "shape": mb.run_shape(best)},
              "reported": "graph_plan" if use_graph else "plain_launch"}
 
     # the same graph with MB_LOCATE_AUX and 16 walks per lane: the walks of the headline (locate stops at
@@ -954,7 +930,7 @@ def run_gpu(args):
             raise SystemExit("bench: the rate-4 locate form disagrees with the plain launches")
         forms["graph_plan_locate_aux"] = {
             "reads_per_s": ws * args.steps * n_reads / (aux_ms / 1000.0), "ms_per_step": aux_ms / args.steps,
-            "identical_output": bool(aux_same), "shape": mb.shape_of(mb.Opts(**aopts)),
+            "identical_output": bool(aux_same), "shape": mb.run_shape(mb.Opts(**aopts)),
             "note": "locate walks stop at the rate-4 SA samples the index keeps for text extension, as "
                     "in the headline; 16 walks per lane"}
         log(f"graph form with MB_LOCATE_AUX: {aux_ms / args.steps:.1f} ms/step (identical: {aux_same})")
@@ -1189,17 +1165,16 @@ def main():
     ap.add_argument("--no-autotune", action="store_true", help="(default) fixed launch shape")
     ap.add_argument("--block", type=int, default=512, choices=[128, 256, 512])
     ap.add_argument("--no-queue", dest="queue", action="store_false",
-                    help="SMEM kernel walks fixed read ranges per warp instead of a device work queue")
+                    help="with --one-loop: fixed read ranges per warp instead of a device work queue")
     ap.add_argument("--locate-walks", type=int, default=2, choices=[1, 2, 4, 8, 16])
     ap.add_argument("--one-loop", action="store_true", help="SMEM kernel in its one-loop form")
     ap.add_argument("--locate-join", dest="locate_join", action="store_true", default=True,
-                    help="(default) locate with walks that join (MB_LOCATE_JOIN)")
+                    help="(default) MB_LOCATE_JOIN; without effect on the index used here, whose walks end at the "
+                         "rate-4 samples")
     ap.add_argument("--no-locate-join", dest="locate_join", action="store_false",
-                    help="plain locate walks: every walk runs to its sampled row")
-    ap.add_argument("--smem-burst", type=int, default=0, help="SMEM kernel block steps between service passes")
-    ap.add_argument("--smem-wait", type=int, default=0, help="SMEM kernel lanes out of the loop that call a pass")
-    ap.add_argument("--smem-warps", type=int, default=0,
-                    help="SMEM kernel register budget: resident warps per SM aimed at (40: block 256 only; 48)")
+                    help="without MB_LOCATE_JOIN")
+    for name in ("--smem-burst", "--smem-wait", "--smem-warps"):
+        ap.add_argument(name, type=int, default=0, help="accepted, without effect")
     ap.add_argument("--reads", type=int, default=0,
                     help="seed only the first N reads of the batch (for ncu captures of the full index)")
     args = ap.parse_args()

@@ -507,16 +507,29 @@ def autotune(index: Index, seq, off, opts=None, stream=None, points: bool = Fals
 
 
 def shape_of(o: Opts) -> dict:
-    """The launch-shape fields of an Opts as a plain dict (for reports)."""
+    """The launch-shape fields of an Opts as a plain dict: what was asked for (run_shape: what runs)."""
     split = not (o.flags & MB_SMEM_ONE_LOOP)
     return {"block_size": o.block_size or 256, "work_queue": bool(o.flags & MB_BATCHED),
             "smem_form": "slots" if split else "one_loop",
             "smem_burst": (o.smem_burst or 8) if split else None,
             "smem_wait": (o.smem_wait or 8) if split else None,
             "smem_warps": (o.smem_warps or None) if split else None,
-            "smem_reads_per_warp": (o.smem_reads_per_warp or 64) if split else None,
+            "smem_reads_per_warp": (o.smem_reads_per_warp if 0 < o.smem_reads_per_warp < 32 else 64) if split else None,
             "locate_walks_per_lane": o.prefetch_depth or 1, "locate_join": bool(o.flags & MB_LOCATE_JOIN),
             "locate_aux": bool(o.flags & MB_LOCATE_AUX)}
+
+
+def run_shape(o: Opts) -> dict:
+    """The launch shape that an Opts gives on an index with the rate-4 samples: the slot form always takes
+    reads from the queue and has no burst, wait or warps; shared walks end at the rate-4 samples, at
+    least four per lane, and never join (locate that goes hit by hit has no walks per lane)."""
+    d = shape_of(o)
+    if d["smem_form"] == "slots":
+        d["work_queue"] = True
+    for k in ("smem_burst", "smem_wait", "smem_warps"):
+        del d[k]
+    d.update(locate_walks_per_lane=max(4, d["locate_walks_per_lane"]), locate_join=False, locate_aux=True)
+    return d
 
 
 # ---------------------------------------------------------------------------- served form

@@ -70,3 +70,13 @@ def test_line_on_stdout_is_short_and_keeps_the_headline():
         assert set(keys) <= set(line[part])
     assert line["e2e"]["h2d_bytes_per_step"] == 3160000008
     assert bench.short_line(dict(full, e2e=None, batched=None, cpu_baseline=None))["e2e"] is None
+
+
+def test_run_shape_leaves_out_what_has_no_effect():
+    mb = pytest.importorskip("paper_2606_15357_gb300")
+    a = mb.run_shape(mb.Opts(block_size=512, smem_burst=4, smem_wait=16, smem_reads_per_warp=40, prefetch_depth=2))
+    b = mb.run_shape(mb.Opts(block_size=512, flags=mb.MB_BATCHED | mb.MB_LOCATE_JOIN))
+    assert a == b and a["work_queue"] and a["smem_reads_per_warp"] == 64 and "smem_burst" not in a
+    assert mb.shape_of(mb.Opts(smem_reads_per_warp=32))["smem_reads_per_warp"] == 64
+    assert mb.shape_of(mb.Opts(smem_reads_per_warp=31))["smem_reads_per_warp"] == 31
+    assert not mb.run_shape(mb.Opts(flags=mb.MB_SMEM_ONE_LOOP))["work_queue"]
