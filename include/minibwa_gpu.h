@@ -100,8 +100,8 @@ typedef struct {
                                  device has room (built with the index, also on load; not in files;
                                  MB_NO_KMER declines it) */
     uint32_t flags;           /* MB_* flags above */
-    uint32_t chunk_reads;     /* mb_seed_locate: reads per pipelined chunk (0 = 2^22; with host
-                                 inputs the first chunk is a quarter of the others) */
+    uint32_t chunk_reads;     /* mb_seed_locate: reads per pipelined chunk (0 = 2^22; host inputs of
+                                 2^28 to 2^30 bases go in two chunks, the first a third) */
     uint32_t prefetch_depth;  /* tuning: LF-walks in flight per lane in locate, 1/2/4/8/16 (0 = 1) */
     uint32_t block_size;      /* tuning: threads per block (0 = default) */
     uint32_t smem_burst;      /* accepted, without effect: the slot form picks its steps itself */

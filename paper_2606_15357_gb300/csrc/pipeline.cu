@@ -25,7 +25,6 @@ namespace {
 
 constexpr u32 PIPE_READS = 1u << 22;      // default reads per chunk
 constexpr u64 PIPE_BASES = 1ull << 29;    // at most this many bases per chunk (at least one read)
-constexpr u32 PIPE_GROW = 4;              // how much smaller the first chunk is (host inputs)
 constexpr u32 SLICE_READS = 1u << 25;     // at most this many reads per slice (located at once)
                                           // (MB_SLICE_READS in the environment may lower it)
 constexpr u64 SLICE_BASES = 1ull << 33;   // and this many bases (at least one chunk)
@@ -181,10 +180,19 @@ extern "C" int mb_seed_locate(const mb_index *idx, const uint8_t *seq, const uin
     }
     MB_TRY(mb_check_span(seq + hoff[0], hoff[n_reads] - hoff[0], "mb_seed_locate: seq[off[0], off[n_reads])"));
     const u32 per = opts && opts->chunk_reads ? opts->chunk_reads : PIPE_READS;
-    // inputs from the host: the first chunk's copy has nothing to hide behind, so chunks start at a quarter
-    // and double (a chunk's seeding takes about four times its copy; 4M reads: 18.9 -> 18.3 ms, starting
-    // at a sixteenth 19.1: each chunk ends with a tail and a wait of its own)
-    u32 grow = (opts && opts->chunk_reads) || seq_dev ? 1u : PIPE_GROW;
+    // Inputs from the host: the first chunk's copy has nothing to hide behind, and each chunk ends with a tail
+    // of its own (the chains of reads inside repeats, about 1 ms).  So a batch of more than half a chunk's and
+    // at most two chunks' bases goes in two chunks, the first a third of it (or what a full second one
+    // leaves); a smaller one goes whole and a larger one in full chunks.  150-base reads on 1 Gbp, full
+    // chunks -> two: 2M 10.3 -> 9.9 ms, 3M 14.5 -> 13.6, 4M 19.0 -> 17.4, 5M 22.4 -> 21.0, 6M 25.9 -> 25.1,
+    // 7M 29.1 either way.  First chunks of 40% and 50% are slower (4M: 17.6, 17.9), chunks that start at a
+    // quarter of the largest and double lose outside 1.7M to 4M reads (1.1M 6.8 -> 7.3, 6M 25.9 -> 27.0).
+    u64 first = PIPE_BASES;
+    const u64 all = hoff[n_reads] - hoff[0];
+    if (!(opts && opts->chunk_reads) && !seq_dev && all > PIPE_BASES / 2 && all <= 2 * PIPE_BASES) {
+        const u64 want = hoff[0] + std::max(all / 3, all - std::min(all, PIPE_BASES));
+        first = std::min(PIPE_BASES, *std::lower_bound(hoff + 1, hoff + n_reads, want) - hoff[0]);
+    }
     std::vector<Chunk> chunks;
     u32 max_nr = 0;
     u64 max_nb = 0;
@@ -194,9 +202,8 @@ extern "C" int mb_seed_locate(const mb_index *idx, const uint8_t *seq, const uin
         c.o0 = hoff[r];
         // the chunk ends before the first read (after read r) whose end passes o0 + PIPE_BASES, and
         // after at most `per` reads: a binary search over the offsets (which must not decrease)
-        const u32 emax = (u32)std::min<u64>((u64)n_reads, (u64)r + std::max(1u, per / grow));
-        const u64 lim = c.o0 + PIPE_BASES / grow;
-        grow = grow > 1 ? grow / 2 : 1;
+        const u32 emax = (u32)std::min<u64>((u64)n_reads, (u64)r + per);
+        const u64 lim = c.o0 + (r == 0 ? first : PIPE_BASES);
         u32 e = (u32)(std::upper_bound(hoff + r + 2, hoff + emax + 1, lim) - (hoff + 1));
         if (e < r + 1) e = r + 1;
         c.nr = e - r;

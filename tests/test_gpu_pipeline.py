@@ -245,3 +245,38 @@ def test_kept_workspace_serves_options_without_effect(mb, repeat_rich):
     sm2, hits2 = mb.seed_locate(G, rd.seq, rd.off, opts=dict(smem_burst=4, smem_wait=16, smem_warps=40))
     assert torch.cuda.mem_get_info()[0] == free
     assert sm2.tobytes() == sm.tobytes() and np.array_equal(hits2, hits)
+
+
+@pytest.fixture(scope="module")
+def uniform(mb):
+    ref = np.random.default_rng(17).integers(0, 4, 3_000_000).astype(np.uint8)
+    return ref, mb.mb_index_build(ref)
+
+
+@pytest.mark.parametrize("bases", [1 << 27, 1 << 28, (1 << 28) + 1, 1 << 29, (1 << 29) + 1, (1 << 30) - 9000, 1 << 30,
+                                   (1 << 30) + 1])
+@pytest.mark.parametrize("lo,hi", [(300, 300), (1000, 9000)])
+def test_chunks_of_host_inputs(mb, uniform, bases, lo, hi):
+    """Host inputs go whole up to half a chunk's bases, in two chunks up to two (the first a third), else in full
+    ones; device inputs in full ones throughout.  Results are the same; up to 2^28 bases the launches too, and
+    between there and 2^29, one full chunk, there are more."""
+    ref, G = uniform
+    r = np.random.default_rng(bases % 97)
+    lens = r.integers(lo, hi + 1, bases // lo + 1)
+    n = int(np.searchsorted(np.cumsum(lens), bases)) + 1
+    off = np.concatenate([[0], np.cumsum(lens[:n])])
+    off[-1] = bases
+    seq = np.resize(ref, bases)   # reads follow each other along the reference, again and again
+    got = []
+    for s, o in ((seq, off.astype(np.uint64)), (torch.from_numpy(seq).cuda(), torch.from_numpy(off).cuda())):
+        out, hits = np.zeros(2 * n, mb.SMEM_DTYPE), np.zeros(2 * n, np.uint32)
+        l0 = mb.launch_count()
+        m, nh = mb.seed_locate(G, s, o, opts=dict(min_len=30, max_occ=1), out=out, cap=len(out), hits=hits,
+                               hits_cap=len(hits))
+        got.append((m, nh, out[:m].tobytes(), hits[:nh].tobytes(), mb.launch_count() - l0))
+    host, device = got
+    assert host[:4] == device[:4] and host[0] >= n - 1
+    if bases <= 1 << 28:
+        assert host[4] == device[4]
+    elif bases <= 1 << 29:
+        assert host[4] > device[4]
