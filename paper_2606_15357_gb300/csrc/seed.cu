@@ -7,9 +7,10 @@
 // the way to keep many block reads in flight.
 //
 // Output: each read first writes its SMEMs into a private run of slots in scratch memory
-// (off[r]/16 + 8r slots before it), further ones into a pool all reads share; a prefix sum over the
-// per-read counts gives the final positions, and a gather writes the 48-byte records.  A read with a
-// record that found no room at all is listed and recomputed straight into the final records.
+// (off[r]/16 + 8r slots before it; the pieces of a read that is cut share its run), further ones into a
+// pool all reads share; a prefix sum over the per-read counts gives the final positions, and a gather
+// writes the 48-byte records.  A read with a record that found no room at all is listed and recomputed
+// straight into the final records.
 #include <climits>
 #include <vector>
 #include "common.cuh"
@@ -490,10 +491,16 @@ struct WarpRange {
 constexpr u64 LONG_BASES = 1ull << 29;
 constexpr int LONG_LEN = 1024;
 constexpr u32 STEPS_LONG = 0x3FFFFFu;   // in the step count: cut at once
+//
+// The slots that the cut read has not used are dealt out among its items in runs, so that a batch of long
+// reads has as many as if its reads were not cut, a record per 16 bases; what an item finds beyond its run
+// goes to the pool.  (With the pool alone, of one record per 256 bases, 20,000 reads of 10 kb with a
+// record per 190 bases filled it, and the pass that recomputes a read took 24 of 47 ms.)
 struct Item {
     u32 read;
     int c0, c1;
-    u32 cnt;      // its records (bit 31: one found no room), then the records of the read before it
+    u32 cnt;      // first where its run starts in the read's slots, then its records (bit 31: one found no room),
+                  // then the records of the read before it
 };
 struct HeavyRead {
     u32 read, first, n, cnt;   // its items and the records found before the cut (bit 31: one found no room)
@@ -508,6 +515,7 @@ struct SplitBufs {
     u32 *n = nullptr;   // counters: items, cut reads, pool records, the items' queue head
     Item *items = nullptr;
     HeavyRead *heavy = nullptr;
+    uint2 *runs = nullptr;   // per item: its run of slots, and how many it filled
     PoolRec *pool = nullptr;
     u32 items_cap = 0, pool_cap = 0;   // zero: no read is cut, no record goes to the pool
     u32 steps = ~0u, starts = 64;
@@ -734,6 +742,16 @@ struct WarpSlots {
     u8 cls[SLOTS];
     u8 list[32];                                   // the slots of the current step
 };
+// With items also their runs of slots, 6 bytes: two blocks of 16 warps just stay within 196 KB, which leaves 60
+// KB of L1 (12 bytes more, and so 28 KB of L1: the items of 200,000 reads of 100 bp - 10 kb take 6.4 ms, not
+// 5.1; the runs read from the items at each record: 5.6).
+template <bool ITEMS>
+struct SlotTable : WarpSlots {};
+template <>
+struct SlotTable<true> : WarpSlots {
+    u32 run[SLOTS];
+    unsigned short room[SLOTS];
+};
 
 // Sixteen bases (bytes) to 2-bit codes, first base in the low bits.  Per word of four bytes one
 // multiply moves byte b to bits 24 + 2b; the eight other products stay below bit 24 or pass bit 31.
@@ -782,7 +800,7 @@ __global__ void __launch_bounds__(512, 2)
                  u64 slot_total, u64 *__restrict__ counts, u32 *__restrict__ ovf_list, u32 *__restrict__ ovf_n,
                  u32 *qhead, const u32 *__restrict__ lc, bool uext, u32 nslots, u32 *err, u32 *chk, SplitBufs sp) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    WarpSlots &W = reinterpret_cast<WarpSlots *>(smem_raw)[threadIdx.x >> 5];
+    SlotTable<ITEMS> &W = reinterpret_cast<SlotTable<ITEMS> *>(smem_raw)[threadIdx.x >> 5];
     const u32 FULL = 0xffffffffu;
     const u32 lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
     const u32 n = (u32)I.n, prim = (u32)I.primary;
@@ -1016,15 +1034,20 @@ __global__ void __launch_bounds__(512, 2)
                 at = W.at[x];
                 const int c1 = ITEMS ? W.c1[x] : INT_MAX;
                 const bool done2 = S.u == 2 && S.j == S.L, done7 = S.u == 7 && S.s == 0;
-                // the read's slots (an item has none)
+                // the read's slots (an item has a run of them, below)
                 const u64 sb = slots_before(at - o0, r), se = slots_before(at - o0 + (u64)S.L, (u64)r + 1);
                 const u32 cap = !ITEMS && se <= slot_total ? (u32)(se - sb) : 0u;
                 if ((meta & M_PEND) || done2 || done7) {   // the match P[i, j) ends: its record
                     if (!ITEMS || (S.i >= W.c0[x] && S.i < c1)) {
                         const SlotRec rec{(u32)S.i, (u32)S.j, S.k, S.kr, done7 ? 1u : S.s, done7 ? S.pos : NOPOS};
+                        bool kept = false;
+                        if constexpr (ITEMS) {
+                            kept = cnt < W.room[x];
+                            if (kept) slots[W.run[x] + cnt] = rec;
+                        }
                         if (!ITEMS && cnt < cap) {
                             slots[sb + cnt] = rec;
-                        } else {
+                        } else if (!kept) {
                             const u32 q = sp.pool_cap ? atomicAdd(sp.n + 2, 1u) : 0u;
                             if (q < sp.pool_cap) sp.pool[q] = PoolRec{ITEMS ? r | NO_ROOM : r, cnt, rec};
                             else meta |= M_DROP;
@@ -1054,17 +1077,22 @@ __global__ void __launch_bounds__(512, 2)
                             for (u32 t = q; t < sp.items_cap; ++t) sp.items[t] = Item{NO_READ, 0, 0, 0u};
                         if (q < sp.items_cap && k <= sp.items_cap - q) {
                             cut = true;
+                            // (their runs of slots come after the read's records and the slot that ends them)
                             for (u32 t = 0; t < k; ++t)
                                 sp.items[q + t] = Item{r, c + (int)(t * starts),
-                                                       t + 1 < k ? c + (int)((t + 1) * starts) : INT_MAX, 0u};
+                                                       t + 1 < k ? c + (int)((t + 1) * starts) : INT_MAX,
+                                                       cnt + 1 + t * (starts / 16)};
                             sp.heavy[atomicAdd(sp.n + 1, 1u)] = HeavyRead{r, q, k, cnt | (meta & M_DROP ? NO_ROOM : 0u)};
                             if (!ITEMS && cnt < cap) slots[sb + cnt].qend = 0;   // ends the read's slots
                             fin = true;
                         }
                     }
                 }
-                if (fin && ITEMS) {
-                    sp.items[r].cnt = cnt | (meta & M_DROP ? NO_ROOM : 0u);
+                if constexpr (ITEMS) {
+                    if (fin) {
+                        sp.items[r].cnt = cnt | (meta & M_DROP ? NO_ROOM : 0u);
+                        sp.runs[r] = make_uint2(W.run[x], min(cnt, (u32)W.room[x]));
+                    }
                 } else if (fin) {
                     counts[r] = cnt;
                     if ((meta & M_DROP) && !cut) ovf_list[atomicAdd(ovf_n, 1u)] = r;
@@ -1104,9 +1132,15 @@ __global__ void __launch_bounds__(512, 2)
                     S.i = max(it.c0 - 1, 0);
                     S.j = S.i + (int)lr - 1;
                     S.u = S.j < S.L ? 1 : 0;                  // Algorithm 3 queues a read only if l - 1 < |P|
-                    if (ITEMS) {
+                    if constexpr (ITEMS) {
                         W.c0[x] = it.c0;
                         W.c1[x] = it.c1;
+                        // its run: a slot per 16 starts, the last item's up to the end of the read's slots
+                        const u64 sb = slots_before(b - o0, it.read), se = slots_before(e - o0, (u64)it.read + 1);
+                        const u32 cap = !none && se <= slot_total && se < (1ull << 32) ? (u32)(se - sb) : 0u;
+                        const u32 most = it.c1 == INT_MAX ? 0xFFFFu : (u32)(it.c1 - it.c0) / 16;
+                        W.run[x] = (u32)sb + it.cnt;
+                        W.room[x] = (unsigned short)(it.cnt < cap ? min(min(most, 0xFFFFu), cap - it.cnt) : 0u);
                     }
                     S.pos = 0;
                     restart();
@@ -1235,30 +1269,20 @@ __device__ __forceinline__ void write_rec(mb_smem *out, u64 *hitc, u64 m, u32 r,
     hitc[m] = s > max_occ ? 0 : s;
 }
 
-// Copies each read's SMEMs from its slots to the records (a slot with qend = 0 ends them early: a cut
-// read).  Its other records are in the pool, or k_smem_overflow recomputes the read.  A warp takes 32
-// reads, whose records are neighbours in the output: its lanes take the records in order, so that the
-// 48-byte records, their hit counts and positions leave in whole sectors (one read per lane, 34M records:
-// 1.34 ms).
-__global__ void __launch_bounds__(256)
-    k_gather(const u64 *__restrict__ off, u32 nr, const SlotRec *__restrict__ slots, u64 slot_total,
-                         const u64 *__restrict__ counts, const u64 *__restrict__ soff, u32 max_occ,
-                         mb_smem *__restrict__ out, u64 *__restrict__ hitc, u64 out_cap,
-                         u32 *__restrict__ known = nullptr) {
-    __shared__ u32 s_end[8][32];
-    __shared__ u64 s_slot[8][32], s_out[8][32];
-    __shared__ u64 s_rec[8][32 * 6];
-    const u32 FULL = 0xffffffffu, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const u64 r0 = (blockIdx.x * (u64)blockDim.x + threadIdx.x) & ~31ull, r = r0 + lane;
-    if (r0 >= nr) return;
-    u32 cnt = 0;
-    u64 sb = 0, o = 0;
-    if (r < nr) {
-        sb = slot_base(off, r);
-        const u64 se = slot_base(off, r + 1), c = counts[r];
-        o = soff[r];
-        if (se <= slot_total) cnt = (u32)(c < se - sb ? c : se - sb);
-    }
+// Copies SMEMs from slots to the records, for 32 runs of slots by a warp, lane q describing run q: cnt slots
+// from sb, their records at o on, of read rd.  The runs' records are neighbours in the output, and the lanes
+// take them in order, so that the 48-byte records, their hit counts and positions leave in whole sectors (one
+// read per lane, 34M records: 1.34 ms).  ENDS: a slot with qend = 0 ends its run early (a cut read).
+struct GatherWarp {
+    u32 end[32], read[32];
+    u64 slot[32], out[32];
+    u64 rec[32 * 6];
+};
+template <bool ENDS>
+__device__ __forceinline__ void gather_runs(GatherWarp &G, u32 cnt, u64 sb, u64 o, u32 rd, const SlotRec *__restrict__ slots,
+                                            u32 max_occ, mb_smem *__restrict__ out, u64 *__restrict__ hitc, u64 out_cap,
+                                            u32 *__restrict__ known) {
+    const u32 FULL = 0xffffffffu, lane = threadIdx.x & 31;
     u32 incl = cnt;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
@@ -1266,34 +1290,36 @@ __global__ void __launch_bounds__(256)
         if (lane >= (u32)d) incl += v;
     }
     const u32 total = __shfl_sync(FULL, incl, 31);
-    s_end[w][lane] = incl;
-    s_slot[w][lane] = sb - (incl - cnt);
-    s_out[w][lane] = o - (incl - cnt);
+    G.end[lane] = incl;
+    G.read[lane] = rd;
+    G.slot[lane] = sb - (incl - cnt);
+    G.out[lane] = o - (incl - cnt);
     __syncwarp();
-    u32 ended = 32;   // the read, if any, that goes on into the next 32 slots but has ended before them
+    u32 ended = 32;   // the run, if any, that goes on into the next 32 slots but has ended before them
     for (u32 t0 = 0; t0 < total; t0 += 32) {
         const u32 t = t0 + lane;
-        u32 q = 0, first = 0;   // the slot's read, and that read's first t
+        u32 q = 0, first = 0;   // the slot's run, and that run's first t
         bool ok = t < total;
         u64 m = 0;
         SlotRec x{};
         if (ok) {
 #pragma unroll
             for (u32 b = 16; b; b >>= 1)
-                if (s_end[w][q + b - 1] <= t) q += b;
-            first = q ? s_end[w][q - 1] : 0u;
-            x = slots[s_slot[w][q] + t];
-            m = s_out[w][q] + t;
+                if (G.end[q + b - 1] <= t) q += b;
+            first = q ? G.end[q - 1] : 0u;
+            x = slots[G.slot[q] + t];
+            m = G.out[q] + t;
         }
-        // a slot with qend = 0 ends its read; what lies behind it was never written
-        const u32 ends = __ballot_sync(FULL, ok && x.qend == 0), from_lane = first > t0 ? first - t0 : 0u;
-        ok = ok && !((ends & (FULL >> (31 - lane))) >> from_lane) && !(q == ended && first < t0);
-        ended = __shfl_sync(FULL, ok ? 32u : q, 31);
+        if (ENDS) {   // what lies behind a slot with qend = 0 is not the run's
+            const u32 ends = __ballot_sync(FULL, ok && x.qend == 0), from_lane = first > t0 ? first - t0 : 0u;
+            ok = ok && !((ends & (FULL >> (31 - lane))) >> from_lane) && !(q == ended && first < t0);
+            ended = __shfl_sync(FULL, ok ? 32u : q, 31);
+        }
         ok = ok && m < out_cap;
         if (ok) {
             const bool over = x.s > max_occ;
-            u64 *rec = s_rec[w] + 6 * lane;
-            rec[0] = (u64)(u32)(r0 + q) | ((u64)x.qbeg << 32);
+            u64 *rec = G.rec + 6 * lane;
+            rec[0] = (u64)G.read[q] | ((u64)x.qbeg << 32);
             rec[1] = (u64)x.qend | ((u64)(over ? MB_SMEM_OVER_MAX_OCC : 0u) << 32);
             rec[2] = x.k;
             rec[3] = x.kr;
@@ -1309,17 +1335,51 @@ __global__ void __launch_bounds__(256)
         for (u32 u = 0; u < 6; ++u) {
             const u32 k = u * 32 + lane, from = k / 6;
             const u64 to = __shfl_sync(FULL, m, (int)from);
-            if ((mask >> from) & 1u) reinterpret_cast<u64 *>(out)[to * 6 + (k - 6 * from)] = s_rec[w][k];
+            if ((mask >> from) & 1u) reinterpret_cast<u64 *>(out)[to * 6 + (k - 6 * from)] = G.rec[k];
         }
         __syncwarp();
     }
 }
 
-// The pool's records to their places.
-__global__ void k_pool_write(SplitBufs sp, const u64 *__restrict__ soff, u32 max_occ, mb_smem *__restrict__ out,
-                             u64 *__restrict__ hitc, u64 out_cap, u32 *__restrict__ known = nullptr) {
-    const u32 np = min(sp.n[2], sp.pool_cap);
-    for (u32 q = blockIdx.x * blockDim.x + threadIdx.x; q < np; q += gridDim.x * blockDim.x) {
+// The records in the reads' own slots.  Others are in their items' runs or the pool (k_rest_write), or
+// k_smem_overflow recomputes the read.
+__global__ void __launch_bounds__(256)
+    k_gather(const u64 *__restrict__ off, u32 nr, const SlotRec *__restrict__ slots, u64 slot_total,
+                         const u64 *__restrict__ counts, const u64 *__restrict__ soff, u32 max_occ,
+                         mb_smem *__restrict__ out, u64 *__restrict__ hitc, u64 out_cap,
+                         u32 *__restrict__ known = nullptr) {
+    __shared__ GatherWarp sg[8];
+    const u64 r = blockIdx.x * (u64)blockDim.x + threadIdx.x;
+    if ((r & ~31ull) >= nr) return;
+    u32 cnt = 0;
+    u64 sb = 0, o = 0;
+    if (r < nr) {
+        sb = slot_base(off, r);
+        const u64 se = slot_base(off, r + 1), c = counts[r];
+        o = soff[r];
+        if (se <= slot_total) cnt = (u32)(c < se - sb ? c : se - sb);
+    }
+    gather_runs<true>(sg[threadIdx.x >> 5], cnt, sb, o, (u32)r, slots, max_occ, out, hitc, out_cap, known);
+}
+
+// The records in the items' runs of slots, and those in the pool, to their places.
+__global__ void __launch_bounds__(256)
+    k_rest_write(SplitBufs sp, const SlotRec *__restrict__ slots, const u64 *__restrict__ soff, u32 max_occ,
+                 mb_smem *__restrict__ out, u64 *__restrict__ hitc, u64 out_cap, u32 *__restrict__ known = nullptr) {
+    __shared__ GatherWarp sg[8];
+    const u32 ni = min(sp.n[0], sp.items_cap), np = min(sp.n[2], sp.pool_cap);
+    const u32 step = gridDim.x * blockDim.x, t0 = blockIdx.x * blockDim.x + threadIdx.x;
+    for (u32 g = t0 & ~31u; g < ni; g += step) {
+        const u32 t = g + (threadIdx.x & 31);
+        Item it{NO_READ, 0, 0, 0u};
+        if (t < ni) it = sp.items[t];
+        const bool on = it.read != NO_READ;
+        const uint2 run = on ? sp.runs[t] : make_uint2(0u, 0u);
+        gather_runs<false>(sg[threadIdx.x >> 5], run.y, run.x, on ? soff[it.read] + it.cnt : 0, it.read, slots, max_occ,
+                           out, hitc, out_cap, known);
+        __syncwarp();
+    }
+    for (u32 q = t0; q < np; q += step) {
         const PoolRec p = sp.pool[q];
         u32 r = p.who, idx = p.idx;
         if (r & NO_ROOM) {
@@ -2106,9 +2166,9 @@ unsigned resident_grid(const void *kernel, int block, u64 work_items, size_t sme
 template <bool ITEMS>
 int launch_slots(const SmemArgs &a, int block, cudaStream_t st) {
     const int wpb = block / 32;
-    const size_t smem = wpb * sizeof(WarpSlots);
+    const size_t smem = wpb * sizeof(SlotTable<ITEMS>);
     const void *f = (const void *)k_smem_slots<ITEMS>;
-    MB_CK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(16 * sizeof(WarpSlots))));
+    MB_CK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(16 * sizeof(SlotTable<ITEMS>))));
     const unsigned g = resident_grid(f, block, ITEMS ? 1ull << 40 : (u64)a.nr * 32, smem);
     const u64 each = (a.nr + (u64)g * wpb - 1) / ((u64)g * wpb);
     const u32 most = a.per_warp && a.per_warp < (u32)SLOTS ? a.per_warp : (u32)SLOTS;
@@ -2149,7 +2209,8 @@ struct SplitRoom {
         pool = n_reads < NO_ROOM ? (u32)(po < (1u << 30) ? po : 1u << 30) : 0u;
     }
     size_t items_at() const { return ((size_t)pool * sizeof(PoolRec) + 255) & ~(size_t)255; }
-    size_t heavy_at() const { return items_at() + (((size_t)items * sizeof(Item) + 255) & ~(size_t)255); }
+    size_t runs_at() const { return items_at() + (((size_t)items * sizeof(Item) + 255) & ~(size_t)255); }
+    size_t heavy_at() const { return runs_at() + (((size_t)items * sizeof(uint2) + 255) & ~(size_t)255); }
     size_t bytes() const { return heavy_at() + (size_t)heavy * sizeof(HeavyRead); }
     SplitBufs bufs(void *mem, u32 *counters) const {
         char *m = (char *)mem;
@@ -2157,6 +2218,7 @@ struct SplitRoom {
         b.n = counters;
         b.pool = (PoolRec *)m;
         b.items = (Item *)(m + items_at());
+        b.runs = (uint2 *)(m + runs_at());
         b.heavy = (HeavyRead *)(m + heavy_at());
         b.items_cap = pool ? items : 0;
         b.pool_cap = pool;
@@ -2395,6 +2457,7 @@ bool locate_joins(const DevIndex &I, u32 flags) {
 
 // The SMEM kernel in the requested shape: work counters, work queue, threads per block.
 // With `items` the items of cut reads too (launch_items), which a caller may also do later.
+constexpr unsigned REST_GRID = 152 * 4;   // k_rest_write
 constexpr u32 LATE_ITEMS = 65536;   // mb_seed_device: reads up to which it does
 int launch_items(const SmemArgs &a, cudaStream_t st) {
     if (!a.sp.items_cap) return MB_OK;
@@ -2485,7 +2548,7 @@ int mb_seed_device(const mb_index *idx, const u8 *dseq, const u64 *doff, u32 n_r
         kt_items.stop();
     }
     const u64 total = v[0];
-    const u32 err = (u32)v[4], over = (u32)v[2], pooled = (u32)v[9];
+    const u32 err = (u32)v[4], over = (u32)v[2], rest = (u32)v[8] | (u32)v[9];   // items, records in the pool
     if (err) {
         mb_set_error("mb_seed_batch: device check failed (0x%x): %s", err,
                      (err & DEVCHK_OFFSETS) ? "read offsets decrease or leave [off[0], off[n_reads]]"
@@ -2512,8 +2575,8 @@ int mb_seed_device(const mb_index *idx, const u8 *dseq, const u64 *doff, u32 n_r
     u64 *hitc = bhit.as<u64>();
     k_gather<<<G, B, 0, st>>>(doff, n_reads, slots, nslots, counts, soff, max_occ, dout, hitc, total);
     MB_KCHECK();
-    if (pooled) {
-        k_pool_write<<<152, 256, 0, st>>>(split, soff, max_occ, dout, hitc, total);
+    if (rest) {
+        k_rest_write<<<REST_GRID, 256, 0, st>>>(split, slots, soff, max_occ, dout, hitc, total);
         MB_KCHECK();
     }
     if (over) {
@@ -3040,7 +3103,7 @@ static int plan_seed(mb_plan *P, const uint8_t *seq, const uint64_t *off, uint32
     k_gather<<<G, 256, 0, st>>>(off, n_reads, P->slots, P->nslots, P->counts, P->soff, P->max_occ, P->out, P->hitc,
                                 P->max_smem, P->known);
     MB_KCHECK();
-    k_pool_write<<<152, 256, 0, st>>>(P->split, P->soff, P->max_occ, P->out, P->hitc, P->max_smem, P->known);
+    k_rest_write<<<REST_GRID, 256, 0, st>>>(P->split, P->slots, P->soff, P->max_occ, P->out, P->hitc, P->max_smem, P->known);
     MB_KCHECK();
     k_smem_overflow<<<resident_grid((const void *)k_smem_overflow, 128, 1ull << 40), 128, 0, st>>>(I, seq, off, n_reads, mate, bs, P->l, P->c, P->kmer, P->ovf, ovf_n, P->soff,
                                          P->max_occ, P->out, P->hitc, P->max_smem, nullptr, P->known);

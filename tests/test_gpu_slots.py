@@ -94,3 +94,39 @@ def test_profile_counts_the_items_of_cut_reads(mb, tandem):
         mb.profile_enable(False)
         ms, n = mb.profile_get("smem")
         assert n == launches and ms > 0
+
+
+def test_batch_of_long_reads_has_slots_for_its_records(mb):
+    """6,000 reads of 10 kb, all cut before their first step, with a record per 100 bases: more than the pool
+    holds (a record per 256 bases).  The records are those of the one-loop form, which cuts nothing, and
+    the call takes little more than the same bases in reads of 150 (1.1 and 0.8 ms; 21 ms when reads were
+    recomputed one per thread)."""
+    ref = np.random.default_rng(12).integers(0, 4, 5_000_000).astype(np.uint8)
+    G = mb.mb_index_build(ref)
+    G.drop_sa()
+    n, length = 6000, 10_000
+    rd = synth.reads(ref, n, 13, mode=0, read_len=length, sub_lo=0.01)
+    seq, off = torch.from_numpy(rd.seq).cuda(), torch.from_numpy(rd.off.view(np.int64)).cuda()
+    short = torch.arange(0, n * length + 1, 150, device="cuda")
+    cap = 2 * n * length // 100
+    out = torch.zeros(cap * 48, dtype=torch.uint8, device="cuda")
+    ms, recs = {}, {}
+    for name, o, opts in (("long", off, {}), ("short", short, {}), ("one loop", off, dict(flags=mb.MB_SMEM_ONE_LOOP))):
+        t = []
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            _, m, nh = mb.mb_seed_batch(G, seq, o, opts=opts, out=out, cap=cap)
+            b.record()
+            torch.cuda.synchronize()
+            t.append(a.elapsed_time(b))
+        ms[name], recs[name] = min(t), (m, nh, out[:48 * m].cpu().numpy().tobytes())
+    assert recs["long"] == recs["one loop"]
+    assert recs["long"][0] > n // 2 + n * length // 256 + 16384
+    assert ms["long"] < 4 * ms["short"], ms
+    P = mb.Plan(G, n, n * length, recs["long"][0] + 1, recs["long"][1] + 1)
+    P.run(seq, off)
+    psm, phits = P.result()
+    assert psm.tobytes() == recs["long"][2]
+    hits, _ = mb.mb_locate(G, psm, len(psm), cap=len(phits))
+    assert np.array_equal(hits, phits)
