@@ -7,8 +7,8 @@
 // original reference under it and cut at every such position; the pieces of at least min_len bases
 // are the output.
 //
-// A warp takes a tile of 256 hits, finds the tile's first record by one binary search and then reads the
-// records 32 at a time, each hit finding its record among them in shared memory.  Only the read's C (or
+// A warp takes a tile of up to 256 hits, finds the tile's first record by one binary search and then reads
+// the records 32 at a time, each hit finding its record among them in shared memory.  Only the read's C (or
 // G) positions can cut, and conversion leaves few: they are marked once per record, and a hit reads the
 // reference there only.  The pieces are counted per tile, the tiles' counts scanned, and the tiles
 // written (a hit found uncut while counting reads no reference again).  14M hits: the two passes of the
@@ -18,7 +18,7 @@
 
 namespace {
 
-constexpr u32 TILE = 256;        // hits per tile
+constexpr u32 TILE = 256;        // hits per tile at most
 constexpr u32 MARKS = 8;         // words of cut marks per record: seeds of up to 256 bases
 constexpr u32 NO_MARKS = 1u << 31;
 enum { BS_FILTER = 0, BS_COUNT = 1, BS_WRITE = 2 };
@@ -36,6 +36,7 @@ struct BsArgs {
     const u64 *off;
     const u8 *mate;
     u32 min_len;
+    u32 per_tile;         // hits per tile
     u64 *tile;            // pieces of each tile, then of the tiles before it
     u8 *kind;             // per hit: no piece, one uncut piece, or pieces to find again when writing
     mb_piece *out;
@@ -63,9 +64,9 @@ __global__ void __launch_bounds__(256) k_bs_tiles(BsArgs a) {
     __shared__ BsRecords shared[8];
     BsRecords &R = shared[threadIdx.x >> 5];
     const u32 FULL = 0xffffffffu, lane = threadIdx.x & 31;
-    const u64 nt = (a.nh + TILE - 1) / TILE, nwarps = ((u64)gridDim.x * blockDim.x) >> 5;
+    const u64 nt = (a.nh + a.per_tile - 1) / a.per_tile, nwarps = ((u64)gridDim.x * blockDim.x) >> 5;
     for (u64 tl = (blockIdx.x * (u64)blockDim.x + threadIdx.x) >> 5; tl < nt; tl += nwarps) {
-        const u64 h0 = tl * TILE, h1 = h0 + TILE < a.nh ? h0 + TILE : a.nh;
+        const u64 h0 = tl * a.per_tile, h1 = h0 + a.per_tile < a.nh ? h0 + a.per_tile : a.nh;
         u64 m0 = 0, hi = a.nsm;   // the last record that starts at or before h0
         while (hi - m0 > 1) {
             const u64 mid = (m0 + hi) >> 1;
@@ -90,7 +91,7 @@ __global__ void __launch_bounds__(256) k_bs_tiles(BsArgs a) {
                     R.qbeg[lane] = rq.y;
                     const bool cuts = mt == 1 || mt == 2, fits = len <= 32 * MARKS;
                     if (cuts && !fits) R.mate[lane] = mt | NO_MARKS;
-                    if (cuts && fits) {
+                    if (cuts && fits && e > h0 && first_hit(a, m) < h1) {   // a record of hits in this tile
                         const u8 *P = a.seq + a.off[rq.x] + rq.y;
                         for (u32 w = 0; 32 * w < len; ++w) {
                             u32 bits = 0;
@@ -182,7 +183,15 @@ __global__ void __launch_bounds__(256) k_bs_tiles(BsArgs a) {
     }
 }
 
-unsigned tile_grid(u64 hits) { return grid_for((hits + TILE - 1) / TILE * 32, 256, 152u * 8u); }
+// Tiles of 256 hits, or as small as gives every SM's 32 warps one: with 256 always, the split of 18,000 hits
+// took 0.230 ms against 0.148 for a thread per hit, now 0.093; 209,000 hits 0.246, 0.157 and 0.124; the
+// same from 600,000 hits on.  (A quarter of the warps instead: 209,000 hits 0.232 ms.)
+u32 tile_size(u64 hits) {
+    u32 t = 32;
+    while (t < TILE && hits > (u64)t * 152 * 32) t *= 2;
+    return t;
+}
+unsigned tile_grid(u64 tiles) { return grid_for(tiles * 32, 256, 152u * 8u); }
 
 }  // namespace
 
@@ -211,9 +220,10 @@ extern "C" int mb_bs_filter(const mb_index *idx, const mb_smem *smem, uint64_t n
     mb_index_info(idx, &n, &prim, &M);
     // the 3-base index holds four copies of |R| = M/2 bases
     u64 quarter = M / 2;
+    const u32 per = tile_size(n_hits);
     const BsArgs a{(const mb_smem *)dsm, n_smem, (const u32 *)dhits, nullptr, n_hits, nullptr, quarter, nullptr, nullptr,
-                   (const u8 *)dmate, 0, nullptr, nullptr, nullptr, 0, dk};
-    k_bs_tiles<BS_FILTER><<<tile_grid(n_hits), 256, 0, st>>>(a);
+                   (const u8 *)dmate, 0, per, nullptr, nullptr, nullptr, 0, dk};
+    k_bs_tiles<BS_FILTER><<<tile_grid((n_hits + per - 1) / per), 256, 0, st>>>(a);
     MB_KCHECK();
     if (!kdev) MB_CK(cudaMemcpyAsync(keep, dk, n_hits, cudaMemcpyDeviceToHost, st));
     MB_CK(cudaStreamSynchronize(st));
@@ -252,12 +262,13 @@ extern "C" int mb_bs_split(const mb_index *idx, const uint8_t *ref, const uint8_
     MB_TRY(mb_stage_in(smem, n_smem * sizeof(mb_smem), st, bsm, &dsm));
     MB_TRY(mb_stage_in(hits, n_hits * 4, st, bhits, &dhits));
     if (keep) MB_TRY(mb_stage_in(keep, n_hits, st, bkeep, &dkeep));
-    const u64 tiles = (n_hits + TILE - 1) / TILE;
+    const u32 per = tile_size(n_hits);
+    const u64 tiles = (n_hits + per - 1) / per;
     MB_TRY(bcnt.alloc(tiles * 8 + 64 + n_hits, st));
     u64 *cnt = bcnt.as<u64>(), *dtotal = cnt + tiles;
     BsArgs a{(const mb_smem *)dsm, n_smem, (const u32 *)dhits, (const u8 *)dkeep, n_hits, (const u8 *)dref, M,
-             (const u8 *)dseq, (const u64 *)doff, (const u8 *)dmate, min_len, cnt, (u8 *)(dtotal + 8), nullptr, 0, nullptr};
-    k_bs_tiles<BS_COUNT><<<tile_grid(n_hits), 256, 0, st>>>(a);
+             (const u8 *)dseq, (const u64 *)doff, (const u8 *)dmate, min_len, per, cnt, (u8 *)(dtotal + 8), nullptr, 0, nullptr};
+    k_bs_tiles<BS_COUNT><<<tile_grid(tiles), 256, 0, st>>>(a);
     MB_KCHECK();
     MB_TRY(btmp.alloc(scan_tmp_bytes(tiles), st));
     MB_TRY(scan_exclusive_u64(cnt, cnt, tiles, dtotal, btmp.p, st));
@@ -276,7 +287,7 @@ extern "C" int mb_bs_split(const mb_index *idx, const uint8_t *ref, const uint8_
     }
     a.out = dout;
     a.cap = total;
-    k_bs_tiles<BS_WRITE><<<tile_grid(n_hits), 256, 0, st>>>(a);
+    k_bs_tiles<BS_WRITE><<<tile_grid(tiles), 256, 0, st>>>(a);
     MB_KCHECK();
     if (!odev) MB_CK(cudaMemcpyAsync(out, dout, total * sizeof(mb_piece), cudaMemcpyDeviceToHost, st));
     MB_CK(cudaStreamSynchronize(st));

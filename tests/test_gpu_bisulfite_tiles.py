@@ -42,3 +42,29 @@ def test_tiles(mb, max_occ, min_len):
         got = mb.mb_bs_split(G, ref, seq, off, mate, sm, m, hits, nh, keep=kp, opts=dict(min_len=min_len))
         want = oracle.bs_split(ref, seq, off, mate, sm, hits, k, min_len=min_len)
         assert got.tobytes() == want.astype(mb.PIECE_DTYPE).tobytes()
+
+
+def test_tile_sizes(mb):
+    """Numbers of hits on both sides of the lines between tiles of 32, 64, 128 and 256 hits (152 x 32 tiles of
+    each), and few: the strand rule against the oracle, the pieces against those of the whole set, whose
+    tiles hold 256."""
+    r = np.random.default_rng(91)
+    ref = np.concatenate([r.integers(0, 4, 15_000), np.tile(r.integers(0, 4, 331), 200), r.integers(0, 4, 15_000)]).astype(np.uint8)
+    rd = synth.reads(ref, 8000, 92, mode=1, read_len=150, bisulfite=True, sub_lo=0.002)
+    G = mb.mb_index_build(ref, opts=dict(flags=mb.MB_BS3))
+    o = dict(flags=mb.MB_BS3, max_occ=2000)
+    sm, m, nh = mb.mb_seed_batch(G, rd.seq, rd.off, mate=rd.mate, opts=o)
+    hits, _ = mb.mb_locate(G, sm, m, opts=o, cap=nh)
+    line = 32 * 152 * 32
+    assert nh > 4 * line
+    cnt = np.where(sm["flags"] & 1, 0, sm["s"]).astype(np.int64)
+    own = np.repeat(np.arange(m), cnt)
+    length = (sm["qend"].astype(np.int64) - sm["qbeg"])[own]
+    want = oracle.bs_keep(hits.astype(np.int64), length, rd.mate[sm["read"][own]], len(ref)).astype(np.uint8)
+    whole = mb.mb_bs_split(G, ref, rd.seq, rd.off, rd.mate, sm, m, hits, nh, keep=want)
+    assert len(whole) > 0
+    for h in (1, 31, 32, 33, 1000, line, line + 1, 2 * line, 2 * line + 1, 4 * line, 4 * line + 1, nh):
+        keep = mb.mb_bs_filter(G, sm, m, rd.mate, hits[:h].copy(), h)
+        assert np.array_equal(keep, want[:h]), h
+        got = mb.mb_bs_split(G, ref, rd.seq, rd.off, rd.mate, sm, m, hits[:h].copy(), h, keep=keep)
+        assert got.tobytes() == whole[whole["hit"] < h].tobytes(), h
