@@ -219,11 +219,16 @@ __global__ void __launch_bounds__(256) k_qmer_words(const u8 *__restrict__ reads
     }
 }
 
-// The longest read and window, and the first pair whose offsets decrease (npairs: none).
+// mx (zero before): the longest read and window, npairs less the first pair whose offsets decrease (0: none),
+// and the ends of both arrays, so that one copy takes all to the host.
 __global__ void k_pair_sizes(const u64 *__restrict__ roff, const u64 *__restrict__ woff, u32 npairs,
-                             unsigned long long *__restrict__ mx, u32 *__restrict__ bad) {
+                             unsigned long long *__restrict__ mx) {
     u64 a = 0, b = 0;
     u32 first = npairs;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        mx[3] = roff[npairs];
+        mx[4] = woff[npairs];
+    }
     for (u32 p = blockIdx.x * blockDim.x + threadIdx.x; p < npairs; p += gridDim.x * blockDim.x) {
         const u64 r0 = roff[p], r1 = roff[p + 1], w0 = woff[p], w1 = woff[p + 1];
         if (r1 < r0 || w1 < w0) {
@@ -242,7 +247,7 @@ __global__ void k_pair_sizes(const u64 *__restrict__ roff, const u64 *__restrict
     if ((threadIdx.x & 31) == 0) {
         if (a) atomicMax(mx, (unsigned long long)a);
         if (b) atomicMax(mx + 1, (unsigned long long)b);
-        if (first < npairs) atomicMin(bad, first);
+        if (first < npairs) atomicMax(mx + 2, (unsigned long long)(npairs - first));
     }
 }
 
@@ -310,21 +315,19 @@ extern "C" int mb_rescue_prefilter(const uint8_t *reads, const uint64_t *read_of
         rend = read_off[n_pairs];
         wend = win_off[n_pairs];
     } else {
-        MB_TRY(bsz.alloc(24, st));
+        MB_TRY(bsz.alloc(40, st));
         unsigned long long *mx = bsz.as<unsigned long long>();
-        MB_CK(cudaMemsetAsync(mx, 0, 16, st));
-        MB_CK(cudaMemsetAsync(mx + 2, 0xFF, 4, st));
-        k_pair_sizes<<<grid_for(n_pairs, 256, 152 * 4), 256, 0, st>>>((const u64 *)dro, (const u64 *)dwo, n_pairs, mx,
-                                                                     (u32 *)(mx + 2));
+        MB_CK(cudaMemsetAsync(mx, 0, 40, st));
+        k_pair_sizes<<<grid_for(n_pairs, 256, 152 * 4), 256, 0, st>>>((const u64 *)dro, (const u64 *)dwo, n_pairs, mx);
         MB_KCHECK();
-        u64 v[3] = {0, 0, 0};
-        MB_CK(cudaMemcpyAsync(v, mx, 24, cudaMemcpyDeviceToHost, st));
-        MB_CK(cudaMemcpyAsync(&rend, (const u64 *)dro + n_pairs, 8, cudaMemcpyDeviceToHost, st));
-        MB_CK(cudaMemcpyAsync(&wend, (const u64 *)dwo + n_pairs, 8, cudaMemcpyDeviceToHost, st));
+        u64 v[5];
+        MB_CK(cudaMemcpyAsync(v, mx, sizeof v, cudaMemcpyDeviceToHost, st));
         MB_CK(cudaStreamSynchronize(st));
         mmax = v[0];
         wmax = v[1];
-        if ((u32)v[2] < n_pairs) bad = (u32)v[2];
+        bad = n_pairs - (u32)v[2];
+        rend = v[3];
+        wend = v[4];
     }
     if (bad < n_pairs) {
         mb_set_error("mb_rescue_prefilter: offsets decrease at pair %u", bad);
