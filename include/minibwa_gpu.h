@@ -58,7 +58,10 @@ enum {
                               host checks every device buffer against its allocation (MB_ERR_ARG) */
 #define MB_NO_KMER  0x8u   /* seeding: do not use the k-mer ds-interval table; index: without the deeper
                               table that kmer_k describes (nor when loaded from its file) */
-#define MB_COUNT    0x10u  /* seeding/locate: also count the work done (mb_work_counters) */
+#define MB_COUNT    0x10u  /* seeding/locate: also count the work done (mb_work_counters): that of the
+                              one-loop SMEM kernel with the table of kmer_k and text comparisons of 16
+                              bases, and of shared locate walks.  The default kernel, with the deeper
+                              table where the index has one and comparisons of 64, does less */
 #define MB_NO_AUX   0x20u  /* index: build without the packed text and the rate-4 SA / ISA samples
                               (2.25 bytes per text position) that let seeding extend unique matches
                               by comparing text */
@@ -73,8 +76,9 @@ enum {
 #define MB_LOCATE_AUX 0x200u /* locate: walks stop at the rate-4 SA samples the index keeps for
                               extending unique matches (a row that is a multiple of 4) instead of
                               the rate-r samples of Section 2.4: about r/4 times fewer LF steps, same
-                              positions; no joins.  The default but under MB_COUNT and MB_CHECKED.
-                              Ignored for an index built with MB_NO_AUX */
+                              positions; no joins.  The default but under MB_COUNT and MB_CHECKED (with
+                              sa_rate 1 or 2 the index's own samples, which are denser, unless MB_COUNT
+                              is given too).  Ignored for an index built with MB_NO_AUX */
 #define MB_SMEM_ONE_LOOP 0x80u /* tuning: the SMEM kernel in its one-loop form (one read per lane, every
                               iteration runs every stage's code) instead of the slot form (a warp
                               holds up to 64 reads and runs one kind of step for up to 32 of them at
@@ -231,15 +235,17 @@ int mb_seed_batch_noalloc(const mb_index *idx, const uint8_t *seq, const uint64_
  * mb_locate — text positions of every row of every SMEM without MB_SMEM_OVER_MAX_OCC
  * (Section 2.4, Algorithm 2): row x is LF-walked to a sampled row; its position is
  * (steps + S(sampled row)) mod n.  Every row is a sample while the index keeps its full suffix array
- * (until mb_index_drop_sa); else every fourth, or every r-th on an index built with MB_NO_AUX.
+ * (until mb_index_drop_sa); else every fourth, or every r-th for sa_rate 1 or 2.  On an index built with
+ * MB_NO_AUX it is every r-th, with the full array too unless sa_rate is 1, 2 or 4.
  *   smem     host or device, n_smem records from mb_seed_batch (hit_off must be as written).
  *   hits     host or device, room for `cap` u32 positions; hit t of record m is written at
  *            hits[m.hit_off + t], rows k..k+s-1 in order.
  *   n_hits   receives the total.  If it exceeds cap: MB_ERR_CAPACITY, nothing written.
  * With MB_BS3 in opts, hits are still all written; mb_bs_filter applies the strand rule.
- * Without the full array, and for more than 2^25 hits, an index built with MB_NO_AUX, MB_COUNT or
- * MB_CHECKED, a row that several records share (the same or nested intervals) is walked once and its
- * position copied to each of their hits; with MB_COUNT the work counters count those walks.
+ * With MB_COUNT or MB_CHECKED, on an index built with MB_NO_AUX (but for sa_rate 1, 2 or 4), and for more
+ * than 2^25 hits without the full array, a row that several records share (the same or nested intervals) is
+ * walked once and its position copied to each of their hits; with MB_COUNT the work counters count those
+ * walks.
  * Device workspace, allocated per call: 8 bytes per 256 to 8,192 hits; with shared walks about 40
  * bytes per record and 8 per hit.
  */

@@ -3,7 +3,7 @@
 // Section 2.4 sampled suffix array, Section 2.5 k-mer ds-interval table).
 //
 //   T = R . revcomp(R) . $            (bisulfite: R -> CT(R) . GA(R), Section 2.9)
-//   S = suffix array of T             prefix doubling: sort by the first 21 symbols, then
+//   S = suffix array of T             prefix doubling: sort by the first 20 symbols, then
 //                                     repeatedly re-sort the suffixes whose 2h-prefix is still
 //                                     shared by (rank of the h-prefix, rank of the h-prefix at +h)
 //   B[i] = T[S(i) - 1], T[-1] = $     written straight into 32-byte occurrence blocks
@@ -513,8 +513,9 @@ static int make_sa_ref(mb_index *x) {
 // Seeding's own k-mer table, as deep as 4^k <= n / 2 (13 at 100 Mbp, 14 at 1 Gbp), where the index's
 // table (k = 10 by default, Section 2.5, sized for a CPU cache) is shallower: every further base is an
 // extension less per lookup, of a wide interval and so of two blocks.  Same SMEMs with any k.  It takes
-// 1.5 to 6 bytes per text position; without room for it seeding uses the index's own.  2M reads on
-// 100 Mbp (k = 10 -> 13), seeded and located: 3.36 -> 3.10 ms.
+// 1.5 to 6 bytes per text position (MB_NO_KMER at the build declines it) and is made after every array that
+// the index must have; without room for it seeding uses the index's own.  2M reads on 100 Mbp (k = 10 ->
+// 13), seeded and located: 3.36 -> 3.10 ms; a load of 20 Mbp takes 2.8 ms more for it.
 static int build_kmer2(mb_index *x, cudaStream_t st) {
     if (x->flags & MB_NO_KMER) return MB_OK;   // declined at the build (kept in the file's flags)
     u32 k = x->kmer_k;

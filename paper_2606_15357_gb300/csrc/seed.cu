@@ -486,8 +486,10 @@ struct WarpRange {
 //
 // In a batch of at most LONG_BASES bases, reads of LONG_LEN bases or more are cut before their first step:
 // such a batch takes as long as its longest chains, not as its work (200,000 reads of 100 bp - 10 kb, 430
-// Mbases: 8.4 -> 7.4 ms; a served mix with a few long reads 7.1 -> 2.8 ms).  A cut costs about 35 steps
-// per item, so larger batches, which fill the chip, keep their reads whole until `steps`.
+// Mbases: 8.6 -> 6.8 ms; a served mix with a few long reads 7.1 -> 2.8 ms).  A cut costs about 35 steps
+// per item, so larger batches, which fill the chip, keep their reads whole until `steps`.  Both sides of the
+// line, reads of 100 bp - 10 kb kept whole and cut (into items of 256 starts): 640 Mbases 9.9 and 9.1 ms on
+// 100 Mbp, 15.4 and 15.9 on 1 Gbp; 860 Mbases 9.5 and 9.7, 16.8 and 19.0; 1.7 Gbases 12.7 and 14.3.
 constexpr u64 LONG_BASES = 1ull << 29;
 constexpr int LONG_LEN = 1024;
 constexpr u32 STEPS_LONG = 0x3FFFFFu;   // in the step count: cut at once
@@ -721,11 +723,12 @@ __global__ void __launch_bounds__(BLOCK, BLOCK == 128 ? 6 : 1024 / BLOCK) k_smem
 // read per lane, all kinds of step in one loop) had 9.8 active lanes per instruction and cost a read
 // 2,100 warp instructions (1 Gbp, k = 14); this one has 16.5 (19-26 in its block steps) and 1,370.  20M
 // reads of 150 bases there: 54.5 -> 37.3 ms (331M hits; another genome, 605M hits: 59.2 -> 45), 36 -> 52 G
-// DRAM sectors/s with the sequential ones, the rate the random-read probe reaches; 2M reads on a 100
-// Mbp index 5.17 -> 2.6 ms.  More reads in flight help
+// DRAM sectors/s with the sequential ones, the rate the random-read probe reaches (40.4 ms on a GPU whose
+// probe gives 7% less); 2M reads on a 100 Mbp index 5.17 -> 2.5 ms, 776 warp instructions a read at
+// 18.4 lanes and 95 G DRAM sectors/s.  More reads in flight help
 // (32 slots per warp instead of 64: 20% slower; 24 warps per SM instead of 32: 6%), so the table takes
 // the shared memory it can get: 64 slots x 32 warps x 89 bytes.  A lone read (a small batch's tail)
-// advances one extension per 0.7 us.
+// advances one extension per 0.7 us (how much of that is its loads was not measured).
 constexpr int SLOTS = 64;           // reads a warp holds (two per lane: at most 2-way bank conflicts)
 constexpr int WIN = 64;             // bases of a read kept in its slot, 2 bits each
 enum { C_BLOCK = 0, C_TEXT = 1, C_LOOK = 2, C_SERV = 3, C_FREE = 4 };
